@@ -139,8 +139,8 @@ def _points(target, n, seed):
         r = torch.sqrt(1.0 - z * z)
         t = i * (math.pi * (3.0 - math.sqrt(5.0)))
         p = torch.stack([r * torch.cos(t), r * torch.sin(t), z], 1)
-        q, _ = torch.linalg.qr(torch.randn(3, 3, generator=g, device=DEV, dtype=torch.float64))
-        p = p @ q
+        q, _ = torch.linalg.qr(torch.randn(3, 3, generator=g, device=DEV, dtype=torch.float64).cpu())
+        p = p @ q.to(DEV)
         return p.float().contiguous(), p.float().contiguous()
     else:                                       # trihedral, plate and cylinder, by area
         a_tri, a_pl, a_cy = 1.08, 1.0, 2 * math.pi * 0.3
