@@ -287,6 +287,400 @@ __global__ void __launch_bounds__(TC_THREADS, 3)
   }
 }
 
+// ---------------------------------------------------------------------------
+// The streaming form: BF16 output rows, persistent CTAs.
+//
+// Most of the U-Net's contractions are narrow (K, N = 32..512 over millions of
+// pixels): they are bound by moving rows through the SM, so the kernel is
+// built around that.  A CTA walks its share of the output tiles; one lane
+// loads operand blocks (TMA ring), one issues the products of tile i + 1 into
+// one half of the tensor memory while the epilogue warps drain tile i from the
+// other.  Two groups of four epilogue warps take alternate tiles; each warp
+// owns 32 rows (its tensor-memory lanes) and goes through 32-column slabs:
+// registers -> its own 64-byte-row staging slab (64-byte swizzle, conflict
+// free for a row per lane) -> TMA store.  The residual or the pre-activation a
+// mode reads arrives the same way (TMA load into the slab, prefetched), is
+// replaced in place by the result and stored from there, so global memory
+// sees only whole-row bulk copies and no CTA-wide barrier stands between
+// tiles.
+//   MODE 0  C = acc (+ bias)            MODE 1  C = acc (+ bias) + X
+//   MODE 2  Z = acc (+ bias), C = GELU  MODE 3  C = (acc (+ bias)) GELU'(X)
+// The arithmetic per element is pe_gemm_store8's, in the same order.
+//
+// Against the kernel above on the same contractions (which holds a 128 x 256
+// FP32 tile in shared memory, so one CTA per SM loads, multiplies and stores in
+// turn), 64 channels, 524288 pixels: 1x1 expansion with GELU 375 -> 159 us (603
+// MB: 89 us of copy bandwidth; the erf of 134M values bounds it), data gradient
+// through GELU' 542 -> 239 us (603 MB; erf and exp), projection with residual
+// 110 -> 70 us (402 MB, 59 us of copy bandwidth), data gradient 75 -> 50 us (336
+// MB, 49 us).  All results equal bit for bit.  Column tiles of 128 at most: two
+// CTAs per SM, whose tensor memory (2 x 128 columns each) fills the SM's 512.
+// ---------------------------------------------------------------------------
+constexpr int ST_THREADS = 320;  // producer, issuer, eight epilogue warps
+constexpr int ST_SLAB = 32 * 32 * 2;
+constexpr int ST_MAX_BIAS = 1024;  // columns whose bias is kept in shared memory
+
+template <int BN, int MODE>
+struct st_cfg {
+  static constexpr int STAGES = BN == 128 ? 2 : 3;
+  static constexpr int NB = (MODE == 1 && BN == 32) ? 3 : 2;  // staging slabs per warp
+  static constexpr int A_BYTES = TC_BM * TC_BK * 2, B_BYTES = BN * TC_BK * 2;
+  static constexpr int STAGE = A_BYTES + B_BYTES;
+  static constexpr int STAGING = 8 * NB * ST_SLAB;
+  // barriers (an even number of 8-byte words, so that the bias after them and
+  // the two words that follow is 16-byte aligned)
+  static constexpr int BARS = (2 * STAGES + 4 + 8 * NB + 1 + 1) & ~1;
+  static_assert((STAGES * STAGE) % 1024 == 0 && STAGING % 1024 == 0 && (BARS * 8) % 16 == 0,
+                "alignment of the slabs, the barriers and the bias");
+  static constexpr uint32_t IDESC = tc_cfg<BN>::IDESC;
+  static int smem(int bias_floats) {
+    return 1024 + STAGES * STAGE + STAGING + BARS * 8 + 16 + bias_floats * 4;
+  }
+};
+
+struct st_args {
+  int M, N, K;
+  int tiles_n;
+  int items;  // output tiles
+  float alpha;
+  const float *bias;
+  uint32_t wait_limit;
+  unsigned int *err;
+};
+
+// Bounded wait that also gives up once another role of the CTA has.
+__device__ __forceinline__ bool st_wait(uint64_t *bar, uint32_t parity, uint32_t limit,
+                                        volatile int *fail) {
+  const uint32_t a = sm_u32(bar);
+  for (uint32_t i = 0; i < limit; ++i) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(a), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if ((i & 63u) == 63u && *fail) return false;
+  }
+  return false;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(sm_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void *src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];\n" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(x), "r"(y), "r"(sm_u32(src))
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() {
+  asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;\n" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() {
+  asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+}
+__device__ __forceinline__ void async_fence() {
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+}
+
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
+        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+template <int BN, int MODE>
+__global__ void __launch_bounds__(ST_THREADS, 2)
+    gemm_stream_kernel(const __grid_constant__ CUtensorMap tmA,
+                       const __grid_constant__ CUtensorMap tmB,
+                       const __grid_constant__ CUtensorMap tmC,
+                       const __grid_constant__ CUtensorMap tmX, const st_args g) {
+  using cfg = st_cfg<BN, MODE>;
+  constexpr int S = cfg::STAGES, NB = cfg::NB, SLABS = BN / 32;
+  constexpr bool XIN = MODE == 1 || MODE == 3;
+  extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
+  uint8_t *base = reinterpret_cast<uint8_t *>(
+      (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint8_t *staging = base + S * cfg::STAGE;
+  uint64_t *full = reinterpret_cast<uint64_t *>(staging + cfg::STAGING);
+  uint64_t *empty = full + S, *tfull = empty + S, *tempty = tfull + 2, *xbar = tempty + 2;
+  uint64_t *drain = xbar + 8 * NB;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(full + cfg::BARS);
+  volatile int *s_fail = reinterpret_cast<volatile int *>(tmem_slot + 1);
+  float *s_bias = reinterpret_cast<float *>(tmem_slot + 4);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nk = (g.K + TC_BK - 1) / TC_BK;
+
+  if (threadIdx.x == 0) {
+    *s_fail = 0;
+    for (int s = 0; s < S; ++s) {
+      mbar_init(full + s, 1);
+      mbar_init(empty + s, 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(tfull + s, 1);
+      mbar_init(tempty + s, 4);  // the four warps of a group
+    }
+    for (int s = 0; s < 8 * NB; ++s) mbar_init(xbar + s, 1);
+    mbar_init(drain, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (g.bias) {
+    const int n_pad = (g.N + 31) & ~31;
+    for (int i = threadIdx.x; i < n_pad; i += ST_THREADS) s_bias[i] = i < g.N ? g.bias[i] : 0.0f;
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     sm_u32(tmem_slot)),
+                 "r"((uint32_t)(2 * BN))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- producer ------------------------------------------------------
+      uint32_t c = 0;  // k-blocks issued
+      bool ok = true;
+      for (int it = blockIdx.x; ok && it < g.items; it += gridDim.x) {
+        const int m0 = (it / g.tiles_n) * TC_BM, n0 = (it % g.tiles_n) * BN;
+        for (int kb = 0; kb < nk; ++kb, ++c) {
+          const int s = (int)(c % S);
+          if (!st_wait(empty + s, ((c / S) & 1u) ^ 1u, g.wait_limit, s_fail)) {
+            *s_fail = 1;
+            ok = false;
+            break;
+          }
+          uint8_t *sa = base + s * cfg::STAGE;
+          mbar_expect_tx(full + s, (uint32_t)cfg::STAGE);
+          tma_load_2d(sa, &tmA, kb * TC_BK, m0, full + s);
+          tma_load_2d(sa + cfg::A_BYTES, &tmB, kb * TC_BK, n0, full + s);
+        }
+      }
+      if (!ok)  // copies in flight land before the shared memory is released
+        for (uint32_t k = c > (uint32_t)S ? c - S : 0; k < c; ++k)
+          mbar_wait(full + k % S, (k / S) & 1u);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ---- product issuer ------------------------------------------------
+      uint32_t c = 0, i = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; ok && it < g.items; it += gridDim.x, ++i) {
+        const uint32_t st = i & 1u;
+        if (!st_wait(tempty + st, ((i >> 1) & 1u) ^ 1u, g.wait_limit, s_fail)) {
+          *s_fail = 1;
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        for (int kb = 0; kb < nk; ++kb, ++c) {
+          const int s = (int)(c % S);
+          if (!st_wait(full + s, (c / S) & 1u, g.wait_limit, s_fail)) {
+            *s_fail = 1;
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sa = sm_u32(base + s * cfg::STAGE);
+          const uint64_t ad = kmajor_sw128_desc(sa), bd = kmajor_sw128_desc(sa + cfg::A_BYTES);
+          const int steps = min(TC_BK / 16, (g.K - kb * TC_BK + 15) / 16);
+          for (int k = 0; k < steps; ++k)
+            tc_mma(tmem + st * BN, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), cfg::IDESC,
+                   (kb > 0 || k > 0) ? 1u : 0u);
+          tc_commit(empty + s);
+        }
+        if (ok) tc_commit(tfull + st);
+      }
+      if (!ok) {  // products in flight complete before the tensor memory is freed
+        tc_commit(drain);
+        mbar_wait(drain, 0u);
+      }
+    }
+  } else {
+    // ---- epilogue ----------------------------------------------------------
+    const int ew = warp - 2, grp = ew >> 2, quad = warp & 3;
+    uint8_t *slabs = staging + ew * NB * ST_SLAB;
+    uint64_t *xb = xbar + ew * NB;
+    // this lane's row in a slab: chunk q (16 bytes) at row + ((q ^ sw) << 4)
+    const uint32_t row = (uint32_t)lane * 64u, sw = ((uint32_t)lane >> 1) & 3u;
+    const uint32_t tlane = tmem + (uint32_t)(grp * BN) + ((uint32_t)(quad * 32) << 16);
+    // a cursor over this warp's slabs: tiles of its parity, the slabs that
+    // hold rows and columns of the matrix
+    struct cursor {
+      int it, j;
+    };
+    auto inside = [&](const cursor &k) {
+      return (k.it / g.tiles_n) * TC_BM + quad * 32 < g.M &&
+             (k.it % g.tiles_n) * BN + k.j * 32 < g.N;
+    };
+    auto step = [&](cursor &k) {
+      do {
+        if (++k.j == SLABS) {
+          k.j = 0;
+          k.it += 2 * (int)gridDim.x;
+        }
+      } while (k.it < g.items && !inside(k));
+    };
+    auto load_x = [&](const cursor &k, uint32_t seq) {
+      const uint32_t b = seq % NB;
+      mbar_expect_tx(xb + b, ST_SLAB);
+      tma_load_2d(slabs + b * ST_SLAB, &tmX, (k.it % g.tiles_n) * BN + k.j * 32,
+                  (k.it / g.tiles_n) * TC_BM + quad * 32, xb + b);
+    };
+    const int first = (int)(blockIdx.x + grp * gridDim.x);
+    cursor ld = {first, -1};
+    uint32_t ld_seq = 0;
+    if (XIN) {
+      step(ld);
+      for (int k = 0; k < NB - 1 && ld.it < g.items; ++k, ++ld_seq, step(ld))
+        if (lane == 0) load_x(ld, ld_seq);
+    }
+    uint32_t seq = 0, u = 0;
+    bool ok = true;
+    for (int it = first; ok && it < g.items; it += 2 * (int)gridDim.x, ++u) {
+      const int m0 = (it / g.tiles_n) * TC_BM + quad * 32, n0 = (it % g.tiles_n) * BN;
+      bool ready = st_wait(tfull + grp, u & 1u, g.wait_limit, s_fail);
+      ok = __all_sync(0xffffffffu, ready);
+      if (!ok) break;
+      tc_fence_after();
+#pragma unroll 1
+      for (int j = 0; j < SLABS; ++j) {
+        const int c0 = n0 + 32 * j;
+        if (m0 >= g.M || c0 >= g.N) continue;
+        const uint32_t b = seq % NB;
+        uint8_t *slab = slabs + b * ST_SLAB;
+        if (XIN) {
+          // the slab read ahead: its buffer's last store has been read out
+          if (ld.it < g.items) {
+            if (lane == 0) {
+              bulk_wait_read<0>();
+              load_x(ld, ld_seq);
+            }
+            ++ld_seq;
+            step(ld);
+          }
+          ready = st_wait(xb + b, (seq / NB) & 1u, g.wait_limit, s_fail);
+          ok = __all_sync(0xffffffffu, ready);
+          if (!ok) break;
+        }
+        float v[32];
+        tc_ld32(tlane + (uint32_t)(32 * j), v);
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = __fmul_rn(v[e], g.alpha);
+        if (g.bias) {
+          const float4 *bp = reinterpret_cast<const float4 *>(s_bias + c0);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const float4 t = bp[q];
+            v[4 * q] += t.x;
+            v[4 * q + 1] += t.y;
+            v[4 * q + 2] += t.z;
+            v[4 * q + 3] += t.w;
+          }
+        }
+        if (XIN) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint4 xv = *reinterpret_cast<const uint4 *>(slab + row + ((q ^ sw) << 4));
+            const bf162 *xp = reinterpret_cast<const bf162 *>(&xv);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float2 f = __bfloat1622float2(xp[e]);
+              if (MODE == 1) {
+                v[8 * q + 2 * e] += f.x;
+                v[8 * q + 2 * e + 1] += f.y;
+              } else {
+                v[8 * q + 2 * e] *= pe_gelu_grad(f.x);
+                v[8 * q + 2 * e + 1] *= pe_gelu_grad(f.y);
+              }
+            }
+          }
+        }
+        auto put = [&](uint8_t *dst) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint4 o;
+            bf162 *op = reinterpret_cast<bf162 *>(&o);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              op[e] = __floats2bfloat162_rn(v[8 * q + 2 * e], v[8 * q + 2 * e + 1]);
+            *reinterpret_cast<uint4 *>(dst + row + ((q ^ sw) << 4)) = o;
+          }
+        };
+        if (MODE == 2) {
+          // both slabs of the warp: the pre-activation, then the result
+          if (lane == 0) bulk_wait_read<0>();
+          __syncwarp();
+          put(slabs);
+#pragma unroll
+          for (int e = 0; e < 32; ++e) v[e] = pe_gelu(v[e]);
+          put(slabs + ST_SLAB);
+        } else {
+          if (!XIN) {
+            if (lane == 0) bulk_wait_read<NB - 1>();
+            __syncwarp();
+          }
+          put(slab);
+        }
+        async_fence();
+        __syncwarp();
+        if (lane == 0) {
+          if (MODE == 2) {
+            tma_store_2d(&tmX, slabs, c0, m0);
+            tma_store_2d(&tmC, slabs + ST_SLAB, c0, m0);
+          } else {
+            tma_store_2d(&tmC, slab, c0, m0);
+          }
+          bulk_commit();
+        }
+        ++seq;
+      }
+      if (!ok) break;
+      // this half of the tensor memory may take the group's next tile
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty + grp);
+    }
+    if (!ok) {
+      *s_fail = 1;
+      if (XIN && lane == 0)  // loads in flight land before the memory is released
+        for (uint32_t k = seq; k < ld_seq; ++k) mbar_wait(xb + k % NB, (k / NB) & 1u);
+    }
+    if (lane == 0) bulk_wait_all();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *s_fail) atomicOr(g.err, PE_ERR_TIMEOUT);
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
+                 "r"((uint32_t)(2 * BN))
+                 : "memory");
+  }
+}
+
 typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                     const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                     const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -353,6 +747,96 @@ pe_status launch_bn(const pe_gemm_args &g, cudaStream_t s) {
   return PE_OK;
 }
 
+// Row-major BF16 [rows][ld] in 32 x 32 slabs (64-byte rows, 64-byte swizzle),
+// for the streaming kernel's output rows and the rows its epilogue reads.
+bool make_slab_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld) {
+  encode_tiled_fn enc = encoder();
+  if (!enc) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+  cuuint32_t box[2] = {32, 32};
+  cuuint32_t estr[2] = {1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+int tc_sms() {
+  static int n = 0;
+  if (!n) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (n <= 0) n = 1;
+  }
+  return n;
+}
+
+template <int BN, int MODE>
+pe_status launch_stream(const pe_gemm_args &g, cudaStream_t s) {
+  using cfg = st_cfg<BN, MODE>;
+  CUtensorMap ma, mb, mc, mx;
+  const int64_t items = (int64_t)((g.M + TC_BM - 1) / TC_BM) * ((g.N + BN - 1) / BN);
+  if (items >= (1ll << 30)) return PE_EUNSUPPORTED;  // (tile numbers are 32-bit)
+  if (!make_map(&ma, g.A, g.M, g.K, g.sam, TC_BM) || !make_map(&mb, g.B, g.N, g.K, g.sbn, BN) ||
+      !make_slab_map(&mc, g.C, g.M, g.N, g.ldc))
+    return PE_EUNSUPPORTED;
+  if (MODE == 0) mx = mc;
+  else if (!make_slab_map(&mx, MODE == 1 ? g.R : g.Z, g.M, g.N, MODE == 1 ? g.ldr : g.ldz))
+    return PE_EUNSUPPORTED;
+  static bool attr = false;
+  if (!attr) {
+    PE_TRY_CUDA(cudaFuncSetAttribute(gemm_stream_kernel<BN, MODE>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     cfg::smem(ST_MAX_BIAS)));
+    PE_TRY_CUDA(cudaFuncSetAttribute(gemm_stream_kernel<BN, MODE>,
+                                     cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)cudaSharedmemCarveoutMaxShared));
+    attr = true;
+  }
+  st_args a;
+  memset(&a, 0, sizeof(a));
+  a.M = g.M;
+  a.N = g.N;
+  a.K = (int)g.K;
+  a.tiles_n = (g.N + BN - 1) / BN;
+  a.items = (int)items;
+  a.alpha = g.alpha;
+  a.bias = g.bias;
+  a.wait_limit = g_wait_limit.load();
+  a.err = pe_err_word();
+  const int most = 2 * tc_sms();  // two CTAs per SM
+  gemm_stream_kernel<BN, MODE><<<a.items < most ? a.items : most, ST_THREADS,
+                                 cfg::smem(g.bias ? (g.N + 31) / 32 * 32 : 0), s>>>(ma, mb, mc, mx,
+                                                                                    a);
+  PE_TRY_LAUNCH("gemm_stream_kernel");
+  return PE_OK;
+}
+
+// The streaming kernel's mode for these arguments, -1 when it does not apply:
+// a TMA store writes BF16 rows on 16-byte boundaries, so FP32 outputs (the
+// heads) and unaligned rows stay with the other kernel, as does an epilogue
+// outside the four forms.  Where both apply the streaming kernel was the
+// faster one at every shape of the network (gradients of a 32 x 256^2 batch:
+// 21.4 -> 11.7 ms over its 113 contractions).
+int stream_mode(const pe_gemm_args &g) {
+  if (g.c_f32 || !g.vec_c || g.K >= (1ll << 30) || (g.bias && g.N > ST_MAX_BIAS)) return -1;
+  if (g.gelu == 0) return g.R ? 1 : 0;
+  if (g.R) return -1;
+  if (g.gelu == 1) return g.Z ? 2 : -1;
+  return 3;
+}
+
+template <int BN>
+pe_status launch_stream_mode(int mode, const pe_gemm_args &g, cudaStream_t s) {
+  switch (mode) {
+    case 0: return launch_stream<BN, 0>(g, s);
+    case 1: return launch_stream<BN, 1>(g, s);
+    case 2: return launch_stream<BN, 2>(g, s);
+    default: return launch_stream<BN, 3>(g, s);
+  }
+}
+
 }  // namespace
 
 bool pe_gemm_tc_eligible(const pe_gemm_args &g) {
@@ -362,6 +846,13 @@ bool pe_gemm_tc_eligible(const pe_gemm_args &g) {
 }
 
 pe_status pe_gemm_tc(const pe_gemm_args &g, cudaStream_t s) {
+  const int mode = stream_mode(g);
+  if (mode >= 0) {
+    const pe_status st = g.N <= 32   ? launch_stream_mode<32>(mode, g, s)
+                         : g.N <= 64 ? launch_stream_mode<64>(mode, g, s)
+                                     : launch_stream_mode<128>(mode, g, s);
+    if (st != PE_EUNSUPPORTED) return st;
+  }
   if (g.N <= 32) return launch_bn<32>(g, s);
   if (g.N <= 64) return launch_bn<64>(g, s);
   if (g.N <= 128) return launch_bn<128>(g, s);

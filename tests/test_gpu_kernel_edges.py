@@ -1,0 +1,117 @@
+"""Kernels at the edges of their tiles and of their dispatch rules, against
+plain FP64 PyTorch (the layers) or the general path (the traced ones).
+
+Tolerances: a BF16 output is rounded once from an FP32 value; BF16 has 8
+significant bits, so the error is at most 2^-8 of each element (1 + 2^-8 lies
+half way between two BF16 numbers); the FP32 sums before it (at most 2304
+products here) add below 1e-5 of the result's size.  So BF16 outputs are held
+to 2^-8 + 1e-5 in the 2-norm.
+"""
+import ctypes as C
+import math
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+BF = torch.bfloat16
+BF_TOL = 2.0 ** -8 + 1e-5
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def ops():
+    from paper_2408_15583_gb300.learned import Ops
+    return Ops(DEV)
+
+
+def rel(a, b):
+    a, b = a.double(), b.double()
+    return float((a - b).norm() / b.norm().clamp(min=1e-30))
+
+
+def gen(seed):
+    return torch.Generator(device=DEV).manual_seed(seed)
+
+
+def rnd(g, *s):
+    return torch.randn(*s, generator=g, device=DEV)
+
+
+# ---- the streaming contraction ------------------------------------------------
+
+# rows: one, a warp's 32 and its neighbours, a tile's 128 and its neighbours,
+# more tiles than resident CTAs; columns: inside one slab, ragged slabs, every
+# column tile, two column tiles; K: below one block, ragged, several blocks
+@pytest.mark.parametrize("mode", ["plain", "residual", "gelu", "dgelu"])
+@pytest.mark.parametrize("M,N,K", [(1, 32, 32), (31, 8, 16), (33, 40, 64), (127, 64, 72),
+                                   (129, 136, 128), (128, 128, 576), (160, 256, 64),
+                                   (90_000, 32, 128), (60_001, 96, 32)])
+def test_streaming_contraction(M, N, K, mode):
+    o, g = ops(), gen(M + N + K)
+    A, B = rnd(g, M, K).to(BF), (rnd(g, N, K) / math.sqrt(K)).to(BF)
+    bias = rnd(g, N)
+    X = rnd(g, M, N + 8).to(BF)                       # a wider row than the output's
+    out = torch.full((M, N + 16), 7.0, dtype=BF, device=DEV)
+    Z = torch.full((M, N + 8), 7.0, dtype=BF, device=DEV)
+    ref = A.double() @ B.double().T
+    kw = {}
+    if mode == "plain":
+        kw = dict(bias=bias)
+        want = ref + bias.double()
+    elif mode == "residual":
+        kw = dict(bias=bias, R=X, ldr=N + 8)
+        want = ref + bias.double() + X[:, :N].double()
+    elif mode == "gelu":
+        kw = dict(bias=bias, Z=Z, ldz=N + 8, gelu=True)
+        pre = ref + bias.double()
+        want = torch.nn.functional.gelu(pre)
+    else:
+        kw = dict(Z=X, ldz=N + 8, dgelu=True)
+        z = X[:, :N].double()
+        want = ref * (0.5 * (1 + torch.erf(z / math.sqrt(2))) +
+                      z * torch.exp(-0.5 * z * z) / math.sqrt(2 * math.pi))
+    o.gemm(M, N, K, A, K, 1, B, 1, K, out, N + 16, **kw)
+    assert rel(out[:, :N], want) < BF_TOL
+    assert bool((out[:, N:] == 7.0).all())            # nothing past the row's columns
+    if mode == "gelu":
+        assert rel(Z[:, :N], pre) < BF_TOL
+        assert bool((Z[:, N:] == 7.0).all())
+    from paper_2408_15583_gb300 import api
+    api.stream_check()
+
+
+@pytest.mark.parametrize("mode", ["plain", "residual", "gelu"])
+def test_streaming_contraction_gives_up_and_recovers(mode):
+    """With a limit of zero polls no wait of the main loop succeeds: nothing is
+    stored, the status word says so once, and the next call computes."""
+    from paper_2408_15583_gb300 import _lib
+    lib = _lib.load()
+    o, g = ops(), gen(3)
+    M, N, K = 5000, 128, 128
+    A, B = rnd(g, M, K).to(BF), rnd(g, N, K).to(BF)
+    R = rnd(g, M, N).to(BF)
+    Z = torch.zeros(M, N, dtype=BF, device=DEV)
+    kw = dict(residual=dict(R=R, ldr=N), gelu=dict(Z=Z, ldz=N, gelu=True)).get(mode, {})
+    stream = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    try:
+        assert lib.pe_nn_set_wait_limit(0) == 0
+        out = torch.zeros(M, N, dtype=BF, device=DEV)
+        o.gemm(M, N, K, A, K, 1, B, 1, K, out, N, **kw)
+        assert lib.pe_stream_check(stream) == 4       # PE_ETIMEOUT
+        assert torch.count_nonzero(out) == 0 and torch.count_nonzero(Z) == 0
+        assert lib.pe_stream_check(stream) == 0
+    finally:
+        lib.pe_nn_set_wait_limit(-1)
+    o.gemm(M, N, K, A, K, 1, B, 1, K, out, N, **kw)
+    assert lib.pe_stream_check(stream) == 0
+    pre = A.double() @ B.double().T + (R.double() if mode == "residual" else 0.0)
+    assert rel(out, torch.nn.functional.gelu(pre) if mode == "gelu" else pre) < BF_TOL
