@@ -354,106 +354,253 @@ __global__ void col2im3_kernel(const bf16 *__restrict__ dcol, int B, int H, int 
 // depthwise 7x7 (zero padding 3), weights w[ky][kx][c] FP32; C even, rows of
 // channel pairs (bf16x2).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float2 ld2(const bf162 *p) { return __bfloat1622float2(*p); }
+// Both kernels work on channel pairs as packed FP32 pairs (one fma.f32x2 per
+// tap and pixel: the pipe's rate is that of two FMAs, but one issue slot) and
+// are laid out so that a converted input serves many taps: the FMAs, 49 per
+// value, bound them.  Threads of a block share cpb channel pairs (the block's
+// y index picks which); thread t takes pair t % cpb at position t / cpb.
+constexpr int DW_PX = 8;        // pixels of a row per thread
+constexpr int DW_THREADS = 256;
+constexpr int DWG_THREADS = 256;  // two halves: tap rows 0..3 and 4..6
+
+__device__ __forceinline__ float2 unpack2(uint32_t u) {
+  return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+}
 
 // Y = bias + sum_taps w * X (FLIP = 0), or the data gradient dX = sum_taps
 // w[6-ky][6-kx] * dY[y+ky-3][x+kx-3] (FLIP = 1, X = dY, no bias).  A thread
-// owns one channel pair and eight consecutive pixels of one row; block row y
-// = image row (b, y).
-template <bool FLIP>
-__global__ void __launch_bounds__(256, 4) dw7_kernel(const bf162 *__restrict__ X,
-                                                  const float *__restrict__ w,
-                                                  const float *__restrict__ bias, int B, int H,
-                                                  int W, int C, bf162 *__restrict__ Y) {
-  constexpr int NPX = 8;  // pixels per thread
-  const int cp2 = C >> 1, groups = (W + NPX - 1) / NPX, per_row = groups * cp2, rows = B * H;
-  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
-    const int b = r / H, y = r - b * H;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < per_row; t += gridDim.x * blockDim.x) {
-      const int cp = t % cp2, x0 = (t / cp2) * NPX;
-      float2 acc[NPX];
-      const float2 b0 = bias ? make_float2(bias[2 * cp], bias[2 * cp + 1]) : make_float2(0.f, 0.f);
+// owns eight pixels of R consecutive rows: each input row is loaded and
+// converted once (14 values) and serves the up to R output rows it reaches,
+// 56 packed FMAs each, taps in order (ky, then kx) per output, so the sums
+// are those of one output computed alone.  CT: the channel count when known
+// (the loads' offsets are then immediates), else 0.
+// 64 channels, 32 x 128^2 (33.5M values; 42 us of FMAs, 20 us of copy
+// bandwidth): 96 us, half of its issue slots empty on the weights' shared-memory
+// loads; 240 us with one row per thread, scalar FMAs and a bounds check per
+// load.  Four rows take the registers of two resident blocks (three rows 105,
+// two rows at three blocks 114 us); one row is for images whose positions do
+// not fill the GPU at four rows per thread.
+template <bool FLIP, int R, int CT>
+__global__ void __launch_bounds__(DW_THREADS, 2)
+    dw7_kernel(const uint32_t *__restrict__ X, const float *__restrict__ w,
+               const float *__restrict__ bias, int B, int H, int W, int C_, int cpb_,
+               uint32_t *__restrict__ Y) {
+  const int C = CT ? CT : C_;
+  const int cpb = CT ? (CT / 2 < 32 ? CT / 2 : 32) : cpb_;
+  const int cp2 = C >> 1;
+  extern __shared__ float2 s_w[];  // [49][cpb], tap order of the sum
+  const int cp0 = blockIdx.y * cpb;
+  for (int i = threadIdx.x; i < 49 * cpb; i += DW_THREADS) {
+    const int tap = i / cpb, c = cp0 + i % cpb;
+    s_w[i] = c < cp2 ? __ldg(reinterpret_cast<const float2 *>(w + (FLIP ? 48 - tap : tap) * C) + c)
+                     : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  const int slots = DW_THREADS / cpb;
+  const int slot = threadIdx.x / cpb, lc = threadIdx.x - slot * cpb, cp = cp0 + lc;
+  if (slot >= slots || cp >= cp2) return;
+  const int gx = (W + DW_PX - 1) / DW_PX, gy = (H + R - 1) / R;
+  const int64_t npos = (int64_t)B * gy * gx;
+  const float2 *wl = s_w + lc;
+  const float2 b0 = bias ? make_float2(bias[2 * cp], bias[2 * cp + 1]) : make_float2(0.f, 0.f);
+  for (int64_t pos = (int64_t)blockIdx.x * slots + slot; pos < npos;
+       pos += (int64_t)gridDim.x * slots) {
+    const int x0 = (int)(pos % gx) * DW_PX;
+    const int64_t rr = pos / gx;
+    const int y0 = (int)(rr % gy) * R, b = (int)(rr / gy);
+    uint32_t in_x = 0;  // which of the 14 columns lie in the image
 #pragma unroll
-      for (int i = 0; i < NPX; ++i) acc[i] = b0;
+    for (int k = 0; k < DW_PX + 6; ++k)
+      in_x |= (unsigned)(x0 + k - 3) < (unsigned)W ? 1u << k : 0u;
+    float2 acc[R][DW_PX];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int i = 0; i < DW_PX; ++i) acc[r][i] = b0;
+    // input rows ylo..yhi lie in the image; the next row's loads are issued
+    // before the current row's FMAs
+    const int ylo = max(y0 - 3, 0), yhi = min(y0 + R + 2, H - 1);
+    uint32_t raw[DW_PX + 6];
+    auto load_row = [&](int yy) {
+      const uint32_t *row = X + ((int64_t)(b * H + yy) * W + (x0 - 3)) * cp2 + cp;
+      if (in_x == (1u << (DW_PX + 6)) - 1u) {  // no checks away from the image's sides
+#pragma unroll
+        for (int k = 0; k < DW_PX + 6; ++k) raw[k] = __ldg(row + k * cp2);
+      } else {
+#pragma unroll
+        for (int k = 0; k < DW_PX + 6; ++k) raw[k] = (in_x >> k) & 1u ? __ldg(row + k * cp2) : 0u;
+      }
+    };
+    load_row(ylo);
 #pragma unroll 1
-      for (int ky = 0; ky < 7; ++ky) {
-        const int yy = y + ky - 3;
-        if (yy < 0 || yy >= H) continue;
-        const bf162 *row = X + (size_t)(b * H + yy) * W * cp2 + cp;
-        float2 in[NPX + 6];
+    for (int yy = ylo; yy <= yhi; ++yy) {
+      float2 in[DW_PX + 6];
 #pragma unroll
-        for (int k = 0; k < NPX + 6; ++k) {
-          const int xx = x0 + k - 3;
-          in[k] = (xx >= 0 && xx < W) ? ld2(row + (size_t)xx * cp2) : make_float2(0.f, 0.f);
-        }
-        const int wy = FLIP ? 6 - ky : ky;
+      for (int k = 0; k < DW_PX + 6; ++k) in[k] = unpack2(raw[k]);
+      if (yy < yhi) load_row(yy + 1);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int ky = yy - y0 - r + 3;
+        if (ky < 0 || ky > 6) continue;
+        const float2 *wr = wl + ky * 7 * cpb;
 #pragma unroll
         for (int kx = 0; kx < 7; ++kx) {
-          const int wx = FLIP ? 6 - kx : kx;
-          const float2 wv = __ldg(reinterpret_cast<const float2 *>(w + (wy * 7 + wx) * C) + cp);
+          const float2 wv = wr[kx * cpb];
 #pragma unroll
-          for (int i = 0; i < NPX; ++i) {
-            acc[i].x = fmaf(wv.x, in[i + kx].x, acc[i].x);
-            acc[i].y = fmaf(wv.y, in[i + kx].y, acc[i].y);
-          }
+          for (int i = 0; i < DW_PX; ++i) acc[r][i] = __ffma2_rn(wv, in[i + kx], acc[r][i]);
         }
       }
-      bf162 *out = Y + (size_t)r * W * cp2 + cp;
+    }
 #pragma unroll
-      for (int i = 0; i < NPX; ++i)
-        if (x0 + i < W) out[(size_t)(x0 + i) * cp2] = __floats2bfloat162_rn(acc[i].x, acc[i].y);
+    for (int r = 0; r < R; ++r) {
+      if (y0 + r >= H) break;
+      uint32_t *out = Y + ((int64_t)(b * H + y0 + r) * W + x0) * cp2 + cp;
+#pragma unroll
+      for (int i = 0; i < DW_PX; ++i)
+        if (x0 + i < W) {
+          const bf162 v = __floats2bfloat162_rn(acc[r][i].x, acc[r][i].y);
+          out[i * cp2] = *reinterpret_cast<const uint32_t *>(&v);
+        }
     }
   }
 }
 
-// Partial weight/bias gradients: part[chunk][50][C] (tap 49 = bias) with
-// chunk = blockIdx.x over image rows r = chunk, chunk + gridDim.x, ...  A
-// thread owns channel pair cp and tap row ky and slides a 7-pixel window of X
-// along each row, so every load is used by seven taps.
-__global__ void dw7_wgrad_kernel(const bf162 *__restrict__ X, const bf162 *__restrict__ dY,
-                                 int B, int H, int W, int C, float *__restrict__ part) {
-  const int cp2 = C >> 1;
-  const int cp = blockIdx.y * blockDim.x + threadIdx.x, ky = threadIdx.y;
-  if (cp >= cp2) return;
-  float2 acc[7], accb = make_float2(0.f, 0.f);
+// Partial weight / bias gradients: part[blockIdx.x][50][C] (tap 49 = bias).  A
+// thread keeps the sums of its tap rows and channel pair and walks stretches of `seg`
+// pixels of an input row: per pixel one new value of X (a window of seven in
+// registers) meets the seven values of dY above and below it, 49 packed FMAs
+// for eight loads, split over two halves of the block by tap rows (28 sums
+// fit 128 registers; all 49 in one thread measured 264 us, the loads of its
+// 12 warps per SM in the open).  The block's positions are then added in
+// order.  64 channels, 32 x 128^2: 132 us against 203 us with a thread per tap
+// row, which read a pixel's dY and X for seven FMAs.
+template <int K0, int NK, int CT>
+__device__ __forceinline__ void dw7_wgrad_rows(const uint32_t *__restrict__ X,
+                                               const uint32_t *__restrict__ dY, int B, int H, int W,
+                                               int cp2_, int cp, int seg, int64_t first,
+                                               int64_t stride, float2 (&acc)[28], float2 &accb) {
+  const int cp2 = CT ? CT / 2 : cp2_;
+  const int nseg = (W + seg - 1) / seg;
+  const int64_t items = (int64_t)B * H * nseg, grow = (int64_t)W * cp2;
+  for (int64_t it = first; it < items; it += stride) {
+    const int xs = (int)(it % nseg) * seg, xe = min(W, xs + seg);
+    const int64_t r = it / nseg;
+    const int yy = (int)(r % H);
+    const uint32_t *xr = X + r * grow + cp;
+    // dY row of tap row K0 + k: yy - K0 - k + 3 (outside the image: some row
+    // of it, its values masked to zero)
+    const uint32_t *gp[NK];
+    uint32_t gm[NK];
 #pragma unroll
-  for (int k = 0; k < 7; ++k) acc[k] = make_float2(0.f, 0.f);
-  for (int r = blockIdx.x; r < B * H; r += gridDim.x) {
-    const int b = r / H, y = r - b * H, yy = y + ky - 3;
-    const bool rowok = yy >= 0 && yy < H;
-    if (!rowok && ky != 3) continue;
-    const bf162 *g = dY + (size_t)r * W * cp2 + cp;
-    const bf162 *xr = X + (size_t)(b * H + (rowok ? yy : y)) * W * cp2 + cp;
-    float2 win[7];
-#pragma unroll
-    for (int k = 0; k < 7; ++k) {
-      const int xx = k - 3;
-      win[k] = (xx >= 0 && xx < W) ? ld2(xr + (size_t)xx * cp2) : make_float2(0.f, 0.f);
+    for (int k = 0; k < NK; ++k) {
+      const bool in = (unsigned)(yy - K0 - k + 3) < (unsigned)H;
+      gm[k] = in ? 0xffffffffu : 0u;
+      gp[k] = dY + (r + (in ? 3 - K0 - k : 0)) * grow + cp;
     }
-    for (int x = 0; x < W; ++x) {
-      const float2 gv = ld2(g + (size_t)x * cp2);
-      accb.x += gv.x;
-      accb.y += gv.y;
+    float2 win[8];  // the value at column x + k - 3 in slot k mod 8
 #pragma unroll
-      for (int k = 0; k < 7; ++k) {
-        acc[k].x = fmaf(gv.x, win[k].x, acc[k].x);
-        acc[k].y = fmaf(gv.y, win[k].y, acc[k].y);
+    for (int k = 0; k < 6; ++k) {
+      const int xx = xs + k - 3;
+      win[k] = unpack2(xx >= 0 && xx < W ? __ldg(xr + (int64_t)xx * cp2) : 0u);
+    }
+    uint32_t raw[NK + 1];  // the pixel's dY values and the window's new X, one pixel ahead
+    auto load_px = [&](int xx) {
+#pragma unroll
+      for (int k = 0; k < NK; ++k) raw[k] = xx < xe ? __ldg(gp[k] + (int64_t)xx * cp2) & gm[k] : 0u;
+      raw[NK] = xx < xe && xx + 3 < W ? __ldg(xr + (int64_t)(xx + 3) * cp2) : 0u;
+    };
+    auto pixel = [&](int u, auto &&load_next) {
+      float2 g[NK];
+#pragma unroll
+      for (int k = 0; k < NK; ++k) g[k] = unpack2(raw[k]);
+      win[(u + 6) % 8] = unpack2(raw[NK]);
+      load_next();
+      if (K0 <= 3 && 3 < K0 + NK) {
+        accb.x += g[3 - K0 < NK ? 3 - K0 : 0].x;
+        accb.y += g[3 - K0 < NK ? 3 - K0 : 0].y;
       }
 #pragma unroll
-      for (int k = 0; k < 6; ++k) win[k] = win[k + 1];
-      const int xn = x + 4;
-      win[6] = xn < W ? ld2(xr + (size_t)xn * cp2) : make_float2(0.f, 0.f);
+      for (int k = 0; k < NK; ++k)
+#pragma unroll
+        for (int kx = 0; kx < 7; ++kx)
+          acc[k * 7 + kx] = __ffma2_rn(g[k], win[(u + kx) % 8], acc[k * 7 + kx]);
+    };
+    load_px(xs);
+    int x = xs;
+#pragma unroll 1
+    for (; x + 8 <= xe && x + 11 < W; x += 8) {  // every load in the row: no checks
+      const uint32_t *xp = xr + (int64_t)(x + 4) * cp2;
+      const uint32_t *gx[NK];
+#pragma unroll
+      for (int k = 0; k < NK; ++k) gx[k] = gp[k] + (int64_t)(x + 1) * cp2;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        pixel(u, [&] {
+#pragma unroll
+          for (int k = 0; k < NK; ++k) raw[k] = __ldg(gx[k] + u * cp2) & gm[k];
+          raw[NK] = __ldg(xp + u * cp2);
+        });
+    }
+#pragma unroll 1
+    for (; x < xe; x += 8)  // (past the stretch: zeros)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) pixel(u, [&] { load_px(x + u + 1); });
+  }
+}
+
+template <int CT>
+__global__ void __launch_bounds__(DWG_THREADS, 2)
+    dw7_wgrad_kernel(const uint32_t *__restrict__ X, const uint32_t *__restrict__ dY, int B, int H,
+                     int W, int C_, int cpb_, int seg, float *__restrict__ part) {
+  const int C = CT ? CT : C_;
+  const int cpb = CT ? (CT / 2 < 32 ? CT / 2 : 32) : cpb_;
+  const int cp2 = C >> 1;
+  const int half = threadIdx.x / (DWG_THREADS / 2), t = threadIdx.x % (DWG_THREADS / 2);
+  const int slots = DWG_THREADS / 2 / cpb;
+  const int slot = t / cpb, lc = t - slot * cpb;
+  const int cp = blockIdx.y * cpb + lc;
+  const bool on = slot < slots && cp < cp2;
+  float2 acc[28], accb = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < 28; ++k) acc[k] = make_float2(0.f, 0.f);
+  const int64_t first = (int64_t)blockIdx.x * slots + slot, stride = (int64_t)gridDim.x * slots;
+  if (on) {
+    if (half == 0)
+      dw7_wgrad_rows<0, 4, CT>(X, dY, B, H, W, cp2, cp, seg, first, stride, acc, accb);
+    else
+      dw7_wgrad_rows<4, 3, CT>(X, dY, B, H, W, cp2, cp, seg, first, stride, acc, accb);
+  }
+  // positions of the block, added in order into shared memory
+  extern __shared__ float2 s_w[];  // [50][cpb]
+  for (int i = threadIdx.x; i < 50 * cpb; i += DWG_THREADS) s_w[i] = make_float2(0.f, 0.f);
+  for (int k = 0; k < slots; ++k) {
+    __syncthreads();
+    if (on && slot == k) {
+      const int t0 = half * 28, n = half ? 21 : 28;
+#pragma unroll
+      for (int j = 0; j < 28; ++j) {
+        if (j >= n) break;
+        float2 v = s_w[(t0 + j) * cpb + lc];
+        v.x += acc[j].x;
+        v.y += acc[j].y;
+        s_w[(t0 + j) * cpb + lc] = v;
+      }
+      if (!half) {
+        float2 v = s_w[49 * cpb + lc];
+        v.x += accb.x;
+        v.y += accb.y;
+        s_w[49 * cpb + lc] = v;
+      }
     }
   }
-  float *pb = part + (size_t)blockIdx.x * 50 * C + 2 * cp;
-#pragma unroll
-  for (int k = 0; k < 7; ++k) {
-    pb[(ky * 7 + k) * C] = acc[k].x;
-    pb[(ky * 7 + k) * C + 1] = acc[k].y;
-  }
-  if (ky == 3) {
-    pb[49 * C] = accb.x;
-    pb[49 * C + 1] = accb.y;
+  __syncthreads();
+  for (int i = threadIdx.x; i < 50 * cpb; i += DWG_THREADS) {
+    const int k = i / cpb, c = blockIdx.y * cpb + i % cpb;
+    if (c < cp2) {
+      float *dst = part + ((size_t)blockIdx.x * 50 + k) * C + 2 * c;
+      dst[0] = s_w[i].x;
+      dst[1] = s_w[i].y;
+    }
   }
 }
 
@@ -1122,29 +1269,66 @@ extern "C" pe_status pe_nn_im2col3(const void *X, int32_t B, int32_t H, int32_t 
 
 static bool al4(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 3) == 0; }
 
+// Channel pairs a depthwise block shares.
+static int dw_cpb(int32_t C) { return C / 2 < 32 ? C / 2 : 32; }
+
+template <bool FLIP, int R>
+static pe_status launch_dw7_rows(const void *X, const float *w, const float *bias, int B, int H,
+                                 int W, int C, void *Y, cudaStream_t s) {
+  const int cpb = dw_cpb(C), slots = DW_THREADS / cpb, gy = (C / 2 + cpb - 1) / cpb;
+  const int64_t npos = (int64_t)B * ((H + R - 1) / R) * ((W + DW_PX - 1) / DW_PX);
+  int64_t gx = (npos + slots - 1) / slots;
+  const int64_t cap = ((int64_t)n_sms() * 8 + gy - 1) / gy;  // a few positions per weight load
+  if (gx > cap) gx = cap;
+  const dim3 grid((unsigned)gx, (unsigned)gy);
+  const size_t smem = sizeof(float2) * 49 * cpb;
+  const uint32_t *x = static_cast<const uint32_t *>(X);
+  uint32_t *y = static_cast<uint32_t *>(Y);
+  switch (C) {
+    case 32: dw7_kernel<FLIP, R, 32><<<grid, DW_THREADS, smem, s>>>(x, w, bias, B, H, W, C, cpb, y); break;
+    case 64: dw7_kernel<FLIP, R, 64><<<grid, DW_THREADS, smem, s>>>(x, w, bias, B, H, W, C, cpb, y); break;
+    case 128: dw7_kernel<FLIP, R, 128><<<grid, DW_THREADS, smem, s>>>(x, w, bias, B, H, W, C, cpb, y); break;
+    case 256: dw7_kernel<FLIP, R, 256><<<grid, DW_THREADS, smem, s>>>(x, w, bias, B, H, W, C, cpb, y); break;
+    default: dw7_kernel<FLIP, R, 0><<<grid, DW_THREADS, smem, s>>>(x, w, bias, B, H, W, C, cpb, y);
+  }
+  PE_TRY_LAUNCH("dw7_kernel");
+  return PE_OK;
+}
+
+// Four rows per thread when that still gives every SM its two blocks of
+// threads, else one.
+template <bool FLIP>
+static pe_status launch_dw7(const void *X, const float *w, const float *bias, int B, int H, int W,
+                            int C, void *Y, cudaStream_t s) {
+  const int64_t threads4 = (int64_t)B * ((H + 3) / 4) * ((W + DW_PX - 1) / DW_PX) * (C / 2);
+  return threads4 >= (int64_t)n_sms() * 2 * DW_THREADS
+             ? launch_dw7_rows<FLIP, 4>(X, w, bias, B, H, W, C, Y, s)
+             : launch_dw7_rows<FLIP, 1>(X, w, bias, B, H, W, C, Y, s);
+}
+
 extern "C" pe_status pe_nn_dwconv7(const void *X, const float *w, const float *bias, int32_t B,
                                    int32_t H, int32_t W, int32_t C, void *Y, void *stream) {
   NN_CHECK_STREAM;
   if (!X || !w || !Y || B <= 0 || H <= 0 || W <= 0 || C <= 0 || (C & 1) || !al4(X) || !al4(Y) ||
       (reinterpret_cast<uintptr_t>(w) & 7))
     return pe_fail(PE_EINVAL, "pe_nn_dwconv7: bad arguments (C even, aligned buffers)");
-  const int per_row = ((W + 7) / 8) * (C / 2);
-  dim3 grid((per_row + 255) / 256, (unsigned)(B * H < 65535 ? B * H : 65535));
-  dw7_kernel<false><<<grid, 256, 0, s>>>(static_cast<const bf162 *>(X), w, bias, B, H, W, C,
-                                         static_cast<bf162 *>(Y));
-  PE_TRY_LAUNCH("dw7_kernel");
-  return PE_OK;
+  return launch_dw7<false>(X, w, bias, B, H, W, C, Y, s);
 }
 
-// Chunks (image rows per partial) of the weight gradient: fixed by the shape.
-static int dw_chunks(int32_t B, int32_t H) {
-  int64_t r = (int64_t)B * H;
-  return (int)(r < 1024 ? (r < 1 ? 1 : r) : 1024);
+// Stretch of a row a weight-gradient thread walks at a time, and the partials
+// per channel chunk: about 304 blocks over the chunks (two per SM; a constant,
+// so that the order of the sums does not depend on the device).
+static int dw_seg(int32_t W) { return W >= 128 ? 64 : (W >= 64 ? 32 : 16); }
+static int dw_chunks(int32_t B, int32_t H, int32_t W, int32_t C) {
+  const int cpb = dw_cpb(C), slots = DWG_THREADS / 2 / cpb, gy = (C / 2 + cpb - 1) / cpb;
+  const int64_t items = (int64_t)B * H * ((W + dw_seg(W) - 1) / dw_seg(W));
+  const int64_t need = (items + slots - 1) / slots, most = (304 + gy - 1) / gy;
+  return (int)(need < most ? need : most);
 }
 
 extern "C" size_t pe_nn_dwconv7_bwd_workspace(int32_t B, int32_t H, int32_t W, int32_t C) {
-  (void)W;
-  return (size_t)dw_chunks(B, H) * 50 * C * sizeof(float) + 256;
+  if (B <= 0 || H <= 0 || W <= 0 || C < 2) return 0;
+  return (size_t)dw_chunks(B, H, W, C) * 50 * C * sizeof(float) + 256;
 }
 
 // dX (nullable), dw [7][7][C] and db [C] (FP32, overwritten).
@@ -1156,21 +1340,26 @@ extern "C" pe_status pe_nn_dwconv7_bwd(const void *X, const void *dY, const floa
       !al4(dY) || (dX && !al4(dX)) || (reinterpret_cast<uintptr_t>(w) & 7))
     return pe_fail(PE_EINVAL, "pe_nn_dwconv7_bwd: bad arguments (C even, aligned buffers)");
   if (dX) {
-    const int per_row = ((W + 7) / 8) * (C / 2);
-    dim3 grid((per_row + 255) / 256, (unsigned)(B * H < 65535 ? B * H : 65535));
-    dw7_kernel<true><<<grid, 256, 0, s>>>(static_cast<const bf162 *>(dY), w, nullptr, B, H, W, C,
-                                          static_cast<bf162 *>(dX));
-    PE_TRY_LAUNCH("dw7_kernel");
+    const pe_status st = launch_dw7<true>(dY, w, nullptr, B, H, W, C, dX, s);
+    if (st != PE_OK) return st;
   }
   if (dw || db) {
-    const int chunks = dw_chunks(B, H);
+    const int chunks = dw_chunks(B, H, W, C);
     size_t need = (size_t)chunks * 50 * C * sizeof(float);
     if (!ws || ws_bytes < need) return pe_fail(PE_ENOMEM, "pe_nn_dwconv7_bwd: workspace");
     float *part = static_cast<float *>(ws);
-    const int cp2 = C / 2, bx = cp2 < 32 ? cp2 : 32;
-    dim3 grid((unsigned)chunks, (unsigned)((cp2 + bx - 1) / bx));
-    dw7_wgrad_kernel<<<grid, dim3(bx, 7), 0, s>>>(static_cast<const bf162 *>(X),
-                                                  static_cast<const bf162 *>(dY), B, H, W, C, part);
+    const int cpb = dw_cpb(C);
+    const dim3 grid((unsigned)chunks, (unsigned)((C / 2 + cpb - 1) / cpb));
+    const size_t smem = sizeof(float2) * 50 * cpb;
+    const uint32_t *x = static_cast<const uint32_t *>(X), *g = static_cast<const uint32_t *>(dY);
+    const int seg = dw_seg(W);
+    switch (C) {
+      case 32: dw7_wgrad_kernel<32><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part); break;
+      case 64: dw7_wgrad_kernel<64><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part); break;
+      case 128: dw7_wgrad_kernel<128><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part); break;
+      case 256: dw7_wgrad_kernel<256><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part); break;
+      default: dw7_wgrad_kernel<0><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part);
+    }
     PE_TRY_LAUNCH("dw7_wgrad_kernel");
     // part[chunk][50][C]: taps 0..48 -> dw, 49 -> db; sum the chunks in
     // order into chunk 0 (a block reads only the columns it writes)

@@ -115,3 +115,36 @@ def test_streaming_contraction_gives_up_and_recovers(mode):
     assert lib.pe_stream_check(stream) == 0
     pre = A.double() @ B.double().T + (R.double() if mode == "residual" else 0.0)
     assert rel(out, torch.nn.functional.gelu(pre) if mode == "gelu" else pre) < BF_TOL
+
+
+# ---- depthwise 7x7 --------------------------------------------------------------
+
+# images smaller than the stencil, ragged rows and columns, odd pair counts and
+# more than one chunk of channel pairs, and enough positions for four rows per
+# thread; the weight gradient's FP32 sums (over at most 2 * 96 * 200 pixels, in
+# runs of a few hundred) err below 1e-5
+@pytest.mark.parametrize("B,H,W,C", [(1, 1, 1, 2), (2, 3, 5, 6), (1, 9, 17, 32), (2, 12, 33, 40),
+                                     (1, 7, 70, 130), (2, 96, 200, 64), (3, 130, 131, 256)])
+def test_depthwise(B, H, W, C):
+    o, g = ops(), gen(B + H + W + C)
+    x, dy = rnd(g, B, H, W, C).to(BF), rnd(g, B, H, W, C).to(BF)
+    w, b = rnd(g, 7, 7, C) / 7, rnd(g, C)
+    P = B * H * W
+    y, dx = torch.empty(P, C, dtype=BF, device=DEV), torch.empty(P, C, dtype=BF, device=DEV)
+    dw, db = torch.empty(7, 7, C, device=DEV), torch.empty(C, device=DEV)
+    o.dw(x, w, b, B, H, W, C, y)
+    o.dw_bwd(x, dy, w, B, H, W, C, dx, dw, db)
+    pad = lambda t: torch.nn.functional.pad(t.double(), (0, 0, 3, 3, 3, 3))
+    xp, gp = pad(x), pad(dy)
+    ry = b.double().expand(B, H, W, C).clone()
+    rx, rw = torch.zeros_like(ry), torch.empty(7, 7, C, dtype=torch.float64, device=DEV)
+    for i in range(7):
+        for j in range(7):
+            win = xp[:, i:i + H, j:j + W]
+            ry += w[i, j].double() * win
+            rx += w[6 - i, 6 - j].double() * gp[:, i:i + H, j:j + W]
+            rw[i, j] = (win * dy.double()).sum((0, 1, 2))
+    assert rel(y.view(B, H, W, C), ry) < BF_TOL
+    assert rel(dx.view(B, H, W, C), rx) < BF_TOL
+    assert rel(dw, rw) < 1e-5
+    assert rel(db, dy.double().sum((0, 1, 2))) < 1e-5
