@@ -148,3 +148,28 @@ def test_depthwise(B, H, W, C):
     assert rel(dx.view(B, H, W, C), rx) < BF_TOL
     assert rel(dw, rw) < 1e-5
     assert rel(db, dy.double().sum((0, 1, 2))) < 1e-5
+
+
+# ---- LayerNorm ------------------------------------------------------------------
+
+# one pixel, a block's 64 and its neighbours, more pixels than resident blocks;
+# every channel count of the four-threads-per-pixel kernels and one beside them
+@pytest.mark.parametrize("C", [32, 40, 64, 128, 256])
+@pytest.mark.parametrize("P", [1, 63, 65, 100_003])
+def test_layernorm(P, C):
+    o, g = ops(), gen(P + C)
+    x, dy = (rnd(g, P, C) + 0.5).to(BF), rnd(g, P, C).to(BF)
+    gam, bet = rnd(g, C), rnd(g, C)
+    y, dx = torch.empty(P, C, dtype=BF, device=DEV), torch.empty(P, C, dtype=BF, device=DEV)
+    mean, rstd = torch.empty(P, device=DEV), torch.empty(P, device=DEV)
+    dg, db = torch.empty(C, device=DEV), torch.empty(C, device=DEV)
+    o.ln(x, gam, bet, P, C, y, mean, rstd)
+    o.ln_bwd(dy, x, gam, mean, rstd, P, C, dx, dg, db)
+    xd = x.double().requires_grad_(True)
+    gd, bd = gam.double().requires_grad_(True), bet.double().requires_grad_(True)
+    ref = torch.nn.functional.layer_norm(xd, (C,), gd, bd, 1e-6)
+    ref.backward(dy.double())
+    assert rel(y, ref.detach()) < BF_TOL
+    assert rel(mean, x.double().mean(1)) < 1e-5
+    assert rel(dx, xd.grad) < BF_TOL
+    assert rel(dg, gd.grad) < 1e-5 and rel(db, bd.grad) < 1e-5
