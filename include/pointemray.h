@@ -592,6 +592,14 @@ size_t pe_nn_colsum_workspace(int64_t M, int32_t N);
 pe_status pe_nn_colsum(const void *X, int64_t M, int32_t N, int64_t ld, float *out,
                        int32_t accumulate, void *ws, size_t ws_bytes, void *stream);
 
+/* Weight and bias gradient of a linear layer in one pass: FP32 dW [N][K]
+ * (contiguous, overwritten) = sum over p < P of dY[p][n] X[p][k], db [N]
+ * (nullable, overwritten) = sum over p of dY[p][n]; BF16 dY [P][ldy], X [P][ldx]. */
+size_t pe_nn_linear_wgrad_workspace(int64_t P, int32_t N, int32_t K);
+pe_status pe_nn_linear_wgrad(const void *dY, int64_t ldy, const void *X, int64_t ldx, int64_t P,
+                             int32_t N, int32_t K, float *dW, float *db, void *ws, size_t ws_bytes,
+                             void *stream);
+
 /* dst [Cc][R] = transpose of src [R][Cc] (BF16, row-major, distinct buffers). */
 pe_status pe_nn_transpose(const void *src, int32_t R, int32_t Cc, void *dst, void *stream);
 

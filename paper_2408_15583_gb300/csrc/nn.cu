@@ -724,9 +724,9 @@ __global__ void __launch_bounds__(256) ln_fwd_narrow_kernel(
 // pixels' 64-byte pieces).  The sums are those of a warp per pixel with lane l
 // on channels l, l + 32, ...: over i in the thread, then the butterfly 16, 8
 // (two shuffles of the eight values) and 4, 2, 1 (in the thread), so the
-// results are the same bit for bit.  The warp per pixel spent 224 instructions
-// on a 64-channel pixel with 2-byte loads: 118 us for 524288 pixels (134 MB, 20
-// us of copy bandwidth).
+// results are the same bit for bit.  64 channels, 524288 pixels: forward 28 us
+// (134 MB, 20 us of copy bandwidth), backward 41 us (201 MB, 30 us); a warp per
+// pixel took 224 instructions a pixel over 2-byte loads, 118 and 130 us.
 template <int NI>
 struct ln_quad {
   // the butterfly sum of the 32 per-lane values whose eight this thread holds
@@ -1360,6 +1360,8 @@ static int64_t gemm_split(int32_t M, int32_t N, int64_t K, int64_t *kps_out) {
   return split;
 }
 
+int64_t pe_gemm_split(int32_t M, int32_t N, int64_t K) { return gemm_split(M, N, K, nullptr); }
+
 extern "C" size_t pe_nn_gemm_workspace(int32_t M, int32_t N, int64_t K) {
   if (M <= 0 || N <= 0 || K <= 0) return 0;
   const int64_t split = gemm_split(M, N, K, nullptr);
@@ -1672,6 +1674,33 @@ extern "C" pe_status pe_nn_colsum(const void *X, int64_t M, int32_t N, int64_t l
                                                                       accumulate);
   PE_TRY_LAUNCH("sum_chunks_kernel");
   return PE_OK;
+}
+
+// Workspace of pe_nn_linear_wgrad: either path's.
+extern "C" size_t pe_nn_linear_wgrad_workspace(int64_t P, int32_t N, int32_t K) {
+  if (P <= 0 || N <= 0 || K <= 0) return 0;
+  size_t a = pe_wgrad_tc_workspace(P, N, K), b = pe_nn_gemm_workspace(N, K, P),
+         c = pe_nn_colsum_workspace(P, N);
+  a = a > b ? a : b;
+  return (a > c ? a : c) + 256;
+}
+
+extern "C" pe_status pe_nn_linear_wgrad(const void *dY, int64_t ldy, const void *X, int64_t ldx,
+                                        int64_t P, int32_t N, int32_t K, float *dW, float *db,
+                                        void *ws, size_t ws_bytes, void *stream) {
+  NN_CHECK_STREAM;
+  if (!dY || !X || !dW || P <= 0 || N <= 0 || K <= 0 || ldy < N || ldx < K)
+    return pe_fail(PE_EINVAL, "pe_nn_linear_wgrad: bad arguments");
+  if (!ws || ws_bytes < pe_nn_linear_wgrad_workspace(P, N, K))
+    return pe_fail(PE_ENOMEM, "pe_nn_linear_wgrad: workspace");
+  if (g_gemm_path == 0 && pe_wgrad_tc_eligible(dY, ldy, X, ldx, P, N, K)) {
+    const pe_status st = pe_wgrad_tc(dY, ldy, X, ldx, P, N, K, dW, db, static_cast<float *>(ws), s);
+    if (st != PE_EUNSUPPORTED) return st;
+  }
+  const pe_status st = pe_nn_gemm(N, K, P, dY, 1, ldy, X, ldx, 1, dW, K, 1, nullptr, nullptr, 0,
+                                  nullptr, 0, 0, 1.0f, 0.0f, ws, ws_bytes, stream);
+  if (st != PE_OK || !db) return st;
+  return pe_nn_colsum(dY, P, N, ldy, db, 0, ws, ws_bytes, stream);
 }
 
 extern "C" pe_status pe_nn_gelu_bwd(const void *dA, const void *Z, int64_t n, void *dZ,

@@ -125,3 +125,15 @@ __device__ __forceinline__ void pe_gemm_store8(const pe_gemm_args &g, int m, int
 bool pe_gemm_tc_eligible(const pe_gemm_args &g);
 // The GEMM on the tcgen05 tensor cores (no split-K).
 pe_status pe_gemm_tc(const pe_gemm_args &g, cudaStream_t s);
+
+// Weight and bias gradient of a linear layer on the tcgen05 tensor cores:
+// dW[n][k] = sum_p dY[p][n] X[p][k], db[n] = sum_p dY[p][n] (db nullable), FP32,
+// dW contiguous; part: pe_wgrad_tc_workspace bytes.  Eligible: 16-byte aligned
+// rows.
+bool pe_wgrad_tc_eligible(const void *dY, int64_t ldy, const void *X, int64_t ldx, int64_t P, int32_t N,
+                          int32_t K);
+size_t pe_wgrad_tc_workspace(int64_t P, int32_t N, int32_t K);
+pe_status pe_wgrad_tc(const void *dY, int64_t ldy, const void *X, int64_t ldx, int64_t P, int32_t N,
+                      int32_t K, float *dW, float *db, float *part, cudaStream_t s);
+// Split-K factor of the mma.sync kernel.
+int64_t pe_gemm_split(int32_t M, int32_t N, int64_t K);

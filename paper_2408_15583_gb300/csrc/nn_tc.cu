@@ -681,6 +681,272 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
   }
 }
 
+// ---------------------------------------------------------------------------
+// Weight gradients of a linear layer: dW[n][k] = sum_p dY[p][n] X[p][k] and
+// db[n] = sum_p dY[p][n] in one pass over both matrices.
+//
+// Both operands are contiguous along their channels, so their tiles (64 pixels
+// x 64 channels, TMA with the 128-byte swizzle) are MN-major for the tensor
+// cores and the products accumulate over pixels in tensor memory: up to four
+// accumulators of 128 rows (channels of the wider operand) by up to 256
+// columns (the narrower one), so at the network's narrow levels each pixel is
+// read once.  Four more warps add up dY's columns from the same shared-memory
+// tiles (one column-sum kernel and one read of dY fewer) and write the partial
+// results at the end.  A CTA takes one tile of the result over one stretch of
+// pixels; part[split][N K + N] is then added in split order.
+//
+// The tensor cores truncate where an FP32 addition rounds, so a sum drifts with
+// the number of products added into one accumulator (1e-6 of the result after
+// 1024 pixels, 2.3e-6 after 2048, against 64 bits).  Where a tile leaves room,
+// pixel blocks take several copies of its accumulators in turn, and there are at
+// least as many sums over the pixels as the split mma.sync kernel makes.
+// Bound by reading X and dY: 64 channels, 524288 pixels, both layers of a
+// block (671 MB, 99 us of copy bandwidth) take 153 us with their partials'
+// sums, against 296 us for the split mma.sync kernel and 150 us for the column
+// sums.  Over the gradient of a 32 x 256^2 batch: 14.2 -> 4.8 ms.
+// ---------------------------------------------------------------------------
+constexpr int WG_PX = 64, WG_THREADS = 192, WG_BOX = WG_PX * 128, WG_STAGES = 4;
+
+struct wg_args {
+  int N, K;           // dW is [N][K]
+  int mt, nt;         // accumulators of a tile, columns of each
+  int sets;           // copies of the accumulators, taken in turn by pixel blocks
+  int nbx;            // 64-channel boxes of the column operand per stage
+  int tiles_n;
+  int a_is_dy;        // rows of the accumulators: dY's channels, else X's
+  int64_t P;
+  int px_per_split;   // a multiple of WG_PX
+  int stages;
+  float *part;
+  int want_db;
+  uint32_t cols;      // tensor-memory columns
+  uint32_t wait_limit;
+  unsigned int *err;
+};
+
+// MN-major tile with the 128-byte swizzle: 64 channels (128 bytes) by 8 pixels
+// per 1024-byte atom, `lbo` bytes to the next 64 channels, 1024 to the next 8
+// pixels.
+__device__ __forceinline__ uint64_t mnmajor_sw128_desc(uint32_t saddr, uint32_t lbo) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(lbo >> 4) << 16) |
+         ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+__global__ void __launch_bounds__(WG_THREADS)
+    wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                    const wg_args g) {
+  extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
+  uint8_t *base = reinterpret_cast<uint8_t *>(
+      (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  __shared__ uint64_t full[WG_STAGES], empty[WG_STAGES], accum, drain;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int s_fail;
+  __shared__ float s_db[4][512];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tm = blockIdx.y / g.tiles_n, tn = blockIdx.y % g.tiles_n;
+  const int m0 = tm * g.mt * 128, n0 = tn * g.nt;
+  const int a_boxes = 2 * g.mt;
+  const uint32_t stage_bytes = (uint32_t)(a_boxes + g.nbx) * WG_BOX;
+  const int64_t p0 = (int64_t)blockIdx.x * g.px_per_split;
+  const int64_t pe = p0 + g.px_per_split < g.P ? p0 + g.px_per_split : g.P;
+  const int nk = (int)((pe - p0 + WG_PX - 1) / WG_PX);
+  // the tile whose other operand is its first adds up dY's columns
+  const bool sums = g.want_db && (g.a_is_dy ? tn == 0 : tm == 0);
+
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    for (int s = 0; s < g.stages; ++s) {
+      mbar_init(full + s, 1);
+      mbar_init(empty + s, sums ? 5 : 1);
+    }
+    mbar_init(&accum, 1);
+    mbar_init(&drain, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     sm_u32(&tmem_slot)),
+                 "r"(g.cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      bool ok = true;
+      int kb = 0;
+      for (; kb < nk; ++kb) {
+        const int s = kb % g.stages;
+        if (!st_wait(empty + s, ((uint32_t)(kb / g.stages) & 1u) ^ 1u, g.wait_limit, &s_fail)) {
+          s_fail = 1;
+          ok = false;
+          break;
+        }
+        uint8_t *sa = base + (size_t)s * stage_bytes;
+        const int px = (int)(p0 + (int64_t)kb * WG_PX);
+        mbar_expect_tx(full + s, stage_bytes);
+        for (int b = 0; b < a_boxes; ++b) tma_load_2d(sa + b * WG_BOX, &tmA, m0 + 64 * b, px, full + s);
+        for (int b = 0; b < g.nbx; ++b)
+          tma_load_2d(sa + (a_boxes + b) * WG_BOX, &tmB, n0 + 64 * b, px, full + s);
+      }
+      if (!ok)
+        for (int k = kb > g.stages ? kb - g.stages : 0; k < kb; ++k)
+          mbar_wait(full + k % g.stages, (uint32_t)(k / g.stages) & 1u);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // both operands MN-major (bits 15 and 16), as tc_cfg::IDESC otherwise
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                             ((uint32_t)(g.nt >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+      bool ok = true;
+      for (int kb = 0; kb < nk; ++kb) {
+        const int s = kb % g.stages;
+        if (!st_wait(full + s, (uint32_t)(kb / g.stages) & 1u, g.wait_limit, &s_fail)) {
+          s_fail = 1;
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t sa = sm_u32(base + (size_t)s * stage_bytes);
+        const uint32_t sb = sa + (uint32_t)a_boxes * WG_BOX;
+        for (int i = 0; i < g.mt; ++i) {
+          const uint64_t ad = mnmajor_sw128_desc(sa + (uint32_t)(2 * i) * WG_BOX, WG_BOX);
+          const uint64_t bd = mnmajor_sw128_desc(sb, WG_BOX);
+#pragma unroll
+          for (int k = 0; k < WG_PX / 16; ++k)  // 16 pixels: two atoms of 1024 bytes
+            tc_mma(tmem + (uint32_t)((kb % g.sets * g.mt + i) * g.nt), ad + (uint64_t)(128 * k),
+                   bd + (uint64_t)(128 * k), idesc, (kb >= g.sets || k > 0) ? 1u : 0u);
+        }
+        tc_commit(empty + s);
+      }
+      if (ok) {
+        tc_commit(&accum);
+      } else {
+        tc_commit(&drain);
+        mbar_wait(&drain, 0u);
+      }
+    }
+  } else {
+    const int t = threadIdx.x - 64, j = t & 7, r0 = t >> 3;
+    bool ok = true;
+    float *out = g.part + (int64_t)blockIdx.x * ((int64_t)g.N * g.K + g.N);
+    if (sums) {
+      // dY's columns: thread t adds chunk j (eight channels) of every box at
+      // pixels r0, r0 + 16, ...
+      const int nd = g.a_is_dy ? a_boxes : g.nbx, d0 = g.a_is_dy ? 0 : a_boxes;
+      float sum[8][8];
+#pragma unroll
+      for (int b = 0; b < 8; ++b)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sum[b][e] = 0.0f;
+      for (int kb = 0; kb < nk; ++kb) {
+        const int s = kb % g.stages;
+        ok = __all_sync(0xffffffffu,
+                        st_wait(full + s, (uint32_t)(kb / g.stages) & 1u, g.wait_limit, &s_fail));
+        if (!ok) break;
+        const uint8_t *sd = base + (size_t)s * stage_bytes + (size_t)d0 * WG_BOX + r0 * 128 +
+                            ((j ^ (r0 & 7)) << 4);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+          if (b < nd) {
+#pragma unroll
+            for (int r = 0; r < WG_PX / 16; ++r) {
+              const uint4 u = *reinterpret_cast<const uint4 *>(sd + b * WG_BOX + r * 16 * 128);
+              const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                sum[b][2 * e] += __uint_as_float(w[e] << 16);
+                sum[b][2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
+              }
+            }
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty + s);
+      }
+#pragma unroll
+      for (int b = 0; b < 8; ++b)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          float v = sum[b][e];
+          v += __shfl_xor_sync(0xffffffffu, v, 8);
+          v += __shfl_xor_sync(0xffffffffu, v, 16);
+          if (lane < 8) s_db[warp - 2][64 * b + 8 * j + e] = v;
+        }
+      asm volatile("bar.sync 1, 128;\n" ::: "memory");
+      const int w0 = g.a_is_dy ? m0 : n0, wn = g.a_is_dy ? g.mt * 128 : g.nt;
+      if (ok)
+        for (int c = t; c < wn; c += 128)
+          if (w0 + c < g.N)
+            out[(int64_t)g.N * g.K + w0 + c] = (s_db[0][c] + s_db[1][c]) + (s_db[2][c] + s_db[3][c]);
+    }
+    ok = __all_sync(0xffffffffu, ok && st_wait(&accum, 0u, g.wait_limit, &s_fail));
+    if (!ok) {
+      s_fail = 1;
+    } else {
+      tc_fence_after();
+      const int quad = warp & 3, na = g.a_is_dy ? g.N : g.K, nb = g.a_is_dy ? g.K : g.N;
+      for (int i = 0; i < g.mt; ++i) {
+        const int m = m0 + i * 128 + quad * 32 + lane;
+        for (int c = 0; c < g.nt; c += 16) {
+          float v[16];
+          tc_ld16(tmem + (uint32_t)(i * g.nt + c) + ((uint32_t)(quad * 32) << 16), v);
+          for (int z = 1; z < g.sets && z < nk; ++z) {
+            float a[16];
+            tc_ld16(tmem + (uint32_t)((z * g.mt + i) * g.nt + c) + ((uint32_t)(quad * 32) << 16), a);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] += a[e];
+          }
+          if (m >= na) continue;
+          if (g.a_is_dy) {
+            float *dst = out + (int64_t)m * g.K + n0 + c;
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+              if (n0 + c + e < nb) dst[e] = v[e];
+          } else {  // transposed: consecutive lanes write consecutive k
+            float *dst = out + (int64_t)(n0 + c) * g.K + m;
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+              if (n0 + c + e < nb) dst[(int64_t)e * g.K] = v[e];
+          }
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && s_fail) atomicOr(g.err, PE_ERR_TIMEOUT);
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(g.cols)
+                 : "memory");
+  }
+}
+
+// dW, db = the partials added in split order: eight lanes take splits z, z + 8,
+// ..., and their sums are added in order.
+__global__ void wgrad_reduce_kernel(const float *__restrict__ part, int splits, int64_t nw,
+                                    int64_t n_all, float *__restrict__ dW, float *__restrict__ db) {
+  __shared__ float red[8][33];
+  const int64_t t = (int64_t)blockIdx.x * 32 + threadIdx.x;
+  float v = 0.0f;
+  if (t < n_all)
+    for (int z = threadIdx.y; z < splits; z += 8) v += part[(int64_t)z * n_all + t];
+  red[threadIdx.y][threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.y == 0 && t < n_all) {
+    float s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += red[k][threadIdx.x];
+    if (t < nw) dW[t] = s;
+    else if (db) db[t - nw] = s;
+  }
+}
+
 typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                     const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                     const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -837,6 +1103,48 @@ pe_status launch_stream_mode(int mode, const pe_gemm_args &g, cudaStream_t s) {
   }
 }
 
+// Tile and split of a weight gradient.  The wider operand gives the rows; its
+// 128-row accumulators share a tile as far as tensor memory (512 columns) and
+// shared memory allow.  About 304 CTAs (two per SM where their tensor memory
+// fits; a constant, so that sums do not depend on the device), at least 512
+// pixels each.
+struct wg_plan {
+  int a_is_dy, mt, nt, nbx, sets, tiles_m, tiles_n, stages, smem;
+  int64_t px, splits;
+  uint32_t cols;
+};
+wg_plan plan_wgrad(int64_t P, int N, int K) {
+  wg_plan w;
+  w.a_is_dy = N >= K;
+  const int na = w.a_is_dy ? N : K, nb = w.a_is_dy ? K : N;
+  const int t = (na + 127) / 128;
+  w.nt = nb >= 256 ? 256 : (nb + 15) / 16 * 16;
+  w.nbx = (w.nt + 63) / 64;
+  w.tiles_n = (nb + w.nt - 1) / w.nt;
+  const int most = w.nt > 128 ? 2 : (w.nt > 64 ? 3 : 4);  // <= 512 columns, 64-80 KB a stage
+  w.tiles_m = (t + most - 1) / most;
+  w.mt = (t + w.tiles_m - 1) / w.tiles_m;
+  w.sets = 256 / (w.mt * w.nt);
+  w.sets = w.sets < 1 ? 1 : (w.sets > 8 ? 8 : w.sets);
+  w.cols = 32;
+  while ((int)w.cols < w.sets * w.mt * w.nt) w.cols *= 2;
+  const int stage = (2 * w.mt + w.nbx) * WG_BOX;
+  const int room = w.cols <= 256 ? 100 * 1024 : 208 * 1024;  // two CTAs per SM, or one
+  w.stages = room / stage;
+  w.stages = w.stages < 2 ? 2 : (w.stages > WG_STAGES ? WG_STAGES : w.stages);
+  w.smem = w.stages * stage + 1024;
+  const int64_t tiles = (int64_t)w.tiles_m * w.tiles_n;
+  int64_t splits = ((w.cols <= 256 ? 304 : 152) + tiles - 1) / tiles;
+  const int64_t sums = pe_gemm_split(N, K, P);  // of the mma.sync kernel
+  if (splits * w.sets < sums) splits = (sums + w.sets - 1) / w.sets;
+  const int64_t most_splits = (P + 511) / 512;
+  if (splits > most_splits) splits = most_splits;
+  w.px = (P + splits - 1) / splits;
+  w.px = (w.px + WG_PX - 1) / WG_PX * WG_PX;
+  w.splits = (P + w.px - 1) / w.px;
+  return w;
+}
+
 }  // namespace
 
 bool pe_gemm_tc_eligible(const pe_gemm_args &g) {
@@ -857,6 +1165,59 @@ pe_status pe_gemm_tc(const pe_gemm_args &g, cudaStream_t s) {
   if (g.N <= 64) return launch_bn<64>(g, s);
   if (g.N <= 128) return launch_bn<128>(g, s);
   return launch_bn<256>(g, s);
+}
+
+bool pe_wgrad_tc_eligible(const void *dY, int64_t ldy, const void *X, int64_t ldx, int64_t P, int32_t N,
+                          int32_t K) {
+  auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  return ldy % 8 == 0 && ldx % 8 == 0 && al16(dY) && al16(X) && N >= 8 && K >= 8 && P >= 16 &&
+         P < (1ll << 31) - 4096 && encoder();
+}
+
+size_t pe_wgrad_tc_workspace(int64_t P, int32_t N, int32_t K) {
+  return (size_t)plan_wgrad(P, N, K).splits * ((size_t)N * K + N) * sizeof(float);
+}
+
+pe_status pe_wgrad_tc(const void *dY, int64_t ldy, const void *X, int64_t ldx, int64_t P, int32_t N,
+                      int32_t K, float *dW, float *db, float *part, cudaStream_t s) {
+  const wg_plan w = plan_wgrad(P, N, K);
+  CUtensorMap my, mx;
+  if (!make_map(&my, dY, P, N, ldy, WG_PX) || !make_map(&mx, X, P, K, ldx, WG_PX))
+    return PE_EUNSUPPORTED;
+  static bool attr = false;
+  if (!attr) {
+    PE_TRY_CUDA(cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     209 * 1024));
+    PE_TRY_CUDA(cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)cudaSharedmemCarveoutMaxShared));
+    attr = true;
+  }
+  wg_args g;
+  memset(&g, 0, sizeof(g));
+  g.N = N;
+  g.K = K;
+  g.mt = w.mt;
+  g.nt = w.nt;
+  g.nbx = w.nbx;
+  g.sets = w.sets;
+  g.tiles_n = w.tiles_n;
+  g.a_is_dy = w.a_is_dy;
+  g.P = P;
+  g.px_per_split = (int)w.px;
+  g.stages = w.stages;
+  g.part = part;
+  g.want_db = db != nullptr;
+  g.cols = w.cols;
+  g.wait_limit = g_wait_limit.load();
+  g.err = pe_err_word();
+  const dim3 grid((unsigned)w.splits, (unsigned)(w.tiles_m * w.tiles_n));
+  wgrad_tc_kernel<<<grid, WG_THREADS, w.smem, s>>>(w.a_is_dy ? my : mx, w.a_is_dy ? mx : my, g);
+  PE_TRY_LAUNCH("wgrad_tc_kernel");
+  const int64_t nw = (int64_t)N * K, n_all = nw + N;
+  wgrad_reduce_kernel<<<(unsigned)((n_all + 31) / 32), dim3(32, 8), 0, s>>>(part, (int)w.splits, nw,
+                                                                          n_all, dW, db);
+  PE_TRY_LAUNCH("wgrad_reduce_kernel");
+  return PE_OK;
 }
 
 extern "C" pe_status pe_nn_set_wait_limit(int64_t polls) {

@@ -84,8 +84,10 @@ class Ops:
             check(self.lib.pe_nn_transpose(_p(W), N, K, _p(Wt), self.s()), "pe_nn_transpose")
             self.gemm(P, K, N, dy, N, 1, Wt, 1, N, dx, ldd, Z=gelu_z, ldz=K,
                       dgelu=gelu_z is not None)
-        self.gemm(N, K, P, dy, 1, N, x, ldx, 1, dW, K)
-        self.colsum(dy, P, N, N, db)
+        nb = self.lib.pe_nn_linear_wgrad_workspace(P, N, K)
+        ws = self.ws(nb)
+        check(self.lib.pe_nn_linear_wgrad(_p(dy), N, _p(x), ldx, P, N, K, _p(dW), _p(db), _p(ws),
+                                          ws.numel(), self.s()), "pe_nn_linear_wgrad")
 
     def colsum(self, X, M, N, ld, out, accumulate=False):
         nb = self.lib.pe_nn_colsum_workspace(M, N)

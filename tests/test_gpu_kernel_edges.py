@@ -173,3 +173,34 @@ def test_layernorm(P, C):
     assert rel(mean, x.double().mean(1)) < 1e-5
     assert rel(dx, xd.grad) < BF_TOL
     assert rel(dg, gd.grad) < 1e-5 and rel(db, bd.grad) < 1e-5
+
+
+# ---- weight gradients -------------------------------------------------------------
+
+# pixels below a block, ragged blocks, one and many splits; widths below a box,
+# either operand the wider one, several accumulators, several tiles each way;
+# FP32 sums over P products err below 1e-5 of the result
+@pytest.mark.parametrize("N,K", [(8, 8), (32, 128), (128, 32), (64, 256), (136, 40), (128, 576),
+                                 (264, 520)])
+@pytest.mark.parametrize("P", [16, 63, 200, 70_001])
+def test_linear_weight_gradient(P, N, K):
+    from paper_2408_15583_gb300 import _lib, api
+    lib = _lib.load()
+    g = gen(P + N + K)
+    dy, x = rnd(g, P, N).to(BF), rnd(g, P, K + 8).to(BF)
+    dW, db = torch.full((N, K), 7.0, device=DEV), torch.full((N,), 7.0, device=DEV)
+    nb = lib.pe_nn_linear_wgrad_workspace(P, N, K)
+    ws = torch.empty(nb, dtype=torch.uint8, device=DEV)
+    ptr = lambda t: C.c_void_p(t.data_ptr())
+    stream = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    call = lambda: lib.pe_nn_linear_wgrad(ptr(dy), N, ptr(x), K + 8, P, N, K, ptr(dW), ptr(db),
+                                          ptr(ws), nb, stream)
+    try:                                # its bounded waits give up and say so
+        assert lib.pe_nn_set_wait_limit(0) == 0
+        assert call() == 0 and lib.pe_stream_check(stream) == 4
+    finally:
+        lib.pe_nn_set_wait_limit(-1)
+    assert call() == 0
+    api.stream_check()
+    assert rel(dW, dy.double().T @ x[:, :K].double()) < 1e-5
+    assert rel(db, dy.double().sum(0)) < 1e-5
