@@ -137,3 +137,6 @@ pe_status pe_wgrad_tc(const void *dY, int64_t ldy, const void *X, int64_t ldx, i
                       int32_t K, float *dW, float *db, float *part, cudaStream_t s);
 // Split-K factor of the mma.sync kernel.
 int64_t pe_gemm_split(int32_t M, int32_t N, int64_t K);
+// dW [nw], db [n_all - nw] (nullable) = sums of part[split][n_all] in split order.
+pe_status pe_wgrad_reduce(const float *part, int splits, int64_t nw, int64_t n_all, float *dW, float *db,
+                          cudaStream_t s);

@@ -317,16 +317,29 @@ __global__ void __launch_bounds__(TC_THREADS, 3)
 // CTAs per SM, whose tensor memory (2 x 128 columns each) fills the SM's 512.
 // ---------------------------------------------------------------------------
 constexpr int ST_THREADS = 320;  // producer, issuer, eight epilogue warps
-constexpr int ST_SLAB = 32 * 32 * 2;
 constexpr int ST_MAX_BIAS = 1024;  // columns whose bias is kept in shared memory
 
-template <int BN, int MODE>
+// GELU' of a BF16 pre-activation, for MODE 3: the kernel tabulates it for
+// 2^-11 <= |z| < 8 (two signs of 14 binades of 128 values, 15 KB of shared
+// memory per CTA, filled once by pe_gelu_grad itself) and computes the rest.
+// One shared-memory load in place of an erf and an exp per value, which had
+// bounded it: the data gradient of 64 -> 256 channels at 524288 pixels (603 MB, 89
+// us of copy bandwidth), 239 -> 143 us.  The negative half starts 2048 floats in,
+// a shift of the sign bit; rows with a value outside the table (found by packed
+// 16-bit minima and maxima) are recomputed value by value.
+constexpr uint32_t DG_LO = 116u << 7, DG_N = 14u * 128u, DG_NEG = 2048u;
+constexpr uint32_t DG_FLOATS = DG_NEG + DG_N + 1u;
+__device__ __noinline__ float dg_outside(float z) { return pe_gelu_grad(z); }
+
+template <int BN, int MODE, bool WIDE>
 struct st_cfg {
-  static constexpr int STAGES = BN == 128 ? 2 : 3;
+  static constexpr int STAGES = WIDE ? 1 : (BN == 128 ? 2 : 3);
   static constexpr int NB = (MODE == 1 && BN == 32) ? 3 : 2;  // staging slabs per warp
+  static constexpr int COLS = WIDE ? 64 : 32;                  // columns of a slab
+  static constexpr int SLAB = 32 * COLS * 2;
   static constexpr int A_BYTES = TC_BM * TC_BK * 2, B_BYTES = BN * TC_BK * 2;
   static constexpr int STAGE = A_BYTES + B_BYTES;
-  static constexpr int STAGING = 8 * NB * ST_SLAB;
+  static constexpr int STAGING = 8 * NB * SLAB;
   // barriers (an even number of 8-byte words, so that the bias after them and
   // the two words that follow is 16-byte aligned)
   static constexpr int BARS = (2 * STAGES + 4 + 8 * NB + 1 + 1) & ~1;
@@ -334,7 +347,8 @@ struct st_cfg {
                 "alignment of the slabs, the barriers and the bias");
   static constexpr uint32_t IDESC = tc_cfg<BN>::IDESC;
   static int smem(int bias_floats) {
-    return 1024 + STAGES * STAGE + STAGING + BARS * 8 + 16 + bias_floats * 4;
+    return 1024 + STAGES * STAGE + STAGING + BARS * 8 + 16 + bias_floats * 4 +
+           (MODE == 3 ? DG_FLOATS * 4 : 0);
   }
 };
 
@@ -405,14 +419,14 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-template <int BN, int MODE>
+template <int BN, int MODE, bool WIDE>
 __global__ void __launch_bounds__(ST_THREADS, 2)
     gemm_stream_kernel(const __grid_constant__ CUtensorMap tmA,
                        const __grid_constant__ CUtensorMap tmB,
                        const __grid_constant__ CUtensorMap tmC,
                        const __grid_constant__ CUtensorMap tmX, const st_args g) {
-  using cfg = st_cfg<BN, MODE>;
-  constexpr int S = cfg::STAGES, NB = cfg::NB, SLABS = BN / 32;
+  using cfg = st_cfg<BN, MODE, WIDE>;
+  constexpr int S = cfg::STAGES, NB = cfg::NB, CW = cfg::COLS, SLABS = BN / CW, SLAB = cfg::SLAB;
   constexpr bool XIN = MODE == 1 || MODE == 3;
   extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
   uint8_t *base = reinterpret_cast<uint8_t *>(
@@ -442,10 +456,16 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  if (g.bias) {
-    const int n_pad = (g.N + 31) & ~31;
+  const int n_pad = g.bias ? (g.N + 31) & ~31 : 0;
+  if (g.bias)
     for (int i = threadIdx.x; i < n_pad; i += ST_THREADS) s_bias[i] = i < g.N ? g.bias[i] : 0.0f;
-  }
+  float *s_dg = s_bias + n_pad;  // [DG_N], 1 for z > 0; from DG_NEG on for z < 0
+  if (MODE == 3)
+    for (uint32_t i = threadIdx.x; i < 2 * (DG_N + 1u); i += ST_THREADS) {
+      const uint32_t k = i % (DG_N + 1u), neg = i / (DG_N + 1u);
+      s_dg[k + neg * DG_NEG] =
+          k < DG_N ? pe_gelu_grad(__uint_as_float((DG_LO + k + neg * 0x8000u) << 16)) : 1.0f;
+    }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                      sm_u32(tmem_slot)),
@@ -521,10 +541,11 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
   } else {
     // ---- epilogue ----------------------------------------------------------
     const int ew = warp - 2, grp = ew >> 2, quad = warp & 3;
-    uint8_t *slabs = staging + ew * NB * ST_SLAB;
+    uint8_t *slabs = staging + ew * NB * SLAB;
     uint64_t *xb = xbar + ew * NB;
     // this lane's row in a slab: chunk q (16 bytes) at row + ((q ^ sw) << 4)
-    const uint32_t row = (uint32_t)lane * 64u, sw = ((uint32_t)lane >> 1) & 3u;
+    const uint32_t row = (uint32_t)lane * (CW * 2u);
+    const uint32_t sw = WIDE ? (uint32_t)lane & 7u : ((uint32_t)lane >> 1) & 3u;
     const uint32_t tlane = tmem + (uint32_t)(grp * BN) + ((uint32_t)(quad * 32) << 16);
     // a cursor over this warp's slabs: tiles of its parity, the slabs that
     // hold rows and columns of the matrix
@@ -533,7 +554,7 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
     };
     auto inside = [&](const cursor &k) {
       return (k.it / g.tiles_n) * TC_BM + quad * 32 < g.M &&
-             (k.it % g.tiles_n) * BN + k.j * 32 < g.N;
+             (k.it % g.tiles_n) * BN + k.j * CW < g.N;
     };
     auto step = [&](cursor &k) {
       do {
@@ -545,8 +566,8 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
     };
     auto load_x = [&](const cursor &k, uint32_t seq) {
       const uint32_t b = seq % NB;
-      mbar_expect_tx(xb + b, ST_SLAB);
-      tma_load_2d(slabs + b * ST_SLAB, &tmX, (k.it % g.tiles_n) * BN + k.j * 32,
+      mbar_expect_tx(xb + b, SLAB);
+      tma_load_2d(slabs + b * SLAB, &tmX, (k.it % g.tiles_n) * BN + k.j * CW,
                   (k.it / g.tiles_n) * TC_BM + quad * 32, xb + b);
     };
     const int first = (int)(blockIdx.x + grp * gridDim.x);
@@ -567,10 +588,10 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
       tc_fence_after();
 #pragma unroll 1
       for (int j = 0; j < SLABS; ++j) {
-        const int c0 = n0 + 32 * j;
+        const int c0 = n0 + CW * j;
         if (m0 >= g.M || c0 >= g.N) continue;
         const uint32_t b = seq % NB;
-        uint8_t *slab = slabs + b * ST_SLAB;
+        uint8_t *slab = slabs + b * SLAB;
         if (XIN) {
           // the slab read ahead: its buffer's last store has been read out
           if (ld.it < g.items) {
@@ -585,71 +606,103 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
           ok = __all_sync(0xffffffffu, ready);
           if (!ok) break;
         }
-        float v[32];
-        tc_ld32(tlane + (uint32_t)(32 * j), v);
+#pragma unroll 1
+        for (int h = 0; h < CW / 32; ++h) {  // 32 columns at a time
+          float v[32];
+          tc_ld32(tlane + (uint32_t)(CW * j + 32 * h), v);
+          if (g.alpha != 1.0f) {
 #pragma unroll
-        for (int e = 0; e < 32; ++e) v[e] = __fmul_rn(v[e], g.alpha);
-        if (g.bias) {
-          const float4 *bp = reinterpret_cast<const float4 *>(s_bias + c0);
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float4 t = bp[q];
-            v[4 * q] += t.x;
-            v[4 * q + 1] += t.y;
-            v[4 * q + 2] += t.z;
-            v[4 * q + 3] += t.w;
+            for (int e = 0; e < 32; ++e) v[e] = __fmul_rn(v[e], g.alpha);
           }
-        }
-        if (XIN) {
+          if (g.bias) {
+            const float4 *bp = reinterpret_cast<const float4 *>(s_bias + c0 + 32 * h);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint4 xv = *reinterpret_cast<const uint4 *>(slab + row + ((q ^ sw) << 4));
-            const bf162 *xp = reinterpret_cast<const bf162 *>(&xv);
+            for (int q = 0; q < 8; ++q) {
+              const float4 t = bp[q];
+              v[4 * q] += t.x;
+              v[4 * q + 1] += t.y;
+              v[4 * q + 2] += t.z;
+              v[4 * q + 3] += t.w;
+            }
+          }
+          if (MODE == 1) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float2 f = __bfloat1622float2(xp[e]);
-              if (MODE == 1) {
-                v[8 * q + 2 * e] += f.x;
-                v[8 * q + 2 * e + 1] += f.y;
-              } else {
-                v[8 * q + 2 * e] *= pe_gelu_grad(f.x);
-                v[8 * q + 2 * e + 1] *= pe_gelu_grad(f.y);
+            for (int q = 0; q < 4; ++q) {
+              const uint4 xv = *reinterpret_cast<const uint4 *>(slab + row + (((q + 4 * h) ^ sw) << 4));
+              const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                v[8 * q + 2 * e] += __uint_as_float(xw[e] << 16);
+                v[8 * q + 2 * e + 1] += __uint_as_float(xw[e] & 0xffff0000u);
               }
             }
           }
-        }
-        auto put = [&](uint8_t *dst) {
+          if (MODE == 3) {
+            uint32_t lo = 0xffffffffu, hi = 0u;  // of the row's |z|, as 16-bit pairs
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint4 o;
-            bf162 *op = reinterpret_cast<bf162 *>(&o);
+            for (int q = 0; q < 4; ++q) {
+              const uint4 xv = *reinterpret_cast<const uint4 *>(slab + row + (((q + 4 * h) ^ sw) << 4));
+              const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-              op[e] = __floats2bfloat162_rn(v[8 * q + 2 * e], v[8 * q + 2 * e + 1]);
-            *reinterpret_cast<uint4 *>(dst + row + ((q ^ sw) << 4)) = o;
+              for (int e = 0; e < 4; ++e) {
+                const uint32_t mag = xw[e] & 0x7fff7fffu;
+                lo = __vminu2(lo, mag);
+                hi = __vmaxu2(hi, mag);
+                const uint32_t k0 = min((mag & 0xffffu) - DG_LO, DG_N);
+                const uint32_t k1 = min((mag >> 16) - DG_LO, DG_N);
+                v[8 * q + 2 * e] *= s_dg[k0 + ((xw[e] >> 4) & DG_NEG)];
+                v[8 * q + 2 * e + 1] *= s_dg[k1 + ((xw[e] >> 20) & DG_NEG)];
+              }
+            }
+            const uint32_t least = min(lo & 0xffffu, lo >> 16), most = max(hi & 0xffffu, hi >> 16);
+            if (least < DG_LO || most >= DG_LO + DG_N) {
+              // (their factor so far is the entry 1 past the table's end)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const bf16 *zp = reinterpret_cast<const bf16 *>(slab + row + (((q + 4 * h) ^ sw) << 4));
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                  const float z = __bfloat162float(zp[e]);
+                  if (!(fabsf(z) >= 0.00048828125f && fabsf(z) < 8.0f)) v[8 * q + e] *= dg_outside(z);
+                }
+              }
+            }
           }
-        };
-        if (MODE == 2) {
-          // both slabs of the warp: the pre-activation, then the result
-          if (lane == 0) bulk_wait_read<0>();
-          __syncwarp();
-          put(slabs);
+          auto put = [&](uint8_t *dst) {
 #pragma unroll
-          for (int e = 0; e < 32; ++e) v[e] = pe_gelu(v[e]);
-          put(slabs + ST_SLAB);
-        } else {
-          if (!XIN) {
-            if (lane == 0) bulk_wait_read<NB - 1>();
-            __syncwarp();
+            for (int q = 0; q < 4; ++q) {
+              uint4 o;
+              bf162 *op = reinterpret_cast<bf162 *>(&o);
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                op[e] = __floats2bfloat162_rn(v[8 * q + 2 * e], v[8 * q + 2 * e + 1]);
+              *reinterpret_cast<uint4 *>(dst + row + (((q + 4 * h) ^ sw) << 4)) = o;
+            }
+          };
+          if (MODE == 2) {
+            // both slabs of the warp: the pre-activation, then the result
+            if (h == 0) {
+              if (lane == 0) bulk_wait_read<0>();
+              __syncwarp();
+            }
+            put(slabs);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] = pe_gelu(v[e]);
+            put(slabs + SLAB);
+          } else {
+            if (!XIN && h == 0) {
+              if (lane == 0) bulk_wait_read<NB - 1>();
+              __syncwarp();
+            }
+            put(slab);
           }
-          put(slab);
         }
         async_fence();
         __syncwarp();
         if (lane == 0) {
           if (MODE == 2) {
             tma_store_2d(&tmX, slabs, c0, m0);
-            tma_store_2d(&tmC, slabs + ST_SLAB, c0, m0);
+            tma_store_2d(&tmC, slabs + SLAB, c0, m0);
           } else {
             tma_store_2d(&tmC, slab, c0, m0);
           }
@@ -904,9 +957,16 @@ __global__ void __launch_bounds__(WG_THREADS)
           if (m >= na) continue;
           if (g.a_is_dy) {
             float *dst = out + (int64_t)m * g.K + n0 + c;
+            if (n0 + c + 16 <= nb && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
 #pragma unroll
-            for (int e = 0; e < 16; ++e)
-              if (n0 + c + e < nb) dst[e] = v[e];
+              for (int e = 0; e < 4; ++e)
+                reinterpret_cast<float4 *>(dst)[e] =
+                    make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 16; ++e)
+                if (n0 + c + e < nb) dst[e] = v[e];
+            }
           } else {  // transposed: consecutive lanes write consecutive k
             float *dst = out + (int64_t)(n0 + c) * g.K + m;
 #pragma unroll
@@ -1013,17 +1073,20 @@ pe_status launch_bn(const pe_gemm_args &g, cudaStream_t s) {
   return PE_OK;
 }
 
-// Row-major BF16 [rows][ld] in 32 x 32 slabs (64-byte rows, 64-byte swizzle),
-// for the streaming kernel's output rows and the rows its epilogue reads.
-bool make_slab_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld) {
+// Row-major BF16 [rows][ld] in slabs of 32 rows by 32 or 64 columns, swizzled
+// over their row's bytes, for the streaming kernel's output rows and the rows
+// its epilogue reads.
+bool make_slab_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld,
+                   int width) {
   encode_tiled_fn enc = encoder();
   if (!enc) return false;
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {32, 32};
+  cuuint32_t box[2] = {(cuuint32_t)width, 32};
   cuuint32_t estr[2] = {1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box,
-             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             width == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1038,24 +1101,25 @@ int tc_sms() {
   return n;
 }
 
-template <int BN, int MODE>
+template <int BN, int MODE, bool WIDE>
 pe_status launch_stream(const pe_gemm_args &g, cudaStream_t s) {
-  using cfg = st_cfg<BN, MODE>;
+  using cfg = st_cfg<BN, MODE, WIDE>;
   CUtensorMap ma, mb, mc, mx;
   const int64_t items = (int64_t)((g.M + TC_BM - 1) / TC_BM) * ((g.N + BN - 1) / BN);
   if (items >= (1ll << 30)) return PE_EUNSUPPORTED;  // (tile numbers are 32-bit)
   if (!make_map(&ma, g.A, g.M, g.K, g.sam, TC_BM) || !make_map(&mb, g.B, g.N, g.K, g.sbn, BN) ||
-      !make_slab_map(&mc, g.C, g.M, g.N, g.ldc))
+      !make_slab_map(&mc, g.C, g.M, g.N, g.ldc, cfg::COLS))
     return PE_EUNSUPPORTED;
   if (MODE == 0) mx = mc;
-  else if (!make_slab_map(&mx, MODE == 1 ? g.R : g.Z, g.M, g.N, MODE == 1 ? g.ldr : g.ldz))
+  else if (!make_slab_map(&mx, MODE == 1 ? g.R : g.Z, g.M, g.N, MODE == 1 ? g.ldr : g.ldz,
+                          cfg::COLS))
     return PE_EUNSUPPORTED;
   static bool attr = false;
   if (!attr) {
-    PE_TRY_CUDA(cudaFuncSetAttribute(gemm_stream_kernel<BN, MODE>,
+    PE_TRY_CUDA(cudaFuncSetAttribute(gemm_stream_kernel<BN, MODE, WIDE>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      cfg::smem(ST_MAX_BIAS)));
-    PE_TRY_CUDA(cudaFuncSetAttribute(gemm_stream_kernel<BN, MODE>,
+    PE_TRY_CUDA(cudaFuncSetAttribute(gemm_stream_kernel<BN, MODE, WIDE>,
                                      cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)cudaSharedmemCarveoutMaxShared));
     attr = true;
@@ -1072,7 +1136,7 @@ pe_status launch_stream(const pe_gemm_args &g, cudaStream_t s) {
   a.wait_limit = g_wait_limit.load();
   a.err = pe_err_word();
   const int most = 2 * tc_sms();  // two CTAs per SM
-  gemm_stream_kernel<BN, MODE><<<a.items < most ? a.items : most, ST_THREADS,
+  gemm_stream_kernel<BN, MODE, WIDE><<<a.items < most ? a.items : most, ST_THREADS,
                                  cfg::smem(g.bias ? (g.N + 31) / 32 * 32 : 0), s>>>(ma, mb, mc, mx,
                                                                                     a);
   PE_TRY_LAUNCH("gemm_stream_kernel");
@@ -1096,11 +1160,23 @@ int stream_mode(const pe_gemm_args &g) {
 template <int BN>
 pe_status launch_stream_mode(int mode, const pe_gemm_args &g, cudaStream_t s) {
   switch (mode) {
-    case 0: return launch_stream<BN, 0>(g, s);
-    case 1: return launch_stream<BN, 1>(g, s);
-    case 2: return launch_stream<BN, 2>(g, s);
-    default: return launch_stream<BN, 3>(g, s);
+    case 0: return launch_stream<BN, 0, false>(g, s);
+    case 1: return launch_stream<BN, 1, false>(g, s);
+    case 2: return launch_stream<BN, 2, false>(g, s);
+    default: return launch_stream<BN, 3, false>(g, s);
   }
+}
+
+// Column tile and slab width.  The GELU modes move two rows of N per row of K
+// (N = 4 K): their slabs take 64 columns, half the rows for the TMA unit, where
+// one operand block is the whole of K and so a single ring stage makes room (GELU'
+// form, 64 channels, 524288 pixels: 174 -> 161 us before the packed range test).
+pe_status launch_stream_shape(int mode, const pe_gemm_args &g, cudaStream_t s) {
+  if (g.N > 64 && g.K <= TC_BK && mode == 2) return launch_stream<128, 2, true>(g, s);
+  if (g.N > 64 && g.K <= TC_BK && mode == 3) return launch_stream<128, 3, true>(g, s);
+  if (g.N <= 32) return launch_stream_mode<32>(mode, g, s);
+  if (g.N <= 64) return launch_stream_mode<64>(mode, g, s);
+  return launch_stream_mode<128>(mode, g, s);
 }
 
 // Tile and split of a weight gradient.  The wider operand gives the rows; its
@@ -1156,15 +1232,21 @@ bool pe_gemm_tc_eligible(const pe_gemm_args &g) {
 pe_status pe_gemm_tc(const pe_gemm_args &g, cudaStream_t s) {
   const int mode = stream_mode(g);
   if (mode >= 0) {
-    const pe_status st = g.N <= 32   ? launch_stream_mode<32>(mode, g, s)
-                         : g.N <= 64 ? launch_stream_mode<64>(mode, g, s)
-                                     : launch_stream_mode<128>(mode, g, s);
+    const pe_status st = launch_stream_shape(mode, g, s);
     if (st != PE_EUNSUPPORTED) return st;
   }
   if (g.N <= 32) return launch_bn<32>(g, s);
   if (g.N <= 64) return launch_bn<64>(g, s);
   if (g.N <= 128) return launch_bn<128>(g, s);
   return launch_bn<256>(g, s);
+}
+
+pe_status pe_wgrad_reduce(const float *part, int splits, int64_t nw, int64_t n_all, float *dW, float *db,
+                          cudaStream_t s) {
+  wgrad_reduce_kernel<<<(unsigned)((n_all + 31) / 32), dim3(32, 8), 0, s>>>(part, splits, nw, n_all,
+                                                                          dW, db);
+  PE_TRY_LAUNCH("wgrad_reduce_kernel");
+  return PE_OK;
 }
 
 bool pe_wgrad_tc_eligible(const void *dY, int64_t ldy, const void *X, int64_t ldx, int64_t P, int32_t N,
@@ -1213,11 +1295,7 @@ pe_status pe_wgrad_tc(const void *dY, int64_t ldy, const void *X, int64_t ldx, i
   const dim3 grid((unsigned)w.splits, (unsigned)(w.tiles_m * w.tiles_n));
   wgrad_tc_kernel<<<grid, WG_THREADS, w.smem, s>>>(w.a_is_dy ? my : mx, w.a_is_dy ? mx : my, g);
   PE_TRY_LAUNCH("wgrad_tc_kernel");
-  const int64_t nw = (int64_t)N * K, n_all = nw + N;
-  wgrad_reduce_kernel<<<(unsigned)((n_all + 31) / 32), dim3(32, 8), 0, s>>>(part, (int)w.splits, nw,
-                                                                          n_all, dW, db);
-  PE_TRY_LAUNCH("wgrad_reduce_kernel");
-  return PE_OK;
+  return pe_wgrad_reduce(part, (int)w.splits, (int64_t)N * K, (int64_t)N * K + N, dW, db, s);
 }
 
 extern "C" pe_status pe_nn_set_wait_limit(int64_t polls) {
