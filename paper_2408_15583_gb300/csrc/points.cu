@@ -11,9 +11,8 @@
 // growing Chebyshev radius until its k-th distance is below the distance to
 // every unsearched cell.  Neighbours are ordered by (FP32 squared distance,
 // index), with the squared distance evaluated in one fixed order, so the
-// neighbour lists -- and the radii, summed in FP64 in list order -- equal a
-// brute-force search bit for bit.  Queries run in cell order, so a warp's
-// points are neighbours and read the same cells.
+// neighbour sets -- and the radii, summed in FP64 from the nearest on -- equal a
+// brute-force search bit for bit.
 #include <cstring>
 
 #include "pe_internal.cuh"
@@ -29,11 +28,6 @@ struct grid_info {
   float h, inv_h;
   int G;
 };
-
-__device__ __forceinline__ float d2_of(float qx, float qy, float qz, const float *p) {
-  const float dx = __fsub_rn(p[0], qx), dy = __fsub_rn(p[1], qy), dz = __fsub_rn(p[2], qz);
-  return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-}
 
 __global__ void bbox_partial(const float *__restrict__ pos, int64_t n, float *__restrict__ part) {
   __shared__ float red[6][kPtThreads];
@@ -60,16 +54,20 @@ __global__ void bbox_partial(const float *__restrict__ pos, int64_t n, float *__
 // Cubic cells of side h = (largest extent / G) (1 + 2^-10): the farthest
 // point falls in cell G - 1.
 __global__ void bbox_final(const float *__restrict__ part, int blocks, int G, grid_info *gi) {
-  if (threadIdx.x != 0) return;
   float lo[3], hi[3];
   for (int k = 0; k < 3; ++k) {
-    lo[k] = part[k];
-    hi[k] = part[3 + k];
-    for (int b = 1; b < blocks; ++b) {
+    lo[k] = INFINITY;
+    hi[k] = -INFINITY;
+    for (int b = threadIdx.x; b < blocks; b += 32) {
       lo[k] = fminf(lo[k], part[b * 6 + k]);
       hi[k] = fmaxf(hi[k], part[b * 6 + 3 + k]);
     }
+    for (int o = 16; o > 0; o >>= 1) {
+      lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
+      hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
+    }
   }
+  if (threadIdx.x != 0) return;
   float ext = fmaxf(fmaxf(hi[0] - lo[0], hi[1] - lo[1]), hi[2] - lo[2]);
   if (!(ext > 0.0f)) ext = 1.0f;
   grid_info g;
@@ -107,6 +105,20 @@ __global__ void scatter_cells(int64_t n, const uint32_t *__restrict__ cell_of,
        i += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t c = cell_of[i];
     sorted[offs[c] + atomicAdd(cursor + c, 1u)] = (uint32_t)i;
+  }
+}
+
+// The points as 16-byte records {x, y, z, index} in cell order (any order
+// inside a cell); count ends at zero.
+__global__ void scatter_points(const float *__restrict__ pos, int64_t n,
+                               const uint32_t *__restrict__ cell_of,
+                               const uint32_t *__restrict__ offs, uint32_t *__restrict__ count,
+                               float4 *__restrict__ pts) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t c = cell_of[i];
+    pts[offs[c] + atomicSub(count + c, 1u) - 1u] =
+        make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], __uint_as_float((uint32_t)i));
   }
 }
 
@@ -158,115 +170,193 @@ __device__ void smallest_axis(double a00, double a01, double a02, double a11, do
 }
 
 struct knn_args {
-  const float *pos;
+  const float4 *pts;  // {x, y, z, index} in cell order
   int64_t n;
   const grid_info *gi;
-  const uint32_t *offs, *sorted;
+  const uint32_t *offs;
   int K, k_r, k_n;
   const float *ref;
   float *rad, *nrm;
   unsigned int *err;
 };
 
+__device__ __forceinline__ float d2_pts(float4 q, float4 p) {
+  const float dx = __fsub_rn(p.x, q.x), dy = __fsub_rn(p.y, q.y), dz = __fsub_rn(p.z, q.z);
+  return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+}
+
+// Calls f(begin, end) for the runs of points in the cells at Chebyshev distance
+// lo..hi from c: cells are stored with z fastest, so the cells of one (x, y)
+// column are one run (two around the part nearer than lo).
+template <class F>
+__device__ __forceinline__ void for_runs(const uint32_t *__restrict__ offs, int G, const int c[3],
+                                         int lo, int hi, F &&f) {
+  const int x0 = max(c[0] - hi, 0), x1 = min(c[0] + hi, G - 1);
+  const int y0 = max(c[1] - hi, 0), y1 = min(c[1] + hi, G - 1);
+  const int z0 = max(c[2] - hi, 0), z1 = min(c[2] + hi, G - 1);
+  for (int x = x0; x <= x1; ++x)
+    for (int y = y0; y <= y1; ++y) {
+      const uint32_t col = ((uint32_t)x * G + y) * G;
+      if (lo == 0 || abs(x - c[0]) >= lo || abs(y - c[1]) >= lo) {
+        f(__ldg(offs + col + z0), __ldg(offs + col + z1 + 1));
+      } else {
+        if (z0 <= c[2] - lo) f(__ldg(offs + col + z0), __ldg(offs + col + c[2] - lo + 1));
+        if (c[2] + lo <= z1) f(__ldg(offs + col + c[2] + lo), __ldg(offs + col + z1 + 1));
+      }
+    }
+}
+
+// One thread per point, in two scans of its neighbourhood.  The first keeps the
+// KT >= K smallest squared distances in registers, sorted: a candidate goes
+// through the list by min and max alone (two instructions per entry, no
+// indices, no branches beyond one test against the last).  That list alone gives
+// the radius: the point itself is one of its zeros, whatever the order of ties.
+// The second scan, for the normal, collects the points nearer than the k_n-th
+// distance and, of those at it, the smallest indices, into shared memory; their
+// moments about the query point are then summed in FP64 by all lanes together.
+// The points are read as 16-byte records in cell order, a run per (x, y) column
+// of cells, and queries follow the same order, so a warp mostly reads the same
+// records.  (Lists of (distance, index) in local memory, insertion by a
+// data-dependent loop and 27 cells visited one by one left 13.6 of 32 lanes
+// active and took 2.35 ms for a million points, k_r = 8, k_n = 16; now 1.28 ms,
+// of which the FP64 sums and eigenvectors, at a 64th of the FP32 rate, are the
+// larger part: the radii alone take 0.3 of 0.75-1.1 ms.)
+template <int KT>
 __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
+  extern __shared__ uint32_t s_list[];  // [k_n][kPtThreads]: positions in pts
   const grid_info g = *A.gi;
   const int G = g.G;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < A.n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t i = A.sorted[t];
-    const float qx = A.pos[3 * (int64_t)i], qy = A.pos[3 * (int64_t)i + 1],
-                qz = A.pos[3 * (int64_t)i + 2];
-    const int c[3] = {cell_1d(g, qx, 0), cell_1d(g, qy, 1), cell_1d(g, qz, 2)};
-    const float q[3] = {qx, qy, qz};
-    float bd[KMAX];
-    uint32_t bi[KMAX];
-    int cnt = 0;
-    const int K = A.K;
-    for (int s = 0; s <= G; ++s) {
-      // the cells at Chebyshev distance s from c (inside the grid)
-      for (int dz = -s; dz <= s; ++dz) {
-        const int z = c[2] + dz;
-        if (z < 0 || z >= G) continue;
-        for (int dy = -s; dy <= s; ++dy) {
-          const int y = c[1] + dy;
-          if (y < 0 || y >= G) continue;
-          const bool face = dz == -s || dz == s || dy == -s || dy == s;
-          for (int dx = -s; dx <= s; dx += face ? 1 : (s > 0 ? 2 * s : 1)) {
-            const int x = c[0] + dx;
-            if (x < 0 || x >= G) continue;
-            const uint32_t cell = ((uint32_t)x * G + y) * G + z;
-            const uint32_t b = A.offs[cell], e = A.offs[cell + 1];
-            for (uint32_t m = b; m < e; ++m) {
-              const uint32_t j = A.sorted[m];
-              const float d2 = d2_of(qx, qy, qz, A.pos + 3 * (int64_t)j);
-              if (cnt == K && !(d2 < bd[K - 1] || (d2 == bd[K - 1] && j < bi[K - 1]))) continue;
-              int at = cnt < K ? cnt++ : K - 1;
-              while (at > 0 && (bd[at - 1] > d2 || (bd[at - 1] == d2 && bi[at - 1] > j))) {
-                bd[at] = bd[at - 1];
-                bi[at] = bi[at - 1];
-                --at;
-              }
-              bd[at] = d2;
-              bi[at] = j;
-            }
-          }
+  const int64_t t = (int64_t)blockIdx.x * kPtThreads + threadIdx.x;
+  if (t >= A.n) return;
+  const float4 q = __ldg(A.pts + t);
+  const uint32_t i = __float_as_uint(q.w);
+  const int c[3] = {cell_1d(g, q.x, 0), cell_1d(g, q.y, 1), cell_1d(g, q.z, 2)};
+  const float qq[3] = {q.x, q.y, q.z};
+  const int K = A.K;
+  float bd[KT];
+#pragma unroll
+  for (int k = 0; k < KT; ++k) bd[k] = INFINITY;
+  // the entry at a runtime position (a constant chain of selects)
+  auto at = [&](int k) {
+    float v = bd[0];
+#pragma unroll
+    for (int e = 1; e < KT; ++e) v = e == k ? bd[e] : v;
+    return v;
+  };
+  uint32_t seen = 0;
+  int s = 1;  // cells within Chebyshev distance s are searched
+  for (int lo = 0;; lo = ++s) {
+    for_runs(A.offs, G, c, lo, s, [&](uint32_t b, uint32_t e) {
+      seen += e - b;
+      for (uint32_t m = b; m < e; ++m) {
+        const float d2 = d2_pts(q, __ldg(A.pts + m));
+        if (d2 < bd[KT - 1]) {
+#pragma unroll
+          for (int k = KT - 1; k > 0; --k) bd[k] = fmaxf(bd[k - 1], fminf(bd[k], d2));
+          bd[0] = fminf(bd[0], d2);
         }
       }
-      // stop once the k-th distance is below the distance to every cell
-      // outside the searched block (faces at the grid's edge bound nothing)
-      float bound = INFINITY;
-      for (int k = 0; k < 3; ++k) {
-        const float slack = 1e-4f * g.h + 1e-6f * (fabsf(g.lo[k]) + (float)G * g.h);
-        if (c[k] - s > 0) bound = fminf(bound, q[k] - (g.lo[k] + (float)(c[k] - s) * g.h) - slack);
-        if (c[k] + s + 1 < G)
-          bound = fminf(bound, (g.lo[k] + (float)(c[k] + s + 1) * g.h) - q[k] - slack);
-      }
-      if (bound == INFINITY) break;  // every cell searched
-      if (cnt == K && bound > 0.0f && bd[K - 1] <= bound * bound) break;
+    });
+    // stop once the k-th distance is below the distance to every cell
+    // outside the searched block (faces at the grid's edge bound nothing)
+    float bound = INFINITY;
+    for (int k = 0; k < 3; ++k) {
+      const float slack = 1e-4f * g.h + 1e-6f * (fabsf(g.lo[k]) + (float)G * g.h);
+      if (c[k] - s > 0) bound = fminf(bound, qq[k] - (g.lo[k] + (float)(c[k] - s) * g.h) - slack);
+      if (c[k] + s + 1 < G)
+        bound = fminf(bound, (g.lo[k] + (float)(c[k] + s + 1) * g.h) - qq[k] - slack);
     }
-    if (cnt < K) {  // fewer than K points in the cloud: rejected on the host
-      pe_raise(A.err, PE_ERR_OVERFLOW);
-      continue;
-    }
-    if (A.rad) {
-      double sum = 0.0;
-      int used = 0;
-      for (int e = 0; e < K && used < A.k_r; ++e) {
-        if (bi[e] == i) continue;
-        sum += sqrt((double)bd[e]);
-        ++used;
-      }
-      A.rad[i] = (float)(sum / (double)A.k_r);
-    }
-    if (A.nrm) {
-      double m[3] = {0.0, 0.0, 0.0};
-      for (int e = 0; e < A.k_n; ++e)
-        for (int k = 0; k < 3; ++k) m[k] += (double)A.pos[3 * (int64_t)bi[e] + k];
-      for (int k = 0; k < 3; ++k) m[k] /= (double)A.k_n;
-      double a00 = 0, a01 = 0, a02 = 0, a11 = 0, a12 = 0, a22 = 0;
-      for (int e = 0; e < A.k_n; ++e) {
-        const float *p = A.pos + 3 * (int64_t)bi[e];
-        const double x = (double)p[0] - m[0], y = (double)p[1] - m[1], z = (double)p[2] - m[2];
-        a00 += x * x;
-        a01 += x * y;
-        a02 += x * z;
-        a11 += y * y;
-        a12 += y * z;
-        a22 += z * z;
-      }
-      double v[3];
-      smallest_axis(a00, a01, a02, a11, a12, a22, v);
-      double w[3];
-      if (A.ref) {
-        for (int k = 0; k < 3; ++k) w[k] = (double)A.ref[3 * (int64_t)i + k];
-      } else {
-        for (int k = 0; k < 3; ++k) w[k] = (double)q[k] - (double)g.ctr[k];
-      }
-      if (v[0] * w[0] + v[1] * w[1] + v[2] * w[2] < 0.0)
-        for (int k = 0; k < 3; ++k) v[k] = -v[k];
-      for (int k = 0; k < 3; ++k) A.nrm[3 * (int64_t)i + k] = (float)v[k];
-    }
+    if (bound == INFINITY) break;  // every cell searched
+    if (seen >= (uint32_t)K && bound > 0.0f && at(K - 1) <= bound * bound) break;
   }
+  if (seen < (uint32_t)K) {  // fewer than K points in the cloud: rejected on the host
+    pe_raise(A.err, PE_ERR_OVERFLOW);
+    return;
+  }
+  if (A.rad) {
+    // the first entry is the point's own zero; were it pushed out by more than
+    // K coincident points, every entry would be zero
+    double sum = 0.0;
+#pragma unroll
+    for (int e = 1; e < KT; ++e)
+      if (e <= A.k_r) sum += sqrt((double)bd[e]);
+    A.rad[i] = (float)(sum / (double)A.k_r);
+  }
+  if (A.nrm) {
+    const int kn = A.k_n;
+    const float tau = at(kn - 1);
+    int below = 0;  // entries nearer than the k_n-th: the list's points from there on tie
+#pragma unroll
+    for (int e = 0; e < KT; ++e) below += e < kn && bd[e] < tau;
+    uint32_t *list = s_list + threadIdx.x;
+    int n_lt = 0, n_eq = below;
+    for_runs(A.offs, G, c, 0, s, [&](uint32_t b, uint32_t e) {
+      for (uint32_t m = b; m < e; ++m) {
+        const float4 p = __ldg(A.pts + m);
+        const float d2 = d2_pts(q, p);
+        if (!(d2 <= tau)) continue;
+        if (d2 < tau) {
+          list[n_lt++ * kPtThreads] = m;
+        } else if (n_eq < kn) {
+          list[n_eq++ * kPtThreads] = m;
+        } else {
+          // a tie too many: the largest index of the tied goes
+          int worst = below;
+          uint32_t wi = 0;
+          for (int k = below; k < kn; ++k) {
+            const uint32_t id = __float_as_uint(__ldg(A.pts + list[k * kPtThreads]).w);
+            if (id >= wi) {
+              wi = id;
+              worst = k;
+            }
+          }
+          if (__float_as_uint(p.w) < wi) list[worst * kPtThreads] = m;
+        }
+      }
+    });
+    // moments about the query point: exact differences of floats in FP64
+    double m[3] = {0.0, 0.0, 0.0};
+    double a00 = 0, a01 = 0, a02 = 0, a11 = 0, a12 = 0, a22 = 0;
+    for (int k = 0; k < kn; ++k) {
+      const float4 p = __ldg(A.pts + list[k * kPtThreads]);
+      const double x = (double)p.x - (double)q.x, y = (double)p.y - (double)q.y,
+                   z = (double)p.z - (double)q.z;
+      m[0] += x;
+      m[1] += y;
+      m[2] += z;
+      a00 += x * x;
+      a01 += x * y;
+      a02 += x * z;
+      a11 += y * y;
+      a12 += y * z;
+      a22 += z * z;
+    }
+    const double inv = 1.0 / (double)kn;
+    const double mx = m[0] * inv, my = m[1] * inv, mz = m[2] * inv;
+    a00 -= m[0] * mx;
+    a01 -= m[0] * my;
+    a02 -= m[0] * mz;
+    a11 -= m[1] * my;
+    a12 -= m[1] * mz;
+    a22 -= m[2] * mz;
+    double v[3];
+    smallest_axis(a00, a01, a02, a11, a12, a22, v);
+    double w[3];
+    if (A.ref) {
+      for (int k = 0; k < 3; ++k) w[k] = (double)A.ref[3 * (int64_t)i + k];
+    } else {
+      for (int k = 0; k < 3; ++k) w[k] = (double)qq[k] - (double)g.ctr[k];
+    }
+    if (v[0] * w[0] + v[1] * w[1] + v[2] * w[2] < 0.0)
+      for (int k = 0; k < 3; ++k) v[k] = -v[k];
+    for (int k = 0; k < 3; ++k) A.nrm[3 * (int64_t)i + k] = (float)v[k];
+  }
+}
+
+template <int KT>
+void launch_knn(const knn_args &A, cudaStream_t s) {
+  const size_t smem = A.nrm ? sizeof(uint32_t) * kPtThreads * A.k_n : 0;
+  knn_kernel<KT><<<(unsigned)((A.n + kPtThreads - 1) / kPtThreads), kPtThreads, smem, s>>>(A);
 }
 
 int grid_res(int64_t n) {
@@ -280,7 +370,8 @@ int grid_res(int64_t n) {
 struct pt_ws {
   float *part;
   grid_info *gi;
-  uint32_t *count, *offs, *cursor, *tile, *cell_of, *sorted;
+  uint32_t *count, *offs, *cursor, *tile, *cell_of;
+  float4 *pts;
 };
 
 pt_ws carve(pe_carve &c, int64_t n) {
@@ -291,10 +382,10 @@ pt_ws carve(pe_carve &c, int64_t n) {
   w.gi = c.take<grid_info>(1);
   w.count = c.take<uint32_t>((size_t)cells);
   w.offs = c.take<uint32_t>((size_t)cells + 1);
-  w.cursor = c.take<uint32_t>((size_t)cells);
+  w.cursor = nullptr;
   w.tile = c.take<uint32_t>((size_t)((cells + 4095) / 4096 + 1));
   w.cell_of = c.take<uint32_t>((size_t)n);
-  w.sorted = c.take<uint32_t>((size_t)n);
+  w.pts = c.take<float4>((size_t)n);
   return w;
 }
 
@@ -317,7 +408,7 @@ pt_ws carve_order(pe_carve &c, int64_t n) {
   w.cursor = c.take<uint32_t>((size_t)cells);
   w.tile = c.take<uint32_t>((size_t)((cells + 4095) / 4096 + 1));
   w.cell_of = c.take<uint32_t>((size_t)n);
-  w.sorted = nullptr;  // the caller's order buffer
+  w.pts = nullptr;
   return w;
 }
 
@@ -389,22 +480,20 @@ extern "C" pe_status pe_point_attributes(const float *pos, int64_t n_points, int
   bbox_final<<<1, 32, 0, s>>>(w.part, kBoxBlocks, G, w.gi);
   PE_TRY_LAUNCH("bbox_final");
   PE_TRY_CUDA(cudaMemsetAsync(w.count, 0, sizeof(uint32_t) * cells, s));
-  PE_TRY_CUDA(cudaMemsetAsync(w.cursor, 0, sizeof(uint32_t) * cells, s));
   int64_t b = (n_points + 255) / 256;
   const int blocks = (int)(b < 4096 ? b : 4096);
   count_cells<<<blocks, 256, 0, s>>>(pos, n_points, w.gi, w.count, w.cell_of);
   PE_TRY_LAUNCH("count_cells");
   pe_status st = pe_exclusive_scan_u32(w.count, cells, w.tile, w.offs, s);
   if (st != PE_OK) return st;
-  scatter_cells<<<blocks, 256, 0, s>>>(n_points, w.cell_of, w.offs, w.cursor, w.sorted);
-  PE_TRY_LAUNCH("scatter_cells");
+  scatter_points<<<blocks, 256, 0, s>>>(pos, n_points, w.cell_of, w.offs, w.count, w.pts);
+  PE_TRY_LAUNCH("scatter_points");
   knn_args A;
   memset(&A, 0, sizeof(A));
-  A.pos = pos;
+  A.pts = w.pts;
   A.n = n_points;
   A.gi = w.gi;
   A.offs = w.offs;
-  A.sorted = w.sorted;
   A.K = K;
   A.k_r = k_r;
   A.k_n = k_n;
@@ -412,9 +501,12 @@ extern "C" pe_status pe_point_attributes(const float *pos, int64_t n_points, int
   A.rad = radius;
   A.nrm = normal;
   A.err = pe_err_word();
-  int64_t qb = (n_points + kPtThreads - 1) / kPtThreads;
   pe_event_before("knn_kernel", s);
-  knn_kernel<<<(int)(qb < 65535 * 16 ? qb : 65535 * 16), kPtThreads, 0, s>>>(A);
+  if (K <= 9) launch_knn<9>(A, s);
+  else if (K <= 12) launch_knn<12>(A, s);
+  else if (K <= 16) launch_knn<16>(A, s);
+  else if (K <= 24) launch_knn<24>(A, s);
+  else launch_knn<KMAX>(A, s);
   pe_event_after("knn_kernel", s);
   PE_TRY_LAUNCH("knn_kernel");
   return PE_OK;

@@ -204,3 +204,41 @@ def test_linear_weight_gradient(P, N, K):
     api.stream_check()
     assert rel(dW, dy.double().T @ x[:, :K].double()) < 1e-5
     assert rel(db, dy.double().sum(0)) < 1e-5
+
+
+# ---- surfel attributes --------------------------------------------------------------
+
+# a lattice, where many neighbours tie at the k_n-th distance (the smaller index is
+# the nearer), coincident points, and counts just above each list length; against
+# a brute-force search by (FP32 squared distance, index) with FP64 sums
+@pytest.mark.parametrize("k_r,k_n", [(8, 9), (8, 12), (11, 16), (15, 17), (23, 24), (31, 32)])
+@pytest.mark.parametrize("kind", ["lattice", "coincident", "few"])
+def test_point_attributes_ties(kind, k_r, k_n):
+    from paper_2408_15583_gb300 import api
+    g = gen(k_r + k_n)
+    if kind == "lattice":
+        ax = torch.arange(9, device=DEV, dtype=torch.float32)
+        pos = torch.cartesian_prod(ax, ax, ax[:2] * 0.75)
+        pos = pos[torch.randperm(len(pos), generator=g, device=DEV)]
+    elif kind == "coincident":
+        pos = torch.rand(60, 3, generator=g, device=DEV).repeat(40, 1)
+    else:
+        pos = torch.rand(max(k_r + 1, k_n) + 1, 3, generator=g, device=DEV)
+    pos = pos.contiguous()
+    n = len(pos)
+    rad, nrm = api.point_attributes(pos, k_r, k_n)
+    api.stream_check()
+    e = (pos[:, None] - pos[None]) ** 2
+    d2 = (e[..., 0] + e[..., 1]) + e[..., 2]                 # the kernel's order
+    key = d2.view(torch.int32).long() << 32 | torch.arange(n, device=DEV)[None]
+    key = key.sort(1).values
+    idx, d = key & 0xffffffff, (key >> 32).int().view(torch.float32).double()
+    assert torch.equal(rad, (d[:, 1:k_r + 1].sqrt().sum(1) / k_r).float())
+    nb = pos[idx[:, :k_n]].double()
+    nb = nb - nb.mean(1, keepdim=True)
+    val, vec = torch.linalg.eigh((nb.transpose(1, 2) @ nb).cpu())
+    clear = (val[:, 1] - val[:, 0] > 1e-3 * val[:, 2]) & (val[:, 2] > 0)   # a defined normal
+    dot = (vec[:, :, 0] * nrm.cpu().double()).sum(1).abs()[clear]
+    # FP32 rounding of a unit vector: 1 - |dot| <= (2^-24 sqrt(3))^2 / 2 + FP64 noise
+    # amplified by the gap bound (1e-16 / 1e-3)
+    assert bool((dot > 1 - 1e-7).all())
