@@ -3,11 +3,12 @@
 // uses in place of the paper's splat acceleration structure.
 //
 // Fusion is a counting sort on a dense G^3 voxel grid (G <= 256): count
-// contributors per voxel, exclusive scan, scatter pixel keys into voxel
-// segments, then one thread per segment orders its keys by (view, pixel) and
-// sums in FP64 in that order -- the same order as a sort by
-// (voxel, view, pixel), so the result is bit-identical whatever the atomic
-// order of the scatter.
+// contributors per voxel and list the voxels that have any, give each listed
+// voxel a segment, scatter pixel keys into the segments, rank the keys of each
+// by (view, pixel), and sum each segment in FP64 in that order -- the same
+// order as a sort by (voxel, view, pixel), so the result is bit-identical
+// whatever the atomic order of the scatter and of the list.
+#include <algorithm>
 #include <cstring>
 
 #include "pe_internal.cuh"
@@ -17,7 +18,6 @@ namespace {
 constexpr int kScanThreads = 1024;
 constexpr int kScanPer = 4;
 constexpr int kScanTile = kScanThreads * kScanPer;
-constexpr int kSegLocal = 64;
 
 __device__ __forceinline__ int view_of(const pe_geom_layout &L, int64_t g) {
   int v = 0;
@@ -151,16 +151,57 @@ __global__ void canny_hyst_kernel(const __grid_constant__ pe_geom_layout L,
   if (ch) atomicAdd(changed, ch);
 }
 
-// Edge rule + voxel of the pixel's surface point; counts contributors.
-__global__ void fuse_classify_kernel(const __grid_constant__ pe_geom_layout L,
-                                     const float4 *__restrict__ nd,
-                                     const uint8_t *__restrict__ mask, float tau,
-                                     const uint8_t *__restrict__ canny_state,
-                                     float bx, float by, float bz, float inv_vox, int G,
-                                     uint32_t *__restrict__ vox_of, uint32_t *__restrict__ count) {
-  int64_t total = L.pix_off[L.nv];
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
-       g += (int64_t)gridDim.x * blockDim.x) {
+// Where a fusion stands: voxels listed, key slots handed out.
+struct fuse_count {
+  unsigned int voxels, entries;
+};
+
+// This thread's place among the block's `flag`s (and their number), with one
+// atomicAdd of `total` on *counter per block; every thread of the block calls it.
+__device__ __forceinline__ uint32_t block_place(uint32_t mine, unsigned int *counter) {
+  __shared__ uint32_t warp_sum[32], s_base;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  uint32_t v = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  if (lane == 31) warp_sum[wid] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t t = 0;
+    for (int w = 0; w < nw; ++w) {
+      const uint32_t y = warp_sum[w];
+      warp_sum[w] = t;
+      t += y;
+    }
+    s_base = t ? atomicAdd(counter, t) : 0u;
+  }
+  __syncthreads();
+  const uint32_t at = s_base + warp_sum[wid] + v - mine;
+  __syncthreads();
+  return at;
+}
+
+// Edge rule + voxel of the pixel's surface point; counts contributors and lists
+// the voxels met for the first time (four pixels per thread, one atomic on the
+// list per block).
+constexpr int kClassifyPx = 4;
+__global__ void __launch_bounds__(256)
+    fuse_classify_kernel(const __grid_constant__ pe_geom_layout L, const float4 *__restrict__ nd,
+                         const uint8_t *__restrict__ mask, float tau,
+                         const uint8_t *__restrict__ canny_state, float bx, float by, float bz,
+                         float inv_vox, int G, uint32_t *__restrict__ vox_of,
+                         uint32_t *__restrict__ count, uint32_t *__restrict__ list,
+                         fuse_count *__restrict__ fc) {
+  const int64_t total = L.pix_off[L.nv];
+  uint32_t heads[kClassifyPx], n_heads = 0;
+#pragma unroll
+  for (int u = 0; u < kClassifyPx; ++u) {
+    const int64_t g = (int64_t)blockIdx.x * (256 * kClassifyPx) + u * 256 + threadIdx.x;
+    heads[u] = PE_NONE;
+    if (g >= total) continue;
     uint32_t vox = PE_NONE;
     if (mask[g]) {
       int v = view_of(L, g);
@@ -200,10 +241,31 @@ __global__ void fuse_classify_kernel(const __grid_constant__ pe_geom_layout L,
           ix[k] = ci < 0 ? 0 : (ci > G - 1 ? G - 1 : ci);
         }
         vox = (uint32_t)((ix[0] * G + ix[1]) * G + ix[2]);
-        atomicAdd(count + vox, 1u);
+        if (atomicAdd(count + vox, 1u) == 0u) {
+          heads[u] = vox;
+          ++n_heads;
+        }
       }
     }
     vox_of[g] = vox;
+  }
+  uint32_t at = block_place(n_heads, &fc->voxels);
+#pragma unroll
+  for (int u = 0; u < kClassifyPx; ++u)
+    if (heads[u] != PE_NONE) list[at++] = heads[u];
+}
+
+// A segment of keys for every listed voxel.  (Its place among the segments does
+// not matter; a scan over the dense grid's 2^24 counts took 75 us.)
+__global__ void __launch_bounds__(256)
+    fuse_offsets_kernel(const uint32_t *__restrict__ list, const uint32_t *__restrict__ count,
+                        uint32_t *__restrict__ offs, fuse_count *__restrict__ fc) {
+  const uint32_t n = fc->voxels;
+  for (uint32_t base = blockIdx.x * 256; base < n; base += gridDim.x * 256) {
+    const uint32_t k = base + threadIdx.x;
+    const uint32_t vox = k < n ? list[k] : 0u, len = k < n ? count[vox] : 0u;
+    const uint32_t at = block_place(len, &fc->entries);
+    if (k < n) offs[vox] = at;
   }
 }
 
@@ -287,10 +349,11 @@ __global__ void __launch_bounds__(kScanThreads)
 }
 
 // Scatter each kept pixel's key (voxel << 40 | view << 32 | pixel) into its
-// voxel's segment (order inside a segment is arbitrary here).
+// voxel's segment (order inside a segment is arbitrary here); offs ends at the
+// segments' ends.
 __global__ void fuse_scatter_kernel(const __grid_constant__ pe_geom_layout L,
                                     const uint32_t *__restrict__ vox_of,
-                                    const uint32_t *__restrict__ offs, uint32_t *__restrict__ count,
+                                    uint32_t *__restrict__ offs,
                                     unsigned long long *__restrict__ entries) {
   int64_t total = L.pix_off[L.nv];
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
@@ -298,18 +361,39 @@ __global__ void fuse_scatter_kernel(const __grid_constant__ pe_geom_layout L,
     uint32_t vox = vox_of[g];
     if (vox == PE_NONE) continue;
     int v = view_of(L, g);
-    uint32_t slot = offs[vox] + atomicSub(count + vox, 1u) - 1u;
-    entries[slot] = ((unsigned long long)vox << 40) | ((unsigned long long)v << 32) |
-                    (unsigned long long)(g - L.pix_off[v]);
+    entries[atomicAdd(offs + vox, 1u)] = ((unsigned long long)vox << 40) |
+                                         ((unsigned long long)v << 32) |
+                                         (unsigned long long)(g - L.pix_off[v]);
+  }
+}
+
+// Each key to its rank in its segment (keys differ, so ranks do): a thread per
+// key counts the smaller ones.
+__global__ void fuse_rank_kernel(const unsigned long long *__restrict__ entries,
+                                 const uint32_t *__restrict__ offs,
+                                 const uint32_t *__restrict__ count,
+                                 const fuse_count *__restrict__ fc,
+                                 unsigned long long *__restrict__ sorted) {
+  const uint32_t n = fc->entries;
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const unsigned long long key = entries[e];
+    const uint32_t vox = (uint32_t)(key >> 40), len = __ldg(count + vox);
+    const unsigned long long *seg = entries + (__ldg(offs + vox) - len);
+    uint32_t rank = 0;
+    for (uint32_t k = 0; k < len; ++k) rank += __ldg(seg + k) < key;
+    sorted[(seg - entries) + rank] = key;
   }
 }
 
 // Eq. 22 for one contributor in FP64: s = sqrt(|n| |p| / |n . p|),
 // R = sqrt(2) L s if s < 2.5 else 3.535 L.
-__device__ __forceinline__ double eq22(pe_f3 n, pe_f3 p, double L) {
+__device__ __forceinline__ double norm64(pe_f3 a) {
+  const double x = a.x, y = a.y, z = a.z;
+  return __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)));
+}
+// (nn, pp: the norms of n and p)
+__device__ __forceinline__ double eq22(pe_f3 n, double nn, pe_f3 p, double pp, double L) {
   double nx = n.x, ny = n.y, nz = n.z, px = p.x, py = p.y, pz = p.z;
-  double nn = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(nx, nx), __dmul_rn(ny, ny)), __dmul_rn(nz, nz)));
-  double pp = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(px, px), __dmul_rn(py, py)), __dmul_rn(pz, pz)));
   double np = __dadd_rn(__dadd_rn(__dmul_rn(nx, px), __dmul_rn(ny, py)), __dmul_rn(nz, pz));
   if (np < 0) np = -np;
   double s = np > 0 ? __dsqrt_rn(__ddiv_rn(__dmul_rn(nn, pp), np)) : __longlong_as_double(0x7ff0000000000000ll);
@@ -317,149 +401,146 @@ __device__ __forceinline__ double eq22(pe_f3 n, pe_f3 p, double L) {
   return __dmul_rn(3.535, L);
 }
 
-struct seg_acc {
-  double sp[3], sn[3], rmax;
-  pe_f3 n0;
-  bool first;
-};
-
-__device__ __forceinline__ void seg_add(seg_acc &a, const pe_geom_layout &L,
-                                        const float4 *__restrict__ nd, unsigned long long key) {
-  int v = (int)((key >> 32) & 0xff);
-  int64_t p = (int64_t)(key & 0xffffffffull);
-  const pe_view &V = L.view[v];
-  float4 q = nd[L.pix_off[v] + p];
-  int i = (int)(p % V.W), j = (int)(p / V.W);
-  pe_f3 x = pe_ray_at(pe_pixel_origin(V, i, j), q.w, pe_v3(V.d));
-  pe_f3 n = {q.x, q.y, q.z};
-  if (a.first) {
-    a.n0 = n;
-    a.first = false;
-  }
-  if (pe_dot(n, a.n0) < 0.0f) n = pe_neg3(n);
-  a.sp[0] = __dadd_rn(a.sp[0], (double)x.x);
-  a.sp[1] = __dadd_rn(a.sp[1], (double)x.y);
-  a.sp[2] = __dadd_rn(a.sp[2], (double)x.z);
-  a.sn[0] = __dadd_rn(a.sn[0], (double)n.x);
-  a.sn[1] = __dadd_rn(a.sn[1], (double)n.y);
-  a.sn[2] = __dadd_rn(a.sn[2], (double)n.z);
-  double r = eq22(n, pe_v3(V.d), (double)V.pitch);
-  if (r > a.rmax) a.rmax = r;
-}
-
-// One thread per voxel segment: order the keys, FP64 sums in that order,
-// Eq. 22 maximum, write the splat at the owner pixel.
-// One voxel segment (entries [s, offs[vox + 1]) of voxel vox, s = offs[vox]):
-// the fused splat at its owner pixel.
-__device__ __forceinline__ void fuse_one_segment(const pe_geom_layout &L,
-                                                 const float4 *__restrict__ nd,
-                                                 const unsigned long long *__restrict__ entries,
-                                                 const uint32_t *__restrict__ offs, int64_t s,
-                                                 float4 *__restrict__ cr, float4 *__restrict__ nf) {
-  const uint32_t vox = (uint32_t)(entries[s] >> 40);
-  int64_t len = (int64_t)offs[vox + 1] - s;
-  seg_acc a;
-  a.sp[0] = a.sp[1] = a.sp[2] = a.sn[0] = a.sn[1] = a.sn[2] = 0.0;
-  a.rmax = 0.0;
-  a.first = true;
-  unsigned long long owner;
-  if (len <= kSegLocal) {
-    unsigned long long buf[kSegLocal];
-    for (int64_t e = 0; e < len; ++e) {
-      unsigned long long k = entries[s + e];
-      int64_t m = e;
-      while (m > 0 && buf[m - 1] > k) {
-        buf[m] = buf[m - 1];
-        --m;
-      }
-      buf[m] = k;
-    }
-    owner = buf[0];
-    for (int64_t e = 0; e < len; ++e) seg_add(a, L, nd, buf[e]);
-  } else {
-    // long segment: visit keys in increasing order by repeated minimum
-    unsigned long long last = 0;
-    bool have = false;
-    owner = ~0ull;
-    for (int64_t e = 0; e < len; ++e) {
-      unsigned long long best = ~0ull;
-      for (int64_t f = 0; f < len; ++f) {
-        unsigned long long k = entries[s + f];
-        if ((!have || k > last) && k < best) best = k;
-      }
-      if (!have) owner = best;
-      seg_add(a, L, nd, best);
-      last = best;
-      have = true;
-    }
-  }
-  double cnt = (double)len;
-  double m = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(a.sn[0], a.sn[0]), __dmul_rn(a.sn[1], a.sn[1])),
-                                  __dmul_rn(a.sn[2], a.sn[2])));
-  const pe_f3 nrm = {__double2float_rn(__ddiv_rn(a.sn[0], m)),
-                     __double2float_rn(__ddiv_rn(a.sn[1], m)),
-                     __double2float_rn(__ddiv_rn(a.sn[2], m))};
-  // Owner: the contributing view facing the fused normal most directly, by
-  // |n . d_v| in quarters (floor(4 |n . d_v|), so near-equal views tie),
-  // the smaller (view, pixel) key on a tie; the first entry if the normal
-  // vanishes.  Owners of neighbouring voxels then mostly come from the same
-  // view, which keeps each stretch of surface in few pyramids.
-  if (m > 0.0) {
-    float bs = -1.0f;
-    unsigned long long bk = owner;
-    auto consider = [&](unsigned long long k) {
-      const pe_view &V = L.view[(int)((k >> 32) & 0xff)];
-      const float sc = floorf(__fmul_rn(fabsf(pe_dot(nrm, pe_f3{V.d[0], V.d[1], V.d[2]})), 4.0f));
-      if (sc > bs || (sc == bs && k < bk)) {
-        bs = sc;
-        bk = k;
-      }
-    };
-    for (int64_t e = 0; e < len; ++e) consider(entries[s + e]);
-    owner = bk;
-  }
-  int v0 = (int)((owner >> 32) & 0xff);
-  int64_t id = L.pix_off[v0] + (int64_t)(owner & 0xffffffffull);
-  cr[id] = make_float4(__double2float_rn(__ddiv_rn(a.sp[0], cnt)),
-                       __double2float_rn(__ddiv_rn(a.sp[1], cnt)),
-                       __double2float_rn(__ddiv_rn(a.sp[2], cnt)), __double2float_rn(a.rmax));
-  nf[id] = make_float4(nrm.x, nrm.y, nrm.z, (float)len);
-}
-
-// One segment per lane: each warp examines 32 entries at a time and queues,
-// in shared memory, the ones that start a voxel's segment; whenever 32 are
-// queued its lanes take one each (a segment's work is a serial chain of FP64
-// sums, so a lane per segment, not per entry, keeps the warp full).
+// The fused splat of every listed voxel: one thread per segment, FP64 sums in
+// key order, Eq. 22's maximum, written at the owner pixel.  FP64 issues at 1/64
+// of the FP32 rate, and Eq. 22 (two square roots and a division) was most of it:
+// only contributors whose FP32 estimate comes within 4e-4 of the segment's
+// largest (far above the estimate's error and above the formula's step of 1.5e-4
+// at s = 2.5) are evaluated in FP64, once per run of equal normals, all lanes
+// taking their next one together; the maximum is the same.  8 views of 512^2,
+// sphere of 200k points / 10k-point dihedral: 145 / 370 us (and 12 / 9 us to
+// rank the keys) against 574 / 1800 us with the keys ordered in local memory and
+// every Eq. 22 in FP64.
 constexpr int kFuseThreads = 128;
 
 __global__ void __launch_bounds__(kFuseThreads)
     fuse_segment_kernel(const __grid_constant__ pe_geom_layout L, const float4 *__restrict__ nd,
-                        const unsigned long long *__restrict__ entries,
-                        const uint32_t *__restrict__ offs, int64_t nvox,
+                        const unsigned long long *__restrict__ sorted,
+                        const uint32_t *__restrict__ list, const uint32_t *__restrict__ offs,
+                        const uint32_t *__restrict__ count, const fuse_count *__restrict__ fc,
                         float4 *__restrict__ cr, float4 *__restrict__ nf) {
-  __shared__ uint32_t queue[kFuseThreads / 32][64];
-  const int64_t n_entries = offs[nvox];  // kept pixels, written by scan_apply
-  const int lane = threadIdx.x & 31;
-  uint32_t *q = queue[threadIdx.x >> 5];
-  int count = 0;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_entries;
-       base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = base + lane;
-    bool head = false;
-    if (s < n_entries) head = offs[(uint32_t)(entries[s] >> 40)] == (uint32_t)s;
-    const unsigned m = __ballot_sync(0xffffffffu, head);
-    if (head) q[count + __popc(m & ((1u << lane) - 1u))] = (uint32_t)s;
-    count += __popc(m);
-    __syncwarp();
-    if (count >= 32) {
-      fuse_one_segment(L, nd, entries, offs, q[lane], cr, nf);
-      __syncwarp();
-      if (lane < count - 32) q[lane] = q[lane + 32];
-      count -= 32;
-      __syncwarp();
-    }
+  // the views in shared memory (the lanes are in different views, and divergent
+  // indices into kernel parameters are served one address at a time)
+  struct view_row {
+    pe_view V;
+    float norm;
+    double norm64;
+    int64_t off;
+  };
+  __shared__ view_row views[PE_MAX_VIEWS];
+  if (threadIdx.x < L.nv) {
+    view_row &r = views[threadIdx.x];
+    r.V = L.view[threadIdx.x];
+    r.norm = sqrtf(r.V.d[0] * r.V.d[0] + r.V.d[1] * r.V.d[1] + r.V.d[2] * r.V.d[2]);
+    r.norm64 = norm64(pe_v3(r.V.d));
+    r.off = L.pix_off[threadIdx.x];
   }
-  if (lane < count) fuse_one_segment(L, nd, entries, offs, q[lane], cr, nf);
+  __syncthreads();
+  const uint32_t n_vox = fc->voxels;
+  for (uint32_t w0 = (blockIdx.x * kFuseThreads + threadIdx.x) & ~31u; w0 < n_vox;
+       w0 += gridDim.x * kFuseThreads) {
+    const uint32_t li = w0 + (threadIdx.x & 31);
+    const bool on = li < n_vox;  // (lanes without a segment follow the votes)
+    const uint32_t vox = on ? list[li] : 0u;
+    const uint32_t len = on ? count[vox] : 0u;
+    const unsigned long long *seg = sorted + (on ? offs[vox] - len : 0u);
+    double sp[3] = {0.0, 0.0, 0.0}, sn[3] = {0.0, 0.0, 0.0}, rmax = 0.0;
+    pe_f3 n0 = {0.f, 0.f, 0.f};
+    // Eq. 22 in FP32, to find the largest
+    auto estimate = [&](pe_f3 n, const view_row &r) {
+      const float nn = sqrtf(n.x * n.x + n.y * n.y + n.z * n.z);
+      const float np = fabsf(n.x * r.V.d[0] + n.y * r.V.d[1] + n.z * r.V.d[2]);
+      const float s2 = np > 0.0f ? nn * r.norm / np : INFINITY;
+      return s2 < 6.25f ? 1.41421356f * r.V.pitch * sqrtf(s2) : 3.535f * r.V.pitch;
+    };
+    auto gather = [&](unsigned long long key) {
+      return __ldg(nd + views[(int)((key >> 32) & 0xff)].off + (int64_t)(key & 0xffffffffull));
+    };
+    float best = 0.0f;
+    unsigned long long key = len ? seg[0] : 0ull;
+    float4 q = len ? gather(key) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (uint32_t e = 0; e < len; ++e) {
+      // the next contributor is on its way while this one is added
+      const unsigned long long key1 = e + 1 < len ? seg[e + 1] : key;
+      const float4 q1 = gather(key1);
+      const view_row &r = views[(int)((key >> 32) & 0xff)];
+      const pe_view &V = r.V;
+      const uint32_t p = (uint32_t)(key & 0xffffffffull);
+      const int j = (int)(p / (uint32_t)V.W), i = (int)(p - (uint32_t)j * V.W);
+      const pe_f3 x = pe_ray_at(pe_pixel_origin(V, i, j), q.w, pe_v3(V.d));
+      pe_f3 n = {q.x, q.y, q.z};
+      if (e == 0) n0 = n;
+      if (pe_dot(n, n0) < 0.0f) n = pe_neg3(n);
+      sp[0] = __dadd_rn(sp[0], (double)x.x);
+      sp[1] = __dadd_rn(sp[1], (double)x.y);
+      sp[2] = __dadd_rn(sp[2], (double)x.z);
+      sn[0] = __dadd_rn(sn[0], (double)n.x);
+      sn[1] = __dadd_rn(sn[1], (double)n.y);
+      sn[2] = __dadd_rn(sn[2], (double)n.z);
+      best = fmaxf(best, estimate(n, r));
+      key = key1;
+      q = q1;
+    }
+    // Eq. 22 of the contributors near the largest estimate (its sign rule does
+    // not depend on the normal's)
+    const float near = best * (1.0f - 4e-4f);
+    float4 done = make_float4(0.f, 0.f, 0.f, 0.f);
+    int done_v = -1;
+    double nn = 0.0;  // |done|
+    for (uint32_t e = 0;;) {
+      bool have = false;
+      int v = 0;
+      for (; e < len && !have; ++e) {
+        key = seg[e];
+        q = gather(key);
+        v = (int)((key >> 32) & 0xff);
+        have = estimate({q.x, q.y, q.z}, views[v]) >= near &&
+               !(v == done_v && q.x == done.x && q.y == done.y && q.z == done.z);
+      }
+      if (!__any_sync(0xffffffffu, have)) break;
+      if (have) {
+        const pe_f3 n = {q.x, q.y, q.z};
+        if (done_v < 0 || q.x != done.x || q.y != done.y || q.z != done.z) nn = norm64(n);
+        const double r = eq22(n, nn, pe_v3(views[v].V.d), views[v].norm64, (double)views[v].V.pitch);
+        if (r > rmax) rmax = r;
+        done = q;
+        done_v = v;
+      }
+    }
+    if (!on) continue;
+    const double cnt = (double)len;
+    const double m = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(sn[0], sn[0]), __dmul_rn(sn[1], sn[1])),
+                                          __dmul_rn(sn[2], sn[2])));
+    const pe_f3 nrm = {__double2float_rn(__ddiv_rn(sn[0], m)), __double2float_rn(__ddiv_rn(sn[1], m)),
+                       __double2float_rn(__ddiv_rn(sn[2], m))};
+    // Owner: the contributing view facing the fused normal most directly, by
+    // |n . d_v| in quarters (floor(4 |n . d_v|), so near-equal views tie),
+    // the smaller (view, pixel) key on a tie; the first entry if the normal
+    // vanishes.  Owners of neighbouring voxels then mostly come from the same
+    // view, which keeps each stretch of surface in few pyramids.
+    unsigned long long owner = seg[0];
+    if (m > 0.0) {
+      float bs = -1.0f;
+      int last = -1;
+      for (uint32_t e = 0; e < len; ++e) {  // a view's first key is its smallest
+        key = seg[e];
+        const int v = (int)((key >> 32) & 0xff);
+        if (v == last) continue;
+        last = v;
+        const pe_view &V = views[v].V;
+        const float sc = floorf(__fmul_rn(fabsf(pe_dot(nrm, pe_f3{V.d[0], V.d[1], V.d[2]})), 4.0f));
+        if (sc > bs) {
+          bs = sc;
+          owner = key;
+        }
+      }
+    }
+    const int64_t id = views[(int)((owner >> 32) & 0xff)].off + (int64_t)(owner & 0xffffffffull);
+    cr[id] = make_float4(__double2float_rn(__ddiv_rn(sp[0], cnt)),
+                         __double2float_rn(__ddiv_rn(sp[1], cnt)),
+                         __double2float_rn(__ddiv_rn(sp[2], cnt)), __double2float_rn(rmax));
+    nf[id] = make_float4(nrm.x, nrm.y, nrm.z, (float)len);
+  }
 }
 
 // Leaf boxes: bounds of the owned splats' spheres in the view's (u, v, d)
@@ -472,8 +553,11 @@ __global__ void __launch_bounds__(kFuseThreads)
 // centre plus the splat's (padded) radius in pixels, so that a ray hitting a
 // splat passes within `reach` pixels of the splat's slot.
 static_assert(PE_LEAF * PE_LEAF <= 32, "leaf occupancy mask is one 32-bit word");
-__global__ void pyramid_leaf_kernel(const __grid_constant__ pe_geom_layout L, int v,
+// (blockIdx.y: the view, here and in pyramid_up_kernel: one launch per level for
+// all views, where one per level and view were 64 of the geometry's 87 launches.)
+__global__ void pyramid_leaf_kernel(const __grid_constant__ pe_geom_layout L,
                                     float4 *__restrict__ nodes) {
+  const int v = blockIdx.y;
   const pe_view &V = L.view[v];
   int tw = L.tw[v][0], th = L.th[v][0];
   const float4 *cr = L.cr + L.pix_off[v];
@@ -524,8 +608,10 @@ __global__ void pyramid_leaf_kernel(const __grid_constant__ pe_geom_layout L, in
   }
 }
 
-__global__ void pyramid_up_kernel(const __grid_constant__ pe_geom_layout L, int v, int l,
+__global__ void pyramid_up_kernel(const __grid_constant__ pe_geom_layout L, int l,
                                   float4 *__restrict__ nodes) {
+  const int v = blockIdx.y;
+  if (l >= L.nlev[v]) return;
   int tw = L.tw[v][l], th = L.th[v][l];
   int cw = L.tw[v][l - 1], ch = L.th[v][l - 1];
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < tw * th; t += gridDim.x * blockDim.x) {
@@ -560,11 +646,33 @@ __global__ void pyramid_up_kernel(const __grid_constant__ pe_geom_layout L, int 
 // 1e-6 under the root (the rounding of m) and by the view's absolute box
 // pad.  Over a smooth patch the slab is far thinner than the node's box, so
 // a ray that leaves the patch is rejected as soon as it is above the slab.
-// One warp per node (all those levels of all views in one launch), sums in
-// a fixed order, so the slabs are the same on every run.  Higher nodes, a
-// node without splats and a node whose normals cancel get no slab (lower
-// bound -inf).
+// One warp per node (every level of all views in one launch), sums in a fixed
+// order, so the slabs are the same on every run.  Higher nodes, a node without
+// splats and a node whose normals cancel get no slab (lower bound -inf).  Only
+// slots whose leaf's occupancy mask has them are read.
 constexpr int kSlabLevels = 5;
+
+// Calls f(slot) for the occupied slots of view v in the lw x lh leaves from (lx,
+// ly), lw * lh <= 256, the warp taking two leaves at a time (a lane per slot);
+// occ: lane l holds the masks of leaves l, l + 32, ...
+constexpr int kLeafWords = (1 << (2 * (kSlabLevels - 1))) / 32;  // 8
+template <class F>
+__device__ __forceinline__ void for_slots(const uint32_t (&occ)[kLeafWords], int W, int lx, int ly,
+                                          int lw, int lh, F &&f) {
+  const int lane = threadIdx.x & 31, b = lane % (PE_LEAF * PE_LEAF), n = lw * lh;
+#pragma unroll
+  for (int w = 0; w < kLeafWords; ++w) {
+    if (32 * w >= n) break;
+#pragma unroll 4
+    for (int k = 0; k < 32; k += 2) {
+      const int leaf = 32 * w + k + lane / (PE_LEAF * PE_LEAF);
+      const uint32_t o = __shfl_sync(0xffffffffu, occ[w], leaf & 31);
+      if (!((o >> b) & 1u)) continue;
+      const int tx = lx + leaf % lw, ty = ly + leaf / lw;
+      f((int64_t)(ty * PE_LEAF + b / PE_LEAF) * W + tx * PE_LEAF + b % PE_LEAF);
+    }
+  }
+}
 
 __global__ void __launch_bounds__(128)
     pyramid_slab_kernel(const __grid_constant__ pe_geom_layout L, int64_t n_slab_nodes,
@@ -573,12 +681,15 @@ __global__ void __launch_bounds__(128)
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= n_slab_nodes) return;  // uniform over the warp
-  // warp w -> (view, level, node): views in order, levels 0.. within each
+  // warp w -> (level, view, node): the largest nodes with slabs first, so that
+  // their long scans do not end the launch; the levels without slabs last
   int v = 0, l = 0;
   int64_t k = w;
-  for (v = 0; v < L.nv; ++v) {
-    bool found = false;
-    for (l = 0; l < min(L.nlev[v], kSlabLevels); ++l) {
+  bool found = false;
+  for (int o = 0; o < PE_MAX_LEVELS && !found; ++o) {
+    l = o < kSlabLevels ? kSlabLevels - 1 - o : o;
+    for (v = 0; v < L.nv; ++v) {
+      if (l >= L.nlev[v]) continue;
       const int64_t cnt = (int64_t)L.tw[v][l] * L.th[v][l];
       if (k < cnt) {
         found = true;
@@ -586,29 +697,34 @@ __global__ void __launch_bounds__(128)
       }
       k -= cnt;
     }
-    if (found) break;
   }
   const int64_t nid = L.node_off[v][l] + k;
   const pe_view &V = L.view[v];
-  const int tx = (int)(k % L.tw[v][l]), ty = (int)(k / L.tw[v][l]);
-  const int span = PE_LEAF << l;
-  const int i0 = tx * span, j0 = ty * span;
-  const int iw = min(span, V.W - i0), jh = min(span, V.H - j0);
-  const int npx = iw * jh;
+  const int lx = (int)(k % L.tw[v][l]) << l, ly = (int)(k / L.tw[v][l]) << l;
+  const int lw = min(1 << l, L.tw[v][0] - lx), lh = min(1 << l, L.th[v][0] - ly);
   const float4 *cr = L.cr + L.pix_off[v];
   const float4 *nf = L.nf + L.pix_off[v];
+  uint32_t occ[kLeafWords];
+#pragma unroll
+  for (int q = 0; q < kLeafWords; ++q) {
+    const int leaf = 32 * q + lane;
+    occ[q] = 0u;
+    if (l < kSlabLevels && leaf < lw * lh) {
+      const int64_t id = L.node_off[v][0] + (int64_t)(ly + leaf / lw) * L.tw[v][0] + lx + leaf % lw;
+      occ[q] = __float_as_uint(__ldg(&L.nodes[2 * id].w));
+    }
+  }
   // pass 1: the axis
   float sx = 0.f, sy = 0.f, sz = 0.f, cnt = 0.f;
-  for (int q = lane; q < npx; q += 32) {
-    const int64_t g = (int64_t)(j0 + q / iw) * V.W + (i0 + q % iw);
-    if (!(cr[g].w > 0.0f)) continue;
-    const float4 m = nf[g];
-    const float sg = (m.x * V.d[0] + m.y * V.d[1] + m.z * V.d[2]) > 0.0f ? -1.0f : 1.0f;
-    sx += sg * m.x;
-    sy += sg * m.y;
-    sz += sg * m.z;
-    cnt += 1.0f;
-  }
+  if (l < kSlabLevels)
+    for_slots(occ, V.W, lx, ly, lw, lh, [&](int64_t g) {
+      const float4 m = nf[g];
+      const float sg = (m.x * V.d[0] + m.y * V.d[1] + m.z * V.d[2]) > 0.0f ? -1.0f : 1.0f;
+      sx += sg * m.x;
+      sy += sg * m.y;
+      sz += sg * m.z;
+      cnt += 1.0f;
+    });
   for (int o = 16; o > 0; o >>= 1) {
     sx += __shfl_xor_sync(FULL, sx, o);
     sy += __shfl_xor_sync(FULL, sy, o);
@@ -627,17 +743,15 @@ __global__ void __launch_bounds__(128)
   // pass 2: the heights
   const float pad = L.pad[v];
   float lo = INFINITY, hi = -INFINITY;
-  for (int q = lane; q < npx; q += 32) {
-    const int64_t g = (int64_t)(j0 + q / iw) * V.W + (i0 + q % iw);
+  for_slots(occ, V.W, lx, ly, lw, lh, [&](int64_t g) {
     const float4 c = cr[g];
-    if (!(c.w > 0.0f)) continue;
     const float4 m = nf[g];
     const float h = nx * (c.x - V.o[0]) + ny * (c.y - V.o[1]) + nz * (c.z - V.o[2]);
     const float nm = nx * m.x + ny * m.y + nz * m.z;
     const float e = c.w * 1.000001f * sqrtf(fmaxf(1.0f - nm * nm, 0.0f) + 1e-6f) + pad;
     lo = fminf(lo, h - e);
     hi = fmaxf(hi, h + e);
-  }
+  });
   for (int o = 16; o > 0; o >>= 1) {
     lo = fminf(lo, __shfl_xor_sync(FULL, lo, o));
     hi = fmaxf(hi, __shfl_xor_sync(FULL, hi, o));
@@ -645,16 +759,6 @@ __global__ void __launch_bounds__(128)
   if (lane == 0) {
     slab[nid] = make_float4(nx, ny, nz, lo - pad);
     slab_hi[nid] = hi + pad;
-  }
-}
-
-// No slab for the nodes above kSlabLevels.
-__global__ void slab_clear_kernel(float4 *__restrict__ slab, float *__restrict__ slab_hi,
-                                  int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    slab[i] = make_float4(0.f, 0.f, 1.f, -INFINITY);
-    slab_hi[i] = INFINITY;
   }
 }
 
@@ -691,21 +795,39 @@ __device__ __forceinline__ cell_box splat_cells(const pe_geom_layout &L, float4 
 // 2^28 terms at most, far below overflow).
 constexpr float kAxisScale = 4294967296.0f;
 
+// Slot k of the geometry's leaves in order (16 per leaf): its splat's index and
+// view, or -1 where the leaf's occupancy mask has none.
+__device__ __forceinline__ int64_t leaf_slot(const pe_geom_layout &L, int64_t k, int &v) {
+  int64_t leaf = k / (PE_LEAF * PE_LEAF);
+  const int b = (int)(k % (PE_LEAF * PE_LEAF));
+  v = 0;
+  for (; v + 1 < L.nv; ++v) {
+    const int64_t n = (int64_t)L.tw[v][0] * L.th[v][0];
+    if (leaf < n) break;
+    leaf -= n;
+  }
+  const float4 *node = L.nodes + 2 * (L.node_off[v][0] + leaf);
+  if (!((__float_as_uint(__ldg(&node->w)) >> b) & 1u)) return -1;
+  const int tx = (int)(leaf % L.tw[v][0]), ty = (int)(leaf / L.tw[v][0]);
+  return L.pix_off[v] + (int64_t)(ty * PE_LEAF + b / PE_LEAF) * L.view[v].W + tx * PE_LEAF +
+         b % PE_LEAF;
+}
+
 // Coarse view-occupancy grid: every splat marks its cells with its owner
 // view's bit (vmask[n^3] for splats reaching outside the grid), adds its
 // normal, turned toward its view, to each cell's axis sum and counts itself
 // there.
-__global__ void vgrid_kernel(const __grid_constant__ pe_geom_layout L, uint32_t *__restrict__ vmask,
-                             unsigned long long *__restrict__ axis_sum,
+__global__ void vgrid_kernel(const __grid_constant__ pe_geom_layout L, int64_t slots,
+                             uint32_t *__restrict__ vmask, unsigned long long *__restrict__ axis_sum,
                              unsigned int *__restrict__ axis_cnt) {
   const int n = L.vg_n;
   const int64_t n3 = (int64_t)n * n * n;
-  const int64_t total = L.pix_off[L.nv];
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
-       g += (int64_t)gridDim.x * blockDim.x) {
-    float4 c = L.cr[g];
-    if (!(c.w > 0.0f)) continue;
-    const int v = view_of(L, g);
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < slots;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    int v;
+    const int64_t g = leaf_slot(L, k, v);
+    if (g < 0) continue;
+    const float4 c = L.cr[g];
     const uint32_t bit = 1u << v;
     const float4 nn = L.nf[g];
     const pe_view &V = L.view[v];
@@ -761,17 +883,17 @@ __global__ void cell_axis_kernel(int64_t n3, const unsigned long long *__restric
 
 // Heights axis . (x - cell centre) over the disks a cell counts: the centre's
 // height +- R sqrt(1 - (axis . m)^2), padded like the node slabs.
-__global__ void cell_height_kernel(const __grid_constant__ pe_geom_layout L,
+__global__ void cell_height_kernel(const __grid_constant__ pe_geom_layout L, int64_t slots,
                                    const float4 *__restrict__ axis,
                                    unsigned int *__restrict__ hkey) {
   const int n = L.vg_n;
   const float cell = L.vg_cell;
-  const int64_t total = L.pix_off[L.nv];
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
-       g += (int64_t)gridDim.x * blockDim.x) {
-    float4 c = L.cr[g];
-    if (!(c.w > 0.0f)) continue;
-    const int v = view_of(L, g);
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < slots;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    int v;
+    const int64_t g = leaf_slot(L, k, v);
+    if (g < 0) continue;
+    const float4 c = L.cr[g];
     const float4 m = L.nf[g];
     const cell_box b = splat_cells(L, c, m, v);
     const float rx = c.x - L.vg_min[0], ry = c.y - L.vg_min[1], rz = c.z - L.vg_min[2];
@@ -831,8 +953,9 @@ int sms() {
 }
 
 struct agg_ws {
-  uint32_t *count, *offs, *tile, *vox_of;
-  unsigned long long *entries;
+  uint32_t *count, *offs, *list, *vox_of;
+  fuse_count *fc;
+  unsigned long long *entries, *sorted;
   uint8_t *canny_state;     // edge mode 1 (the other Canny buffers alias
   unsigned int *changed;    // entries and vox_of, which the fusion fills later)
   unsigned long long *axis_sum;  // cell slabs: [n^3][3] fixed-point normal sums
@@ -845,10 +968,12 @@ agg_ws carve_agg(pe_carve &c, int64_t total_pix, int G) {
   agg_ws w;
   int64_t nv = (int64_t)G * G * G;
   w.count = c.take<uint32_t>((size_t)nv);
-  w.offs = c.take<uint32_t>((size_t)nv + 1);
-  w.tile = c.take<uint32_t>((size_t)((nv + kScanTile - 1) / kScanTile));
+  w.offs = c.take<uint32_t>((size_t)nv);
+  w.list = c.take<uint32_t>((size_t)total_pix);
+  w.fc = c.take<fuse_count>(1);
   w.vox_of = c.take<uint32_t>((size_t)total_pix);
   w.entries = c.take<unsigned long long>((size_t)total_pix);
+  w.sorted = c.take<unsigned long long>((size_t)total_pix);
   w.canny_state = c.take<uint8_t>((size_t)total_pix);
   w.changed = c.take<unsigned int>(1);
   const int64_t n3 = (int64_t)PE_VGRID * PE_VGRID * PE_VGRID;
@@ -942,6 +1067,7 @@ extern "C" pe_status pe_aggregate_views(const pe_view *views, int32_t n_views,
   int cap = sms() * 16;
 
   PE_TRY_CUDA(cudaMemsetAsync(w.count, 0, sizeof(uint32_t) * nvox, s));
+  PE_TRY_CUDA(cudaMemsetAsync(w.fc, 0, sizeof(fuse_count), s));
   PE_TRY_CUDA(cudaMemsetAsync(cr, 0, sizeof(float4) * total_pix, s));
   PE_TRY_CUDA(cudaMemsetAsync(nf, 0, sizeof(float4) * total_pix, s));
   const uint8_t *cstate = nullptr;
@@ -974,36 +1100,53 @@ extern "C" pe_status pe_aggregate_views(const pe_view *views, int32_t n_views,
   } else if (prm->edge_mode != 0) {
     return pe_fail(PE_EINVAL, "pe_aggregate_views: edge_mode must be 0 or 1");
   }
-  fuse_classify_kernel<<<grid_for(total_pix, 256, cap), 256, 0, s>>>(
+  const int64_t px_blocks = (total_pix + 256 * kClassifyPx - 1) / (256 * kClassifyPx);
+  fuse_classify_kernel<<<(unsigned)px_blocks, 256, 0, s>>>(
       L, nd, gfb_mask, prm->edge_tau, cstate, prm->bbox_min[0], prm->bbox_min[1],
-      prm->bbox_min[2], prm->inv_voxel, G, w.vox_of, w.count);
+      prm->bbox_min[2], prm->inv_voxel, G, w.vox_of, w.count, w.list, w.fc);
   PE_TRY_LAUNCH("fuse_classify_kernel");
-  int64_t n_tiles = (nvox + kScanTile - 1) / kScanTile;
-  if (n_tiles > kScanTile) return pe_fail(PE_EUNSUPPORTED, "voxel grid too large for the scan");
-  scan_tile_sums<<<(int)n_tiles, kScanThreads, 0, s>>>(w.count, nvox, w.tile);
-  PE_TRY_LAUNCH("scan_tile_sums");
-  scan_tile_offsets<<<1, kScanThreads, 0, s>>>(w.tile, n_tiles);
-  PE_TRY_LAUNCH("scan_tile_offsets");
-  scan_apply<<<(int)n_tiles, kScanThreads, 0, s>>>(w.count, nvox, w.tile, w.offs);
-  PE_TRY_LAUNCH("scan_apply");
-  fuse_scatter_kernel<<<grid_for(total_pix, 256, cap), 256, 0, s>>>(L, w.vox_of, w.offs,
-                                                                     w.count, w.entries);
+  // (the kernels read the numbers of voxels and keys, at most total_pix, on the
+  // device)
+  fuse_offsets_kernel<<<grid_for(total_pix, 256, cap / 4), 256, 0, s>>>(w.list, w.count, w.offs, w.fc);
+  PE_TRY_LAUNCH("fuse_offsets_kernel");
+  fuse_scatter_kernel<<<grid_for(total_pix, 256, cap), 256, 0, s>>>(L, w.vox_of, w.offs, w.entries);
   PE_TRY_LAUNCH("fuse_scatter_kernel");
-  // segment heads are found by slot; the kernel reads the entry count
-  // offs[nvox] on the device (at most total_pix)
+  fuse_rank_kernel<<<grid_for(total_pix, 256, cap), 256, 0, s>>>(w.entries, w.offs, w.count, w.fc,
+                                                                 w.sorted);
+  PE_TRY_LAUNCH("fuse_rank_kernel");
   fuse_segment_kernel<<<grid_for(total_pix, kFuseThreads, cap), kFuseThreads, 0, s>>>(
-      L, nd, w.entries, w.offs, nvox, cr, nf);
+      L, nd, w.sorted, w.list, w.offs, w.count, w.fc, cr, nf);
   PE_TRY_LAUNCH("fuse_segment_kernel");
+  int64_t leaves = 0, most_leaves = 0;
+  int most_lev = 0;
+  for (int v = 0; v < n_views; ++v) {
+    const int64_t n = (int64_t)L.tw[v][0] * L.th[v][0];
+    leaves += n;
+    most_leaves = n > most_leaves ? n : most_leaves;
+    most_lev = L.nlev[v] > most_lev ? L.nlev[v] : most_lev;
+  }
+  pyramid_leaf_kernel<<<dim3((unsigned)grid_for(most_leaves, 128, cap), (unsigned)n_views), 128, 0, s>>>(
+      L, nodes);
+  PE_TRY_LAUNCH("pyramid_leaf_kernel");
+  for (int l = 1; l < most_lev; ++l) {
+    int64_t most = 1;
+    for (int v = 0; v < n_views; ++v)
+      if (l < L.nlev[v]) most = std::max(most, (int64_t)L.tw[v][l] * L.th[v][l]);
+    pyramid_up_kernel<<<dim3((unsigned)grid_for(most, 128, cap), (unsigned)n_views), 128, 0, s>>>(
+        L, l, nodes);
+    PE_TRY_LAUNCH("pyramid_up_kernel");
+  }
+  const int64_t slots = leaves * (PE_LEAF * PE_LEAF);
   const int64_t n3 = (int64_t)PE_VGRID * PE_VGRID * PE_VGRID;
   PE_TRY_CUDA(cudaMemsetAsync(vmask, 0, sizeof(uint32_t) * ((size_t)n3 + 1), s));
   PE_TRY_CUDA(cudaMemsetAsync(w.axis_sum, 0, sizeof(unsigned long long) * 3 * (size_t)n3, s));
   PE_TRY_CUDA(cudaMemsetAsync(w.axis_cnt, 0, sizeof(unsigned int) * (size_t)n3, s));
-  vgrid_kernel<<<grid_for(total_pix, 256, cap), 256, 0, s>>>(L, vmask, w.axis_sum, w.axis_cnt);
+  vgrid_kernel<<<grid_for(slots, 256, cap), 256, 0, s>>>(L, slots, vmask, w.axis_sum, w.axis_cnt);
   PE_TRY_LAUNCH("vgrid_kernel");
   cell_axis_kernel<<<grid_for(n3, 256, cap), 256, 0, s>>>(n3, w.axis_sum, w.axis_cnt, w.axis,
                                                           w.hkey);
   PE_TRY_LAUNCH("cell_axis_kernel");
-  cell_height_kernel<<<grid_for(total_pix, 256, cap), 256, 0, s>>>(L, w.axis, w.hkey);
+  cell_height_kernel<<<grid_for(slots, 256, cap), 256, 0, s>>>(L, slots, w.axis, w.hkey);
   PE_TRY_LAUNCH("cell_height_kernel");
   {
     float mag = 0.0f;
@@ -1016,21 +1159,9 @@ extern "C" pe_status pe_aggregate_views(const pe_view *views, int32_t n_views,
   out->vgrid_n = L.vg_n;
   out->vgrid_cell = L.vg_cell;
   for (int k = 0; k < 3; ++k) out->vgrid_min[k] = L.vg_min[k];
-  for (int v = 0; v < n_views; ++v) {
-    pyramid_leaf_kernel<<<grid_for((int64_t)L.tw[v][0] * L.th[v][0], 128, cap), 128, 0, s>>>(
-        L, v, nodes);
-    PE_TRY_LAUNCH("pyramid_leaf_kernel");
-    for (int l = 1; l < L.nlev[v]; ++l) {
-      pyramid_up_kernel<<<grid_for((int64_t)L.tw[v][l] * L.th[v][l], 128, cap), 128, 0, s>>>(
-          L, v, l, nodes);
-      PE_TRY_LAUNCH("pyramid_up_kernel");
-    }
-  }
-  slab_clear_kernel<<<grid_for(L.n_nodes, 256, cap), 256, 0, s>>>(slab, slab_hi, L.n_nodes);
-  PE_TRY_LAUNCH("slab_clear_kernel");
   int64_t n_slab = 0;
   for (int v = 0; v < n_views; ++v)
-    for (int l = 0; l < L.nlev[v] && l < kSlabLevels; ++l) n_slab += (int64_t)L.tw[v][l] * L.th[v][l];
+    for (int l = 0; l < L.nlev[v]; ++l) n_slab += (int64_t)L.tw[v][l] * L.th[v][l];
   pyramid_slab_kernel<<<(unsigned)((n_slab * 32 + 127) / 128), 128, 0, s>>>(L, n_slab, slab,
                                                                           slab_hi);
   PE_TRY_LAUNCH("pyramid_slab_kernel");
