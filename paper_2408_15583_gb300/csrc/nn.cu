@@ -242,6 +242,29 @@ __global__ void __launch_bounds__(GEMM_THREADS, 3) gemm_kernel(const pe_gemm_arg
   }
 }
 
+// C[m][n] = alpha A[m] B[n] (K = 1: the data gradient of a one-output head), BF16,
+// eight columns per thread.  The one product is exact in FP32, so this is what
+// the contraction kernels give.  (157 us there for 2.1M x 32, 134 MB.)
+__global__ void outer_kernel(const bf16 *__restrict__ A, int64_t sam, const bf16 *__restrict__ Bv,
+                             int64_t sbn, int64_t M, int NV, float alpha, bf16 *__restrict__ Cm,
+                             int64_t ldc) {
+  const int64_t total = M * NV;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int n = (int)(t % NV) * 8;
+    const int64_t m = t / NV;
+    const float a = b2f(A[m * sam]);
+    uint4 u;
+    bf162 *e = reinterpret_cast<bf162 *>(&u);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)  // (+ 0: a product of -0 is a sum of +0 there)
+      e[k] = __floats2bfloat162_rn(
+          __fmul_rn(__fadd_rn(__fmul_rn(a, b2f(Bv[(n + 2 * k) * sbn])), 0.0f), alpha),
+          __fmul_rn(__fadd_rn(__fmul_rn(a, b2f(Bv[(n + 2 * k + 1) * sbn])), 0.0f), alpha));
+    *reinterpret_cast<uint4 *>(Cm + m * ldc + n) = u;
+  }
+}
+
 // Sum of the split-K partials in a fixed order (lane ty of a (32, 8) block
 // takes splits ty, ty + 8, ...; the eight are added in order), then the
 // epilogue.
@@ -1041,6 +1064,63 @@ __global__ void maxpool2_bwd_kernel(const bf16 *__restrict__ dY, const uint8_t *
   }
 }
 
+// Eight channels per thread (16-byte activations, 8-byte argument words); the
+// backward thread owns a pooled pixel and writes the four under it.  (One channel
+// per thread: 218 us backward for 134 + 34 MB.)
+__global__ void maxpool2_wide_kernel(const uint4 *__restrict__ X, int B, int H, int W, int CV,
+                                     uint4 *__restrict__ Y, uint2 *__restrict__ arg, int backward) {
+  const int Ho = H / 2, Wo = W / 2;
+  const int64_t total = (int64_t)B * Ho * Wo * CV;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int c = (int)(t % CV);
+    const int64_t p = t / CV;
+    const int x = (int)(p % Wo);
+    const int64_t by = p / Wo;  // b Ho + y
+    const int64_t g = ((2 * by) * W + 2 * x) * CV + c, row = (int64_t)W * CV;
+    if (!backward) {
+      uint4 in[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) in[k] = __ldg(X + g + (k >> 1) * row + (k & 1) * CV);
+      uint4 o;
+      uint32_t am[2] = {0u, 0u};
+      bf16 *out = reinterpret_cast<bf16 *>(&o);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        float best = -INFINITY;
+        uint32_t bi = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float v = b2f(reinterpret_cast<const bf16 *>(&in[k])[e]);
+          if (v > best) {
+            best = v;
+            bi = k;
+          }
+        }
+        out[e] = f2b(best);
+        am[e >> 2] |= bi << (8 * (e & 3));
+      }
+      Y[t] = o;
+      arg[t] = make_uint2(am[0], am[1]);
+    } else {
+      const uint4 d = __ldg(X + t);
+      const uint2 aw = __ldg(arg + t);
+      const bf16 *dv = reinterpret_cast<const bf16 *>(&d);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        uint4 o;
+        bf16 *out = reinterpret_cast<bf16 *>(&o);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const uint32_t a = ((e < 4 ? aw.x : aw.y) >> (8 * (e & 3))) & 0xffu;
+          out[e] = a == (uint32_t)k ? dv[e] : f2b(0.0f);
+        }
+        Y[g + (k >> 1) * row + (k & 1) * CV] = o;
+      }
+    }
+  }
+}
+
 // out[b, 2y+i, 2x+j, off + c] = in[b, y, x, 4c + 2i + j]; dir 1: the reverse.
 // One thread per pixel (Y, X) of the 2H x 2W image and VEC consecutive
 // channels c: the small image's element [b, Y/2, X/2][4c + 2(Y&1) + (X&1)]
@@ -1081,6 +1161,63 @@ __global__ void pixel_shuffle2_kernel(const bf16 *__restrict__ src, int B, int H
         dst[bbase] = src[sbase];
       else
         dst[sbase] = src[bbase];
+    }
+  }
+}
+
+// The same with everything in 16-byte accesses: a thread moves eight channels of
+// the four pixels under one small pixel, 64 contiguous bytes on the small side
+// and 16 per pixel on the large one.  (The form above touches the small side two
+// bytes at a time: 66 us against 20 for 134 MB each way.)
+__global__ void pixel_shuffle2_wide_kernel(const bf16 *__restrict__ src, int B, int H, int W, int C,
+                                           bf16 *__restrict__ dst, int64_t ld_big, int off,
+                                           int dir) {
+  const int CV = C / 8;
+  const int64_t total = (int64_t)B * H * W * CV;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int c0 = (int)(t % CV) * 8;
+    const int64_t small = t / CV;
+    const int x = (int)(small % W);
+    const int64_t q = small / W;
+    const int64_t big0 = (2 * q * (2 * W) + 2 * x) * ld_big + off + c0;  // (q = b H + y)
+    const int64_t row = 2 * (int64_t)W * ld_big;
+    uint4 s4[4], b4[4];
+    uint4 *sp = reinterpret_cast<uint4 *>(const_cast<bf16 *>(dir == 0 ? src : dst) + small * 4 * C +
+                                          4 * c0);
+    bf16 *bp = const_cast<bf16 *>(dir == 0 ? dst : src) + big0;
+    // s4 holds elements 4 k + sub (channel k, sub-pixel sub), b4[sub] channels k
+    if (dir == 0) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s4[k] = __ldg(sp + k);
+      const uint32_t *sw = reinterpret_cast<const uint32_t *>(s4);
+#pragma unroll
+      for (int sub = 0; sub < 4; ++sub) {
+        uint32_t w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)  // channels 2 k, 2 k + 1
+          w[k] = __byte_perm(sw[4 * k + (sub >> 1)], sw[4 * k + 2 + (sub >> 1)],
+                             (sub & 1) ? 0x7632 : 0x5410);
+        b4[sub] = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+#pragma unroll
+      for (int sub = 0; sub < 4; ++sub)
+        *reinterpret_cast<uint4 *>(bp + (sub >> 1) * row + (sub & 1) * ld_big) = b4[sub];
+    } else {
+#pragma unroll
+      for (int sub = 0; sub < 4; ++sub)
+        b4[sub] = __ldg(reinterpret_cast<const uint4 *>(bp + (sub >> 1) * row + (sub & 1) * ld_big));
+      const uint32_t *bw = reinterpret_cast<const uint32_t *>(b4);
+      uint32_t w[16];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)  // channel k: sub-pixels 0, 1 and 2, 3
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          w[2 * k + h] = __byte_perm(bw[4 * (2 * h) + (k >> 1)], bw[4 * (2 * h + 1) + (k >> 1)],
+                                     (k & 1) ? 0x7632 : 0x5410);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        sp[k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
     }
   }
 }
@@ -1415,6 +1552,12 @@ extern "C" pe_status pe_nn_gemm(int32_t M, int32_t N, int64_t K, const void *A, 
     g.part = static_cast<float *>(ws);
   }
   if ((N + TN - 1) / TN > 65535) return pe_fail(PE_EINVAL, "pe_nn_gemm: N too large");
+  if (g_gemm_path == 0 && K == 1 && !c_f32 && !bias && !R && gelu == 0 && g.vec_c && N % 8 == 0) {
+    outer_kernel<<<grid1((int64_t)M * (N / 8), 256), 256, 0, s>>>(g.A, sam, g.B, sbn, M, N / 8, alpha,
+                                                                  static_cast<bf16 *>(C), ldc);
+    PE_TRY_LAUNCH("outer_kernel");
+    return PE_OK;
+  }
   if (split == 1 && g_gemm_path == 0 && pe_gemm_tc_eligible(g)) {
     const pe_status st = pe_gemm_tc(g, s);
     if (st != PE_EUNSUPPORTED) return st;
@@ -1676,12 +1819,65 @@ extern "C" pe_status pe_nn_colsum(const void *X, int64_t M, int32_t N, int64_t l
   return PE_OK;
 }
 
+// Weight and bias gradient of a layer with N <= 4 outputs (the heads: rows of dY
+// too short for a TMA row): a thread owns eight inputs and strides over the
+// pixels, N x 8 sums in registers; the block's threads of the same inputs are
+// added in order.  part[block][N K + N].  (The mma.sync kernel spent a 128-row
+// tile on one row: 355 us for 2.1M pixels of 32 inputs, 134 MB.)
+namespace {
+constexpr int THIN_THREADS = 256;
+template <int N>
+__global__ void __launch_bounds__(THIN_THREADS)
+    wgrad_thin_kernel(const bf16 *__restrict__ dY, int64_t ldy, const bf16 *__restrict__ X,
+                      int64_t ldx, int64_t P, int K, float *__restrict__ part) {
+  extern __shared__ float s_red[];  // [THIN_THREADS][N * 8 + N]
+  constexpr int NV = N * 8 + N;
+  const int kv = K / 8, j = threadIdx.x % kv, r = threadIdx.x / kv, rows = THIN_THREADS / kv;
+  float acc[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) acc[i] = 0.0f;
+  for (int64_t p = (int64_t)blockIdx.x * rows + r; p < P; p += (int64_t)gridDim.x * rows) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4 *>(X + p * ldx) + j);
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      const float g = b2f(dY[p * ldy + n]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        acc[n * 8 + 2 * e] = fmaf(g, __uint_as_float(w[e] << 16), acc[n * 8 + 2 * e]);
+        acc[n * 8 + 2 * e + 1] = fmaf(g, __uint_as_float(w[e] & 0xffff0000u), acc[n * 8 + 2 * e + 1]);
+      }
+      acc[N * 8 + n] += g;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NV; ++i) s_red[threadIdx.x * NV + i] = acc[i];
+  __syncthreads();
+  float *out = part + (size_t)blockIdx.x * (N * K + N);
+  for (int o = threadIdx.x; o < N * K + N; o += THIN_THREADS) {
+    const int n = o < N * K ? o / K : o - N * K, k = o < N * K ? o % K : 0;
+    const int i = o < N * K ? n * 8 + k % 8 : N * 8 + n;
+    float t = 0.0f;
+    for (int q = 0; q < rows; ++q) t += s_red[(q * kv + k / 8) * NV + i];
+    out[o] = t;
+  }
+}
+}  // namespace
+
+constexpr int kThinBlocks = 608;  // four per SM; a constant, as for the other sums
+static bool thin_wgrad(const void *X, int64_t ldx, int32_t N, int32_t K) {
+  return N <= 4 && K % 8 == 0 && K <= 256 && THIN_THREADS % (K / 8) == 0 && ldx % 8 == 0 &&
+         (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+}
+
 // Workspace of pe_nn_linear_wgrad: either path's.
 extern "C" size_t pe_nn_linear_wgrad_workspace(int64_t P, int32_t N, int32_t K) {
   if (P <= 0 || N <= 0 || K <= 0) return 0;
   size_t a = pe_wgrad_tc_workspace(P, N, K), b = pe_nn_gemm_workspace(N, K, P),
          c = pe_nn_colsum_workspace(P, N);
+  const size_t d = N <= 4 ? (size_t)kThinBlocks * ((size_t)N * K + N) * sizeof(float) : 0;
   a = a > b ? a : b;
+  a = a > d ? a : d;
   return (a > c ? a : c) + 256;
 }
 
@@ -1696,6 +1892,19 @@ extern "C" pe_status pe_nn_linear_wgrad(const void *dY, int64_t ldy, const void 
   if (g_gemm_path == 0 && pe_wgrad_tc_eligible(dY, ldy, X, ldx, P, N, K)) {
     const pe_status st = pe_wgrad_tc(dY, ldy, X, ldx, P, N, K, dW, db, static_cast<float *>(ws), s);
     if (st != PE_EUNSUPPORTED) return st;
+  }
+  if (g_gemm_path == 0 && thin_wgrad(X, ldx, N, K)) {
+    const int64_t need = (P + THIN_THREADS / (K / 8) - 1) / (THIN_THREADS / (K / 8));
+    const int blocks = (int)(need < kThinBlocks ? need : kThinBlocks);
+    const size_t smem = sizeof(float) * THIN_THREADS * 9 * N;
+    const bf16 *y = static_cast<const bf16 *>(dY), *x = static_cast<const bf16 *>(X);
+    float *part = static_cast<float *>(ws);
+    if (N == 1) wgrad_thin_kernel<1><<<blocks, THIN_THREADS, smem, s>>>(y, ldy, x, ldx, P, K, part);
+    else if (N == 2) wgrad_thin_kernel<2><<<blocks, THIN_THREADS, smem, s>>>(y, ldy, x, ldx, P, K, part);
+    else if (N == 3) wgrad_thin_kernel<3><<<blocks, THIN_THREADS, smem, s>>>(y, ldy, x, ldx, P, K, part);
+    else wgrad_thin_kernel<4><<<blocks, THIN_THREADS, smem, s>>>(y, ldy, x, ldx, P, K, part);
+    PE_TRY_LAUNCH("wgrad_thin_kernel");
+    return pe_wgrad_reduce(part, blocks, (int64_t)N * K, (int64_t)N * K + N, dW, db, s);
   }
   const pe_status st = pe_nn_gemm(N, K, P, dY, 1, ldy, X, ldx, 1, dW, K, 1, nullptr, nullptr, 0,
                                   nullptr, 0, 0, 1.0f, 0.0f, ws, ws_bytes, stream);
@@ -1719,6 +1928,14 @@ extern "C" pe_status pe_nn_maxpool2(const void *X, int32_t B, int32_t H, int32_t
   NN_CHECK_STREAM;
   if (!X || !Y || !arg || B <= 0 || H < 2 || W < 2 || C <= 0 || (H & 1) || (W & 1))
     return pe_fail(PE_EINVAL, "pe_nn_maxpool2: bad arguments (even H, W)");
+  if (C % 8 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15) == 0 &&
+      (reinterpret_cast<uintptr_t>(arg) & 7) == 0) {
+    maxpool2_wide_kernel<<<grid1((int64_t)B * H * W * C / 32, 256), 256, 0, s>>>(
+        static_cast<const uint4 *>(X), B, H, W, C / 8, static_cast<uint4 *>(Y),
+        reinterpret_cast<uint2 *>(arg), backward ? 1 : 0);
+    PE_TRY_LAUNCH("maxpool2_wide_kernel");
+    return PE_OK;
+  }
   if (!backward) {
     maxpool2_fwd_kernel<<<grid1((int64_t)B * H * W * C / 4, 256), 256, 0, s>>>(
         static_cast<const bf16 *>(X), B, H, W, C, static_cast<bf16 *>(Y), arg);
@@ -1744,7 +1961,11 @@ extern "C" pe_status pe_nn_pixel_shuffle2(const void *src, int32_t B, int32_t H,
     const bool v8 = C % 8 == 0 && off % 8 == 0 && ld_big % 8 == 0 &&
                     (reinterpret_cast<uintptr_t>(big) & 15) == 0;
     const int64_t n = (int64_t)B * 4 * H * W * (v8 ? C / 8 : C);
-    if (v8)
+    if (v8 && (reinterpret_cast<uintptr_t>(backward ? dst : src) & 15) == 0)
+      pixel_shuffle2_wide_kernel<<<grid1(n / 4, 256), 256, 0, s>>>(
+          static_cast<const bf16 *>(src), B, H, W, C, static_cast<bf16 *>(dst), ld_big, off,
+          backward ? 1 : 0);
+    else if (v8)
       pixel_shuffle2_kernel<8><<<grid1(n, 256), 256, 0, s>>>(
           static_cast<const bf16 *>(src), B, H, W, C, static_cast<bf16 *>(dst), ld_big, off,
           backward ? 1 : 0);

@@ -242,3 +242,52 @@ def test_point_attributes_ties(kind, k_r, k_n):
     # FP32 rounding of a unit vector: 1 - |dot| <= (2^-24 sqrt(3))^2 / 2 + FP64 noise
     # amplified by the gap bound (1e-16 / 1e-3)
     assert bool((dot > 1 - 1e-7).all())
+
+
+# ---- pooling, sub-pixel shuffle, one-output heads -----------------------------------
+
+@pytest.mark.parametrize("B,H,W,C", [(1, 2, 2, 8), (2, 6, 10, 40), (3, 34, 18, 64)])
+def test_pool_and_shuffle(B, H, W, C):
+    o, g = ops(), gen(B + H + W + C)
+    x = rnd(g, B, H, W, C).to(BF)
+    x[:, ::3] = x[:, ::3].round()                     # ties: the first of the four wins
+    y = torch.empty(B, H // 2, W // 2, C, dtype=BF, device=DEV)
+    arg = torch.empty(y.shape, dtype=torch.uint8, device=DEV)
+    o.maxpool(x, B, H, W, C, y, arg)
+    four = x.view(B, H // 2, 2, W // 2, 2, C).permute(0, 1, 3, 2, 4, 5).reshape(*y.shape[:3], 4, C)
+    best = four.float().max(3).values
+    assert torch.equal(y.float(), best)
+    first = (four.float() == best[..., None, :]).float().argmax(3)
+    assert torch.equal(arg.long(), first)
+    dy, dx = rnd(g, *y.shape).to(BF), torch.empty_like(x)
+    o.maxpool(dy, B, H, W, C, dx, arg, backward=True)
+    want = torch.zeros_like(four).scatter_(3, first[..., None, :], dy[..., None, :])
+    assert torch.equal(dx.view(B, H // 2, 2, W // 2, 2, C).permute(0, 1, 3, 2, 4, 5).reshape(four.shape),
+                       want)
+    # [B, H, W, 4 C] <-> channels 8 .. 8 + C of a [B, 2 H, 2 W, C + 24] image
+    small = rnd(g, B, H, W, 4 * C).to(BF)
+    big = torch.full((B, 2 * H, 2 * W, C + 24), 7.0, dtype=BF, device=DEV)
+    o.shuffle(small, B, H, W, C, big, C + 24, 8)
+    ref = torch.nn.functional.pixel_shuffle(small.permute(0, 3, 1, 2).float(), 2).permute(0, 2, 3, 1)
+    assert torch.equal(big[..., 8:8 + C].float(), ref)
+    assert bool((big[..., :8] == 7.0).all()) and bool((big[..., 8 + C:] == 7.0).all())
+    back = torch.empty_like(small)
+    o.shuffle(big, B, H, W, C, back, C + 24, 8, backward=True)
+    assert torch.equal(back, small)
+
+
+# layers of one to four outputs; FP32 sums over P products err below 1e-5, and the
+# data gradient of a one-output layer is one product, rounded once to BF16
+@pytest.mark.parametrize("N", [1, 2, 3, 4])
+@pytest.mark.parametrize("P,K", [(1, 8), (63, 32), (100_001, 32), (5000, 256), (777, 40)])
+def test_thin_layer_gradients(P, K, N):
+    o, g = ops(), gen(P + K + N)
+    dy, x, W = rnd(g, P, N).to(BF), rnd(g, P, K).to(BF), rnd(g, N, K).to(BF)
+    dW, db = torch.empty(N, K, device=DEV), torch.empty(N, device=DEV)
+    dx = torch.empty(P, K, dtype=BF, device=DEV)
+    o.linear_bwd(dy, x, K, W, dx, K, dW, db)
+    assert rel(dW, dy.double().T @ x.double()) < 1e-5 and rel(db, dy.double().sum(0)) < 1e-5
+    if N == 1:
+        assert torch.equal(dx, (dy.float() * W.float()).to(BF))
+    else:
+        assert rel(dx, dy.double() @ W.double()) < BF_TOL
