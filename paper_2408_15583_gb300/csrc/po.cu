@@ -348,16 +348,16 @@ __global__ void __launch_bounds__(kPoThreads, 4)
 #pragma unroll
     for (int i = 0; i < kAcc; ++i) s_red[tid][i] = (double)hi[i] + (double)lo[i];
     __syncthreads();
-    if (tid < FL && f0 + tid < C.nf) {
-      double acc[kAcc];
-#pragma unroll
-      for (int i = 0; i < kAcc; ++i) acc[i] = 0.0;
-      for (int rl = 0; rl < RL; ++rl)
-#pragma unroll
-        for (int i = 0; i < kAcc; ++i) acc[i] += s_red[rl * FL + tid][i];
-      int64_t o = (((int64_t)g * C.n_chunks + chunk) * C.nf + (f0 + tid)) * kAcc;
-#pragma unroll
-      for (int i = 0; i < kAcc; ++i) part[o + i] = acc[i];
+    // a thread per (frequency, sum): an FP64 addition occupies its pipe for a
+    // whole warp whatever its active lanes, and one lane adding all eight sums of
+    // 256 ray lanes took most of a one-frequency launch (184 us for 64 angles of
+    // 128^2 rays)
+    for (int o = tid; o < FL * kAcc; o += kPoThreads) {
+      const int fl = o / kAcc, i = o % kAcc;
+      if (f0 + fl >= C.nf) break;
+      double acc = 0.0;
+      for (int rl = 0; rl < RL; ++rl) acc += s_red[rl * FL + fl][i];
+      part[(((int64_t)g * C.n_chunks + chunk) * C.nf + (f0 + fl)) * kAcc + i] = acc;
     }
     __syncthreads();
   }
@@ -664,17 +664,12 @@ __global__ void __launch_bounds__(kPoThreads, PE_PO_MINB)
                             : (double)hi[SMC ? 0 : a] + (double)lo[SMC ? 0 : a];
       }
       __syncthreads();
-      const int f = (c0 + tid) * FT + q;
-      if (tid < FL && c0 + tid < n_fc && f < C.nf) {
-        double acc[kAcc];
-#pragma unroll
-        for (int i = 0; i < kAcc; ++i) acc[i] = 0.0;
-        for (int rl = 0; rl < RL; ++rl)
-#pragma unroll
-          for (int i = 0; i < kAcc; ++i) acc[i] += s_red[rl * FL + tid][i];
-        int64_t o = (((int64_t)g * C.n_chunks + chunk) * C.nf + f) * kAcc;
-#pragma unroll
-        for (int i = 0; i < kAcc; ++i) part[o + i] = acc[i];
+      for (int o = tid; o < FL * kAcc; o += kPoThreads) {
+        const int fl = o / kAcc, i = o % kAcc, f = (c0 + fl) * FT + q;
+        if (c0 + fl >= n_fc || f >= C.nf) break;
+        double acc = 0.0;
+        for (int rl = 0; rl < RL; ++rl) acc += s_red[rl * FL + fl][i];
+        part[(((int64_t)g * C.n_chunks + chunk) * C.nf + f) * kAcc + i] = acc;
       }
     }
     __syncthreads();
@@ -684,31 +679,38 @@ __global__ void __launch_bounds__(kPoThreads, PE_PO_MINB)
 
 // E[g0+g][f][12] = the chunks' sums (fixed order) taken back from the basis
 // (e1, e2) across ks to Cartesian components: for polarisation p, component
-// x and re/im r, E = e1[x] S[p][e1][r] + e2[x] S[p][e2][r].
+// x and re/im r, E = e1[x] S[p][e1][r] + e2[x] S[p][e2][r].  Eight lanes per (g,
+// f), one sum each: lane i = 4 p + 2 (e1 or e2) + r; the lanes of e1 then write.
+// (One thread per (g, f) added eight chains over the chunks, 135 us for 132 of
+// them over 304 chunks.)
 __global__ void po_reduce_kernel(const double *__restrict__ part, const __grid_constant__ po_consts C,
                                  int nf_total, int f_base, double *__restrict__ E) {
-  const int64_t n = (int64_t)C.ng * C.nf;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int f = (int)(t % C.nf);
-    const int g = (int)(t / C.nf);
-    double S[kAcc];
+  const int64_t n = (int64_t)C.ng * C.nf * kAcc;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x; t0 < n; t0 += step) {
+    const int64_t t = t0 + threadIdx.x;
+    const bool on = t < n;
+    const int i = (int)(t % kAcc);
+    const int f = on ? (int)(t / kAcc % C.nf) : 0, g = on ? (int)(t / kAcc / C.nf) : 0;
+    double S = 0.0;
+    const double *q = part + ((int64_t)g * C.n_chunks * C.nf + f) * kAcc + i;
+    const int64_t next = (int64_t)C.nf * kAcc;
+    int c = 0;
+    for (; on && c + 8 <= C.n_chunks; c += 8) {
+      double v[8];  // eight loads in flight, added in order
 #pragma unroll
-    for (int i = 0; i < kAcc; ++i) S[i] = 0.0;
-    for (int c = 0; c < C.n_chunks; ++c) {
-      const double *q = part + (((int64_t)g * C.n_chunks + c) * C.nf + f) * kAcc;
+      for (int k = 0; k < 8; ++k) v[k] = __ldg(q + (c + k) * next);
 #pragma unroll
-      for (int i = 0; i < kAcc; ++i) S[i] += q[i];
+      for (int k = 0; k < 8; ++k) S += v[k];
     }
-    double *e = E + (((int64_t)(C.g0 + g) * nf_total) + f_base + f) * 12;
-#pragma unroll
-    for (int p = 0; p < 2; ++p)
+    for (; on && c < C.n_chunks; ++c) S += __ldg(q + c * next);
+    const double S2 = __shfl_down_sync(0xffffffffu, S, 2);
+    if (on && !(i & 2)) {
+      double *e = E + (((int64_t)(C.g0 + g) * nf_total) + f_base + f) * 12 + (i >> 2) * 6 + (i & 1);
 #pragma unroll
       for (int x = 0; x < 3; ++x)
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-          e[(p * 3 + x) * 2 + r] = __dadd_rn(__dmul_rn((double)C.e1[g][x], S[(p * 2) * 2 + r]),
-                                             __dmul_rn((double)C.e2[g][x], S[(p * 2 + 1) * 2 + r]));
+        e[x * 2] = __dadd_rn(__dmul_rn((double)C.e1[g][x], S), __dmul_rn((double)C.e2[g][x], S2));
+    }
   }
 }
 
@@ -871,7 +873,7 @@ pe_status pe_launch_po(const pe_hits &h, int32_t n_groups, int64_t rpg, const fl
         pe_event_after("po_kernel", s);
         PE_TRY_LAUNCH("po_kernel");
       }
-      int64_t n = (int64_t)ng * nf;
+      int64_t n = (int64_t)ng * nf * kAcc;
       int blocks = (int)((n + 127) / 128);
       po_reduce_kernel<<<blocks, 128, 0, s>>>(part, C, n_freq, fb, E);
       PE_TRY_LAUNCH("po_reduce_kernel");
