@@ -600,6 +600,18 @@ pe_status pe_nn_linear_wgrad(const void *dY, int64_t ldy, const void *X, int64_t
                              int32_t N, int32_t K, float *dW, float *db, void *ws, size_t ws_bytes,
                              void *stream);
 
+/* 3x3 convolution with zero padding 1: y [B][H][W][Cout] (BF16) = x [B][H][W][Cin]
+ * with w [Cout][3][3][Cin] (BF16) + bias [Cout] (FP32, nullable).  Weight and bias
+ * gradient: FP32 dW [Cout][3][3][Cin], db [Cout] (nullable), overwritten.  x, w, y
+ * and dY on 16-byte boundaries. */
+size_t pe_nn_conv3_workspace(int32_t B, int32_t H, int32_t W, int32_t Cin, int32_t Cout);
+pe_status pe_nn_conv3(const void *x, int32_t B, int32_t H, int32_t W, int32_t Cin, const void *w,
+                      const float *bias, void *y, int32_t Cout, void *ws, size_t ws_bytes,
+                      void *stream);
+pe_status pe_nn_conv3_wgrad(const void *dY, const void *x, int32_t B, int32_t H, int32_t W,
+                            int32_t Cin, int32_t Cout, float *dW, float *db, void *ws,
+                            size_t ws_bytes, void *stream);
+
 /* dst [Cc][R] = transpose of src [R][Cc] (BF16, row-major, distinct buffers). */
 pe_status pe_nn_transpose(const void *src, int32_t R, int32_t Cc, void *dst, void *stream);
 

@@ -113,6 +113,11 @@ SIGNATURES = {
     "pe_nn_linear_wgrad_workspace": (C.c_size_t, [C.c_int64, C.c_int32, C.c_int32]),
     "pe_nn_linear_wgrad": (C.c_int, [P, C.c_int64, P, C.c_int64, C.c_int64, C.c_int32, C.c_int32,
                                      P, P, P, C.c_size_t, P]),
+    "pe_nn_conv3_workspace": (C.c_size_t, [C.c_int32] * 5),
+    "pe_nn_conv3": (C.c_int, [P, C.c_int32, C.c_int32, C.c_int32, C.c_int32, P, P, P, C.c_int32, P,
+                              C.c_size_t, P]),
+    "pe_nn_conv3_wgrad": (C.c_int, [P, P, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, P,
+                                    P, P, C.c_size_t, P]),
     "pe_nn_gelu_bwd": (C.c_int, [P, P, C.c_int64, P, P]),
     "pe_nn_maxpool2": (C.c_int, [P, C.c_int32, C.c_int32, C.c_int32, C.c_int32, P, P, C.c_int32,
                                  P]),

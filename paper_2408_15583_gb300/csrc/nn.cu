@@ -1912,6 +1912,118 @@ extern "C" pe_status pe_nn_linear_wgrad(const void *dY, int64_t ldy, const void 
   return pe_nn_colsum(dY, P, N, ldy, db, 0, ws, ws_bytes, stream);
 }
 
+// 3x3 convolution, y = col(x) w^T + bias with col the neighbourhood matrix.  The
+// TMA loads gather it from the image itself (im2col mode) where its channels
+// fill whole 64-channel blocks and the contraction would run unsplit on the
+// tcgen05 kernel anyway (same products in the same order, same bits); else col is
+// written to the workspace.  Writing and reading col, nine times the image, was
+// a tenth of the network's forward pass: 16 x 256^2 images, 6.15 -> 5.32 ms
+// together with the heads' rows written from registers (nn_tc.cu, MODE 4).
+static pe_gemm_args conv_args(const void *x, int32_t B, int32_t H, int32_t W, int32_t Cin,
+                              const void *w, const float *bias, void *y, int32_t Cout) {
+  pe_gemm_args g;
+  memset(&g, 0, sizeof(g));
+  g.M = B * H * W;
+  g.N = Cout;
+  g.K = 9 * (int64_t)Cin;
+  g.A = static_cast<const bf16 *>(x);
+  g.sak = g.sbk = 1;
+  g.sam = 9 * (int64_t)Cin;
+  g.B = static_cast<const bf16 *>(w);
+  g.sbn = 9 * (int64_t)Cin;
+  g.C = y;
+  g.ldc = Cout;
+  g.bias = bias;
+  g.alpha = 1.0f;
+  auto al = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  g.vec_c = al(y) && Cout % 8 == 0 && (!bias || (reinterpret_cast<uintptr_t>(bias) & 3) == 0);
+  return g;
+}
+
+static bool conv_sizes(int32_t B, int32_t H, int32_t W, int32_t Cin, int32_t Cout) {
+  return B > 0 && H > 0 && W > 0 && Cin > 0 && Cout > 0 && (int64_t)B * H * W < (1ll << 31) - 4096;
+}
+
+// Whether both passes gather (then no col is written and the workspace holds none).
+static bool conv_gathered(int32_t B, int32_t H, int32_t W, int32_t Cin, int32_t Cout) {
+  return g_gemm_path == 0 && gemm_split(B * H * W, Cout, 9 * (int64_t)Cin, nullptr) == 1 &&
+         pe_conv3_tc_sizes(B, H, W, Cin, Cout);
+}
+
+extern "C" size_t pe_nn_conv3_workspace(int32_t B, int32_t H, int32_t W, int32_t Cin, int32_t Cout) {
+  if (!conv_sizes(B, H, W, Cin, Cout)) return 0;
+  const int64_t P = (int64_t)B * H * W;
+  const size_t col = ((size_t)P * 9 * Cin * sizeof(bf16) + 255) & ~size_t(255);
+  const size_t a = pe_nn_gemm_workspace((int32_t)P, Cout, 9 * (int64_t)Cin),
+               b = pe_nn_linear_wgrad_workspace(P, Cout, 9 * Cin);
+  return (conv_gathered(B, H, W, Cin, Cout) ? 0 : col) + (a > b ? a : b) + 512;
+}
+
+// col in the workspace (256-byte aligned), with the rest of it after col.
+static bf16 *conv_col(const void *x, int32_t B, int32_t H, int32_t W, int32_t Cin, void *ws,
+                      size_t ws_bytes, char **rest, size_t *rest_bytes, cudaStream_t s,
+                      pe_status *st) {
+  const uintptr_t p = (reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255);
+  const size_t skip = p - reinterpret_cast<uintptr_t>(ws);
+  const size_t bytes = ((size_t)B * H * W * 9 * Cin * sizeof(bf16) + 255) & ~size_t(255);
+  if (ws_bytes < skip + bytes) {
+    *st = pe_fail(PE_ENOMEM, "pe_nn_conv3: workspace");
+    return nullptr;
+  }
+  *rest = reinterpret_cast<char *>(p) + bytes;
+  *rest_bytes = ws_bytes - skip - bytes;
+  *st = pe_nn_im2col3(x, B, H, W, Cin, reinterpret_cast<void *>(p), 0, s);
+  return reinterpret_cast<bf16 *>(p);
+}
+
+extern "C" pe_status pe_nn_conv3(const void *x, int32_t B, int32_t H, int32_t W, int32_t Cin,
+                                 const void *w, const float *bias, void *y, int32_t Cout, void *ws,
+                                 size_t ws_bytes, void *stream) {
+  NN_CHECK_STREAM;
+  if (!x || !w || !y || !conv_sizes(B, H, W, Cin, Cout))
+    return pe_fail(PE_EINVAL, "pe_nn_conv3: bad arguments");
+  if (!ws || ws_bytes < pe_nn_conv3_workspace(B, H, W, Cin, Cout))
+    return pe_fail(PE_ENOMEM, "pe_nn_conv3: workspace");
+  const pe_gemm_args g = conv_args(x, B, H, W, Cin, w, bias, y, Cout);
+  if (conv_gathered(B, H, W, Cin, Cout)) {
+    if (((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w)) & 15) != 0 || !g.vec_c)
+      return pe_fail(PE_EINVAL, "pe_nn_conv3: pointers on 16-byte boundaries");
+    return pe_conv3_tc(g, B, H, W, Cin, s);
+  }
+  pe_status st;
+  char *rest;
+  size_t rest_bytes;
+  const bf16 *col = conv_col(x, B, H, W, Cin, ws, ws_bytes, &rest, &rest_bytes, s, &st);
+  if (st != PE_OK) return st;
+  return pe_nn_gemm(g.M, Cout, g.K, col, g.K, 1, w, 1, g.K, y, Cout, 0, bias, nullptr, 0, nullptr, 0,
+                    0, 1.0f, 0.0f, rest, rest_bytes, stream);
+}
+
+extern "C" pe_status pe_nn_conv3_wgrad(const void *dY, const void *x, int32_t B, int32_t H, int32_t W,
+                                       int32_t Cin, int32_t Cout, float *dW, float *db, void *ws,
+                                       size_t ws_bytes, void *stream) {
+  NN_CHECK_STREAM;
+  if (!dY || !x || !dW || !conv_sizes(B, H, W, Cin, Cout))
+    return pe_fail(PE_EINVAL, "pe_nn_conv3_wgrad: bad arguments");
+  if (!ws || ws_bytes < pe_nn_conv3_workspace(B, H, W, Cin, Cout))
+    return pe_fail(PE_ENOMEM, "pe_nn_conv3_wgrad: workspace");
+  const int64_t P = (int64_t)B * H * W;
+  if (conv_gathered(B, H, W, Cin, Cout)) {
+    if (((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dY)) & 15) != 0)
+      return pe_fail(PE_EINVAL, "pe_nn_conv3_wgrad: pointers on 16-byte boundaries");
+    const int32_t img[3] = {B, H, W};
+    return pe_wgrad_tc(dY, Cout, x, 9 * (int64_t)Cin, P, Cout, 9 * Cin, dW, db,
+                       static_cast<float *>(ws), s, img);
+  }
+  pe_status st;
+  char *rest;
+  size_t rest_bytes;
+  const bf16 *col = conv_col(x, B, H, W, Cin, ws, ws_bytes, &rest, &rest_bytes, s, &st);
+  if (st != PE_OK) return st;
+  return pe_nn_linear_wgrad(dY, Cout, col, 9 * (int64_t)Cin, P, Cout, 9 * Cin, dW, db, rest,
+                            rest_bytes, stream);
+}
+
 extern "C" pe_status pe_nn_gelu_bwd(const void *dA, const void *Z, int64_t n, void *dZ,
                                     void *stream) {
   NN_CHECK_STREAM;

@@ -134,7 +134,14 @@ bool pe_wgrad_tc_eligible(const void *dY, int64_t ldy, const void *X, int64_t ld
                           int32_t K);
 size_t pe_wgrad_tc_workspace(int64_t P, int32_t N, int32_t K);
 pe_status pe_wgrad_tc(const void *dY, int64_t ldy, const void *X, int64_t ldx, int64_t P, int32_t N,
-                      int32_t K, float *dW, float *db, float *part, cudaStream_t s);
+                      int32_t K, float *dW, float *db, float *part, cudaStream_t s,
+                      const int32_t *conv = nullptr);
+// The contraction with A = the neighbourhood matrix [B H W][9 C] of the image
+// g.A [B][H][W][C] (3x3, zero padding 1), gathered by the TMA loads; and the weight
+// gradient likewise (conv = {B, H, W}, K = 9 C).
+bool pe_conv3_tc_sizes(int32_t B, int32_t H, int32_t W, int32_t C, int32_t N);
+pe_status pe_conv3_tc(const pe_gemm_args &g, int32_t B, int32_t H, int32_t W, int32_t C,
+                      cudaStream_t s);
 // Split-K factor of the mma.sync kernel.
 int64_t pe_gemm_split(int32_t M, int32_t N, int64_t K);
 // dW [nw], db [n_all - nw] (nullable) = sums of part[split][n_all] in split order.

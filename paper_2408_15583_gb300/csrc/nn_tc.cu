@@ -305,6 +305,9 @@ __global__ void __launch_bounds__(TC_THREADS, 3)
 // tiles.
 //   MODE 0  C = acc (+ bias)            MODE 1  C = acc (+ bias) + X
 //   MODE 2  Z = acc (+ bias), C = GELU  MODE 3  C = (acc (+ bias)) GELU'(X)
+//   MODE 4  FP32 C = acc (+ bias) (+ R), N <= 8: the heads, whose rows are too
+//           short to stage; a lane writes its row's few values itself (1048576
+//           rows, K = 32: 37 us, 70 us through the staged kernel)
 // The arithmetic per element is pe_gemm_store8's, in the same order.
 //
 // Against the kernel above on the same contractions (which holds a 128 x 256
@@ -352,12 +355,22 @@ struct st_cfg {
   }
 };
 
+// The image behind an im2col operand: element (p, tap C + c) of the matrix is
+// channel c of the pixel that tap (3 ky + kx) reads at pixel p.
+struct conv_img {
+  int C, W, H;  // C = 0: a plain matrix
+};
+
 struct st_args {
   int M, N, K;
   int tiles_n;
   int items;  // output tiles
   float alpha;
   const float *bias;
+  conv_img img;  // of A
+  float *c32;    // MODE 4
+  int64_t ldc, ldr;
+  const bf16 *r;
   uint32_t wait_limit;
   unsigned int *err;
 };
@@ -389,6 +402,32 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void 
                "r"(x), "r"(y), "r"(sm_u32(src))
                : "memory");
 }
+// A column of the 3x3 neighbourhood matrix: consecutive pixels in raster order
+// from (w, h, n) on, each moved by (ow, oh), channels c .. c + 63; pixels outside
+// the image read as zero (a TMA load in im2col mode).
+__device__ __forceinline__ void tma_load_im2col(void *dst, const CUtensorMap *map, int c, int w,
+                                                int h, int n, uint16_t ow, uint16_t oh,
+                                                uint64_t *bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4, %5}], [%6], {%7, %8};\n" ::"r"(sm_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(w), "r"(h), "r"(n), "r"(sm_u32(bar)),
+      "h"(ow), "h"(oh)
+      : "memory");
+}
+
+__device__ __forceinline__ void load_conv_box(void *dst, const CUtensorMap *map, const conv_img &im,
+                                              int k0, int p, uint64_t *bar) {
+  int tap = k0 / im.C, c = k0 - tap * im.C;
+  if (tap > 8) {  // past the matrix: channels outside the image are zero
+    tap = 8;
+    c = im.C;
+  }
+  const int x = p % im.W, y = p / im.W;
+  tma_load_im2col(dst, map, c, x - 1, y % im.H - 1, y / im.H, (uint16_t)(tap % 3),
+                  (uint16_t)(tap / 3), bar);
+}
+
 __device__ __forceinline__ void bulk_commit() {
   asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
 }
@@ -494,7 +533,8 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
           }
           uint8_t *sa = base + s * cfg::STAGE;
           mbar_expect_tx(full + s, (uint32_t)cfg::STAGE);
-          tma_load_2d(sa, &tmA, kb * TC_BK, m0, full + s);
+          if (MODE == 0 && g.img.C) load_conv_box(sa, &tmA, g.img, kb * TC_BK, m0, full + s);
+          else tma_load_2d(sa, &tmA, kb * TC_BK, m0, full + s);
           tma_load_2d(sa + cfg::A_BYTES, &tmB, kb * TC_BK, n0, full + s);
         }
       }
@@ -586,8 +626,21 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
       ok = __all_sync(0xffffffffu, ready);
       if (!ok) break;
       tc_fence_after();
+      if (MODE == 4 && m0 < g.M) {
+        float v[16];
+        tc_ld16(tlane, v);
+        const int m = m0 + lane;
+#pragma unroll
+        for (int n = 0; n < 8; ++n)
+          if (m < g.M && n < g.N) {
+            float x = __fmul_rn(v[n], g.alpha);
+            if (g.bias) x += s_bias[n];
+            if (g.r) x += __bfloat162float(g.r[(int64_t)m * g.ldr + n]);
+            g.c32[(int64_t)m * g.ldc + n] = x;
+          }
+      }
 #pragma unroll 1
-      for (int j = 0; j < SLABS; ++j) {
+      for (int j = 0; j < (MODE == 4 ? 0 : SLABS); ++j) {
         const int c0 = n0 + CW * j;
         if (m0 >= g.M || c0 >= g.N) continue;
         const uint32_t b = seq % NB;
@@ -772,6 +825,7 @@ struct wg_args {
   int stages;
   float *part;
   int want_db;
+  conv_img img;       // of X
   uint32_t cols;      // tensor-memory columns
   uint32_t wait_limit;
   unsigned int *err;
@@ -842,9 +896,16 @@ __global__ void __launch_bounds__(WG_THREADS)
         uint8_t *sa = base + (size_t)s * stage_bytes;
         const int px = (int)(p0 + (int64_t)kb * WG_PX);
         mbar_expect_tx(full + s, stage_bytes);
-        for (int b = 0; b < a_boxes; ++b) tma_load_2d(sa + b * WG_BOX, &tmA, m0 + 64 * b, px, full + s);
-        for (int b = 0; b < g.nbx; ++b)
-          tma_load_2d(sa + (a_boxes + b) * WG_BOX, &tmB, n0 + 64 * b, px, full + s);
+        const bool ca = g.img.C && !g.a_is_dy, cb = g.img.C && g.a_is_dy;  // where X is
+        for (int b = 0; b < a_boxes; ++b) {
+          if (ca) load_conv_box(sa + b * WG_BOX, &tmA, g.img, m0 + 64 * b, px, full + s);
+          else tma_load_2d(sa + b * WG_BOX, &tmA, m0 + 64 * b, px, full + s);
+        }
+        for (int b = 0; b < g.nbx; ++b) {
+          uint8_t *d = sa + (a_boxes + b) * WG_BOX;
+          if (cb) load_conv_box(d, &tmB, g.img, n0 + 64 * b, px, full + s);
+          else tma_load_2d(d, &tmB, n0 + 64 * b, px, full + s);
+        }
       }
       if (!ok)
         for (int k = kb > g.stages ? kb - g.stages : 0; k < kb; ++k)
@@ -1041,6 +1102,39 @@ bool make_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t K, int64_
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+typedef CUresult (*encode_im2col_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
+                                     const cuuint64_t *, const cuuint64_t *, const int *,
+                                     const int *, cuuint32_t, cuuint32_t, const cuuint32_t *,
+                                     CUtensorMapInterleave, CUtensorMapSwizzle,
+                                     CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+encode_im2col_fn im2col_encoder() {
+  static const encode_im2col_fn fn = []() -> encode_im2col_fn {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeIm2col", &p, 12000,
+                                                     cudaEnableDefault, &q) == cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    return ok ? reinterpret_cast<encode_im2col_fn>(p) : nullptr;
+  }();
+  return fn;
+}
+
+// BF16 [B][H][W][C] as the neighbourhood matrix of a 3x3 convolution with zero
+// padding 1: boxes of `pixels` pixels by 64 channels.
+bool make_conv_map(CUtensorMap *map, const void *ptr, int B, int H, int W, int C, int pixels) {
+  encode_im2col_fn enc = im2col_encoder();
+  if (!enc) return false;
+  cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+  cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
+  int lower[2] = {-1, -1}, upper[2] = {-1, -1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(ptr), dims, strides, lower,
+             upper, 64, (cuuint32_t)pixels, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Polls of the kernel's main-loop waits (pe_nn_set_wait_limit).
 std::atomic<uint32_t> g_wait_limit{kWaitLimit};
 
@@ -1101,16 +1195,21 @@ int tc_sms() {
   return n;
 }
 
+// `conv`: A is the neighbourhood matrix of that image (batch images of it).
 template <int BN, int MODE, bool WIDE>
-pe_status launch_stream(const pe_gemm_args &g, cudaStream_t s) {
+pe_status launch_stream(const pe_gemm_args &g, cudaStream_t s, const conv_img *conv = nullptr,
+                        int batch = 0) {
   using cfg = st_cfg<BN, MODE, WIDE>;
   CUtensorMap ma, mb, mc, mx;
   const int64_t items = (int64_t)((g.M + TC_BM - 1) / TC_BM) * ((g.N + BN - 1) / BN);
   if (items >= (1ll << 30)) return PE_EUNSUPPORTED;  // (tile numbers are 32-bit)
-  if (!make_map(&ma, g.A, g.M, g.K, g.sam, TC_BM) || !make_map(&mb, g.B, g.N, g.K, g.sbn, BN) ||
-      !make_slab_map(&mc, g.C, g.M, g.N, g.ldc, cfg::COLS))
+  if (!(conv ? make_conv_map(&ma, g.A, batch, conv->H, conv->W, conv->C, TC_BM)
+             : make_map(&ma, g.A, g.M, g.K, g.sam, TC_BM)) ||
+      !make_map(&mb, g.B, g.N, g.K, g.sbn, BN) ||
+      (MODE != 4 && !make_slab_map(&mc, g.C, g.M, g.N, g.ldc, cfg::COLS)))
     return PE_EUNSUPPORTED;
-  if (MODE == 0) mx = mc;
+  if (MODE == 4) mx = mc = ma;  // (unused)
+  else if (MODE == 0) mx = mc;
   else if (!make_slab_map(&mx, MODE == 1 ? g.R : g.Z, g.M, g.N, MODE == 1 ? g.ldr : g.ldz,
                           cfg::COLS))
     return PE_EUNSUPPORTED;
@@ -1133,6 +1232,13 @@ pe_status launch_stream(const pe_gemm_args &g, cudaStream_t s) {
   a.items = (int)items;
   a.alpha = g.alpha;
   a.bias = g.bias;
+  if (conv) a.img = *conv;
+  if (MODE == 4) {
+    a.c32 = static_cast<float *>(g.C);
+    a.ldc = g.ldc;
+    a.r = g.R;
+    a.ldr = g.ldr;
+  }
   a.wait_limit = g_wait_limit.load();
   a.err = pe_err_word();
   const int most = 2 * tc_sms();  // two CTAs per SM
@@ -1144,12 +1250,13 @@ pe_status launch_stream(const pe_gemm_args &g, cudaStream_t s) {
 }
 
 // The streaming kernel's mode for these arguments, -1 when it does not apply:
-// a TMA store writes BF16 rows on 16-byte boundaries, so FP32 outputs (the
-// heads) and unaligned rows stay with the other kernel, as does an epilogue
+// a TMA store writes BF16 rows on 16-byte boundaries, so wider FP32 outputs and
+// unaligned rows stay with the other kernel, as does an epilogue
 // outside the four forms.  Where both apply the streaming kernel was the
 // faster one at every shape of the network (gradients of a 32 x 256^2 batch:
 // 21.4 -> 11.7 ms over its 113 contractions).
 int stream_mode(const pe_gemm_args &g) {
+  if (g.c_f32 && g.N <= 8 && g.gelu == 0 && g.beta == 0.0f && g.K < (1ll << 30)) return 4;
   if (g.c_f32 || !g.vec_c || g.K >= (1ll << 30) || (g.bias && g.N > ST_MAX_BIAS)) return -1;
   if (g.gelu == 0) return g.R ? 1 : 0;
   if (g.R) return -1;
@@ -1172,6 +1279,7 @@ pe_status launch_stream_mode(int mode, const pe_gemm_args &g, cudaStream_t s) {
 // one operand block is the whole of K and so a single ring stage makes room (GELU'
 // form, 64 channels, 524288 pixels: 174 -> 161 us before the packed range test).
 pe_status launch_stream_shape(int mode, const pe_gemm_args &g, cudaStream_t s) {
+  if (mode == 4) return launch_stream<32, 4, false>(g, s);
   if (g.N > 64 && g.K <= TC_BK && mode == 2) return launch_stream<128, 2, true>(g, s);
   if (g.N > 64 && g.K <= TC_BK && mode == 3) return launch_stream<128, 3, true>(g, s);
   if (g.N <= 32) return launch_stream_mode<32>(mode, g, s);
@@ -1256,15 +1364,30 @@ bool pe_wgrad_tc_eligible(const void *dY, int64_t ldy, const void *X, int64_t ld
          P < (1ll << 31) - 4096 && encoder();
 }
 
+bool pe_conv3_tc_sizes(int32_t B, int32_t H, int32_t W, int32_t C, int32_t N) {
+  return C % 64 == 0 && N > 64 && N <= ST_MAX_BIAS && N % 8 == 0 && W < 32768 && H < 32768 &&
+         (int64_t)B * H * W >= 16 && (int64_t)B * H * W < (1ll << 31) - 4096 && encoder() &&
+         im2col_encoder();
+}
+
+pe_status pe_conv3_tc(const pe_gemm_args &g, int32_t B, int32_t H, int32_t W, int32_t C,
+                      cudaStream_t s) {
+  const conv_img im = {C, W, H};
+  return launch_stream<128, 0, false>(g, s, &im, B);
+}
+
 size_t pe_wgrad_tc_workspace(int64_t P, int32_t N, int32_t K) {
   return (size_t)plan_wgrad(P, N, K).splits * ((size_t)N * K + N) * sizeof(float);
 }
 
 pe_status pe_wgrad_tc(const void *dY, int64_t ldy, const void *X, int64_t ldx, int64_t P, int32_t N,
-                      int32_t K, float *dW, float *db, float *part, cudaStream_t s) {
+                      int32_t K, float *dW, float *db, float *part, cudaStream_t s,
+                      const int32_t *conv) {
   const wg_plan w = plan_wgrad(P, N, K);
   CUtensorMap my, mx;
-  if (!make_map(&my, dY, P, N, ldy, WG_PX) || !make_map(&mx, X, P, K, ldx, WG_PX))
+  if (!make_map(&my, dY, P, N, ldy, WG_PX) ||
+      !(conv ? make_conv_map(&mx, X, conv[0], conv[1], conv[2], K / 9, WG_PX)
+             : make_map(&mx, X, P, K, ldx, WG_PX)))
     return PE_EUNSUPPORTED;
   static bool attr = false;
   if (!attr) {
@@ -1290,6 +1413,7 @@ pe_status pe_wgrad_tc(const void *dY, int64_t ldy, const void *X, int64_t ldx, i
   g.part = part;
   g.want_db = db != nullptr;
   g.cols = w.cols;
+  if (conv) g.img = conv_img{K / 9, conv[2], conv[1]};
   g.wait_limit = g_wait_limit.load();
   g.err = pe_err_word();
   const dim3 grid((unsigned)w.splits, (unsigned)(w.tiles_m * w.tiles_n));

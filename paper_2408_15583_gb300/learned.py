@@ -71,19 +71,23 @@ class Ops:
         self.gemm(P, N, K, x, ldx, 1, W, 1, K, out, ldo, bias=bias, R=R, ldr=ldr, Z=Z,
                   ldz=N, gelu=gelu)
 
+    def linear_dgrad(self, dy, W, dx, ldd, gelu_z=None):
+        """The data gradient reads W through its transpose, so both of its
+        operands are K-contiguous (the layout of the tensor-core kernel); with
+        gelu_z it is multiplied by GELU'(gelu_z) in the epilogue (the backward
+        of a GELU applied to this layer's input)."""
+        P, N = dy.shape
+        K = W.shape[1]
+        Wt = torch.empty(K, N, dtype=W.dtype, device=self.dev)
+        check(self.lib.pe_nn_transpose(_p(W), N, K, _p(Wt), self.s()), "pe_nn_transpose")
+        self.gemm(P, K, N, dy, N, 1, Wt, 1, N, dx, ldd, Z=gelu_z, ldz=K, dgelu=gelu_z is not None)
+
     def linear_bwd(self, dy, x, ldx, W, dx, ldd, dW, db, need_dx=True, gelu_z=None):
-        """dy [P,N] (BF16, contiguous), x [P,K] with row stride ldx.  The data
-        gradient reads W through its transpose, so both of its operands are
-        K-contiguous (the layout of the tensor-core kernel); with gelu_z it
-        is multiplied by GELU'(gelu_z) in the epilogue (the backward of a
-        GELU applied to this layer's input)."""
+        """dy [P,N] (BF16, contiguous), x [P,K] with row stride ldx."""
         P, N = dy.shape
         K = W.shape[1]
         if need_dx:
-            Wt = torch.empty(K, N, dtype=W.dtype, device=self.dev)
-            check(self.lib.pe_nn_transpose(_p(W), N, K, _p(Wt), self.s()), "pe_nn_transpose")
-            self.gemm(P, K, N, dy, N, 1, Wt, 1, N, dx, ldd, Z=gelu_z, ldz=K,
-                      dgelu=gelu_z is not None)
+            self.linear_dgrad(dy, W, dx, ldd, gelu_z)
         nb = self.lib.pe_nn_linear_wgrad_workspace(P, N, K)
         ws = self.ws(nb)
         check(self.lib.pe_nn_linear_wgrad(_p(dy), N, _p(x), ldx, P, N, K, _p(dW), _p(db), _p(ws),
@@ -98,6 +102,16 @@ class Ops:
     def im2col(self, x, B, H, W, Cc, col, backward=False):
         check(self.lib.pe_nn_im2col3(_p(x), B, H, W, Cc, _p(col), 1 if backward else 0, self.s()),
               "pe_nn_im2col3")
+
+    def conv3(self, x, w, b, B, H, W, Cin, Cout, y):
+        ws = self.ws(self.lib.pe_nn_conv3_workspace(B, H, W, Cin, Cout))
+        check(self.lib.pe_nn_conv3(_p(x), B, H, W, Cin, _p(w), _p(b), _p(y), Cout, _p(ws),
+                                   ws.numel(), self.s()), "pe_nn_conv3")
+
+    def conv3_wgrad(self, dy, x, B, H, W, Cin, Cout, dW, db):
+        ws = self.ws(self.lib.pe_nn_conv3_workspace(B, H, W, Cin, Cout))
+        check(self.lib.pe_nn_conv3_wgrad(_p(dy), _p(x), B, H, W, Cin, Cout, _p(dW), _p(db), _p(ws),
+                                         ws.numel(), self.s()), "pe_nn_conv3_wgrad")
 
     def dw(self, x, w, b, B, H, W, Cc, y):
         check(self.lib.pe_nn_dwconv7(_p(x), _p(w), _p(b), B, H, W, Cc, _p(y), self.s()),
@@ -234,25 +248,21 @@ class UNet:
         return dx
 
     def _conv3_fwd(self, x, name, B, H, W, Cin, Cout, tape):
-        P = B * H * W
-        col = self._empty(P, 9 * Cin)
-        self.ops.im2col(x, B, H, W, Cin, col)
-        y = self._empty(P, Cout)
-        self.ops.linear(col, 9 * Cin, self.pb(name + ".w"), self.pf(name + ".b"), y, Cout)
-        tape.append(("conv3", name, (col, B, H, W, Cin, Cout)))
+        y = self._empty(B * H * W, Cout)
+        self.ops.conv3(x, self.pb(name + ".w"), self.pf(name + ".b"), B, H, W, Cin, Cout, y)
+        tape.append(("conv3", name, (x, B, H, W, Cin, Cout)))
         return y
 
     def _conv3_bwd(self, dy, rec, need_dx=True):
-        name, (col, B, H, W, Cin, Cout) = rec
-        P = B * H * W
-        dcol = self._empty(P, 9 * Cin) if need_dx else None
-        self.ops.linear_bwd(dy, col, 9 * Cin, self.pb(name + ".w"), dcol, 9 * Cin,
-                            self.g(name + ".w").view(Cout, 9 * Cin), self.g(name + ".b"),
-                            need_dx=need_dx)
+        o = self.ops
+        name, (x, B, H, W, Cin, Cout) = rec
+        o.conv3_wgrad(dy, x, B, H, W, Cin, Cout, self.g(name + ".w"), self.g(name + ".b"))
         if not need_dx:
             return None
-        dx = self._empty(P, Cin)
-        self.ops.im2col(dcol, B, H, W, Cin, dx, backward=True)
+        dcol = self._empty(B * H * W, 9 * Cin)
+        o.linear_dgrad(dy, self.pb(name + ".w"), dcol, 9 * Cin)
+        dx = self._empty(B * H * W, Cin)
+        o.im2col(dcol, B, H, W, Cin, dx, backward=True)
         return dx
 
     # ------------------------------------------------------------------------

@@ -291,3 +291,39 @@ def test_thin_layer_gradients(P, K, N):
         assert torch.equal(dx, (dy.float() * W.float()).to(BF))
     else:
         assert rel(dx, dy.double() @ W.double()) < BF_TOL
+
+
+# ---- 3x3 convolution ----------------------------------------------------------------
+
+# channel counts gathered by the loads (multiples of 64) and not; images narrower
+# than a tile of pixels, rows that end inside one, several images to a tile, and
+# enough pixels for the unsplit kernel (128 outputs from 65536 pixels on)
+@pytest.mark.parametrize("B,H,W,Cin,Cout", [(1, 1, 1, 64, 128), (3, 5, 7, 64, 72), (2, 8, 8, 40, 96),
+                                            (5, 130, 101, 64, 128), (40, 41, 43, 128, 256)])
+def test_conv3(B, H, W, Cin, Cout):
+    from paper_2408_15583_gb300 import api
+    o, g = ops(), gen(B + H + W + Cin)
+    x = rnd(g, B, H, W, Cin).to(BF)
+    w = (rnd(g, Cout, 3, 3, Cin) / math.sqrt(9 * Cin)).to(BF)
+    b, dy = rnd(g, Cout), rnd(g, B * H * W, Cout).to(BF)
+    y = torch.empty(B * H * W, Cout, dtype=BF, device=DEV)
+    dW, db = torch.empty(Cout, 9 * Cin, device=DEV), torch.empty(Cout, device=DEV)
+    o.conv3(x, w, b, B, H, W, Cin, Cout, y)
+    o.conv3_wgrad(dy, x, B, H, W, Cin, Cout, dW, db)
+    api.stream_check()
+    xp = torch.nn.functional.pad(x.double(), (0, 0, 1, 1, 1, 1))
+    col = torch.cat([xp[:, i:i + H, j:j + W] for i in range(3) for j in range(3)], -1).view(-1, 9 * Cin)
+    assert rel(y, col @ w.double().view(Cout, -1).T + b.double()) < BF_TOL
+    assert rel(dW, dy.double().T @ col) < 1e-5 and rel(db, dy.double().sum(0)) < 1e-5
+
+
+@pytest.mark.parametrize("M,N,K", [(70000, 1, 64), (66000, 3, 64), (40963, 8, 72), (129, 2, 8)])
+def test_narrow_fp32_output(M, N, K):
+    from paper_2408_15583_gb300 import api
+    o, g = ops(), gen(M + N)
+    a, w, b = rnd(g, M, K).to(BF), rnd(g, N, K).to(BF), rnd(g, N)
+    y = torch.full((M + 1, N), 7.0, device=DEV)
+    o.gemm(M, N, K, a, K, 1, w, 1, K, y, N, bias=b)
+    api.stream_check()
+    ref = a.double() @ w.double().T + b.double()
+    assert float((y[:M].double() - ref).abs().max()) < 2e-5 * K ** 0.5 and bool((y[M] == 7.0).all())
