@@ -122,6 +122,34 @@ __global__ void scatter_points(const float *__restrict__ pos, int64_t n,
   }
 }
 
+// FP64 issues at 1/64 of the FP32 rate here, so sums that need more than FP32
+// run in pairs of floats (sum s and its error c): an addition's error by Knuth's
+// two-sum, a product's by one FMA (the compensated dot product of Ogita, Rump and
+// Oishi, as accurate as twice the working precision).
+struct pair_sum {
+  float s = 0.0f, c = 0.0f;
+  __device__ __forceinline__ void add(float v, float e) {  // v + e, |e| small against |v|
+    const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z)), e));
+    s = t;
+  }
+  // (xh + xl)(yh + yl) without xl yl
+  __device__ __forceinline__ void add_product(float xh, float xl, float yh, float yl) {
+    const float p = __fmul_rn(xh, yh);
+    add(p, fmaf(xh, yl, fmaf(xl, yh, fmaf(xh, yh, -p))));
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+// a - b = h + l exactly
+__device__ __forceinline__ void two_diff(float a, float b, float &h, float &l) {
+  h = __fsub_rn(a, b);
+  const float z = __fsub_rn(h, a);
+  l = __fsub_rn(__fsub_rn(a, __fsub_rn(h, z)), __fadd_rn(b, z));
+}
+// The range of squared distances in which no product or error term of the pair
+// arithmetic that matters leaves the normal floats; outside it FP64 is used.
+constexpr float kPairMin = 1e-20f, kPairMax = 1e30f;
+
 // Smallest-eigenvalue unit eigenvector of the symmetric 3x3 matrix
 // (a00 a01 a02; a11 a12; a22) by the trigonometric solution of the
 // characteristic cubic and the largest cross product of two rows of
@@ -169,12 +197,75 @@ __device__ void smallest_axis(double a00, double a01, double a02, double a11, do
   out[2] = best[2] * s;
 }
 
+// The same axis with FP32 where only a starting value is needed: the matrix is
+// scaled by an approximate 1 / p, the cubic's smallest root starts from the FP32
+// trigonometric solution (error about 1e-6) and takes two Newton steps in FP64,
+// and the length's reciprocal root one; all that is left in FP64 is what the
+// result's precision rests on (about 100 operations; the square roots, divisions,
+// arc cosine and cosine of the full solution take several times as many).  False
+// (and no result) where the two smallest eigenvalues are close, since Newton's
+// steps need the cubic's slope, and for matrices out of the floats' range.
+__device__ bool smallest_axis_newton(double a00, double a01, double a02, double a11, double a12,
+                                     double a22, double out[3]) {
+  const double q = (a00 + a11 + a22) * (1.0 / 3.0);
+  const double b00 = a00 - q, b11 = a11 - q, b22 = a22 - q;
+  float p2;
+  {
+    const float x = (float)b00, y = (float)b11, z = (float)b22, u = (float)a01, v = (float)a02,
+                w = (float)a12;
+    p2 = x * x + y * y + z * z + 2.0f * (u * u + v * v + w * w);
+  }
+  if (!(p2 > 1e-30f && p2 < 1e30f)) return false;
+  const double ip = (double)rsqrtf(p2 * (1.0f / 6.0f));
+  const double c00 = b00 * ip, c11 = b11 * ip, c22 = b22 * ip, c01 = a01 * ip, c02 = a02 * ip,
+               c12 = a12 * ip;
+  // det(C - x I) = -(x^3 - k x - d), k = 3 up to the scale's rounding
+  const double k = 0.5 * (c00 * c00 + c11 * c11 + c22 * c22) + c01 * c01 + c02 * c02 + c12 * c12;
+  const double d = c00 * (c11 * c22 - c12 * c12) - c01 * (c01 * c22 - c12 * c02) +
+                   c02 * (c01 * c12 - c11 * c02);
+  const float r = fminf(fmaxf(0.5f * (float)d, -1.0f), 1.0f);
+  const float x0 = 2.0f * cosf(acosf(r) * (1.0f / 3.0f) + 2.0943951f);  // + 2 pi / 3: smallest
+  const float slope = 3.0f * x0 * x0 - (float)k;
+  if (!(slope > 0.05f)) return false;
+  const double is = (double)__frcp_rn(slope);
+  double x = (double)x0;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) x -= ((x * x - k) * x - d) * is;
+  const double e00 = c00 - x, e11 = c11 - x, e22 = c22 - x;
+  // the largest cross product of two rows
+  double b[3] = {c01 * c12 - c02 * e11, c02 * c01 - e00 * c12, e00 * e11 - c01 * c01};  // 0 x 1
+  double bn = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
+  const double f[3] = {c01 * e22 - c02 * c12, c02 * c02 - e00 * e22, e00 * c12 - c01 * c02};  // 0 x 2
+  const double fn = f[0] * f[0] + f[1] * f[1] + f[2] * f[2];
+  const double h[3] = {e11 * e22 - c12 * c12, c12 * c02 - c01 * e22, c01 * c12 - e11 * c02};  // 1 x 2
+  const double hn = h[0] * h[0] + h[1] * h[1] + h[2] * h[2];
+  if (fn > bn) {
+    bn = fn;
+    b[0] = f[0];
+    b[1] = f[1];
+    b[2] = f[2];
+  }
+  if (hn > bn) {
+    bn = hn;
+    b[0] = h[0];
+    b[1] = h[1];
+    b[2] = h[2];
+  }
+  double s = (double)rsqrtf((float)bn);
+  s *= 1.5 - 0.5 * bn * s * s;
+  out[0] = b[0] * s;
+  out[1] = b[1] * s;
+  out[2] = b[2] * s;
+  return true;
+}
+
 struct knn_args {
   const float4 *pts;  // {x, y, z, index} in cell order
   int64_t n;
   const grid_info *gi;
   const uint32_t *offs;
   int K, k_r, k_n;
+  double inv_r, inv_n;  // 1 / k_r, 1 / k_n
   const float *ref;
   float *rad, *nrm;
   unsigned int *err;
@@ -213,14 +304,14 @@ __device__ __forceinline__ void for_runs(const uint32_t *__restrict__ offs, int 
 // the radius: the point itself is one of its zeros, whatever the order of ties.
 // The second scan, for the normal, collects the points nearer than the k_n-th
 // distance and, of those at it, the smallest indices, into shared memory; their
-// moments about the query point are then summed in FP64 by all lanes together.
+// moments about the query point are then summed by all lanes together, in pairs
+// of floats, and the axis found with as little FP64 as its precision needs.
 // The points are read as 16-byte records in cell order, a run per (x, y) column
 // of cells, and queries follow the same order, so a warp mostly reads the same
-// records.  (Lists of (distance, index) in local memory, insertion by a
-// data-dependent loop and 27 cells visited one by one left 13.6 of 32 lanes
-// active and took 2.35 ms for a million points, k_r = 8, k_n = 16; now 1.28 ms,
-// of which the FP64 sums and eigenvectors, at a 64th of the FP32 rate, are the
-// larger part: the radii alone take 0.3 of 0.75-1.1 ms.)
+// records.  A million points, k_r = 8, k_n = 16: 2.35 ms with lists of (distance,
+// index) in local memory, insertion by a data-dependent loop and 27 cells visited
+// one by one (13.6 of 32 lanes active); 1.28 ms with both scans as above and
+// moments, roots and eigenvectors in FP64, at a 64th of the FP32 rate; 0.68 ms now.
 template <int KT>
 __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
   extern __shared__ uint32_t s_list[];  // [k_n][kPtThreads]: positions in pts
@@ -276,11 +367,20 @@ __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
   if (A.rad) {
     // the first entry is the point's own zero; were it pushed out by more than
     // K coincident points, every entry would be zero
-    double sum = 0.0;
+    // (a root of d: its float r and the rest d - r^2, exact in one FMA, over 2 r)
+    pair_sum sum;
+    double tiny = 0.0;
 #pragma unroll
     for (int e = 1; e < KT; ++e)
-      if (e <= A.k_r) sum += sqrt((double)bd[e]);
-    A.rad[i] = (float)(sum / (double)A.k_r);
+      if (e <= A.k_r) {
+        if (bd[e] > kPairMin && bd[e] < kPairMax) {
+          const float r = __fsqrt_rn(bd[e]);
+          sum.add(r, __fdividef(fmaf(-r, r, bd[e]), 2.0f * r));
+        } else {
+          tiny += sqrt((double)bd[e]);
+        }
+      }
+    A.rad[i] = (float)((sum.value() + tiny) * A.inv_r);
   }
   if (A.nrm) {
     const int kn = A.k_n;
@@ -314,25 +414,53 @@ __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
         }
       }
     });
-    // moments about the query point: exact differences of floats in FP64
+    // moments about the query point, of exact differences
     double m[3] = {0.0, 0.0, 0.0};
     double a00 = 0, a01 = 0, a02 = 0, a11 = 0, a12 = 0, a22 = 0;
-    for (int k = 0; k < kn; ++k) {
-      const float4 p = __ldg(A.pts + list[k * kPtThreads]);
-      const double x = (double)p.x - (double)q.x, y = (double)p.y - (double)q.y,
-                   z = (double)p.z - (double)q.z;
-      m[0] += x;
-      m[1] += y;
-      m[2] += z;
-      a00 += x * x;
-      a01 += x * y;
-      a02 += x * z;
-      a11 += y * y;
-      a12 += y * z;
-      a22 += z * z;
+    if (tau > kPairMin && tau < kPairMax) {
+      pair_sum mx, my, mz, xx, xy, xz, yy, yz, zz;
+      for (int k = 0; k < kn; ++k) {
+        const float4 p = __ldg(A.pts + list[k * kPtThreads]);
+        float x, y, z, dx, dy, dz;
+        two_diff(p.x, q.x, x, dx);
+        two_diff(p.y, q.y, y, dy);
+        two_diff(p.z, q.z, z, dz);
+        mx.add(x, dx);
+        my.add(y, dy);
+        mz.add(z, dz);
+        xx.add_product(x, dx, x, dx);
+        xy.add_product(x, dx, y, dy);
+        xz.add_product(x, dx, z, dz);
+        yy.add_product(y, dy, y, dy);
+        yz.add_product(y, dy, z, dz);
+        zz.add_product(z, dz, z, dz);
+      }
+      m[0] = mx.value();
+      m[1] = my.value();
+      m[2] = mz.value();
+      a00 = xx.value();
+      a01 = xy.value();
+      a02 = xz.value();
+      a11 = yy.value();
+      a12 = yz.value();
+      a22 = zz.value();
+    } else {
+      for (int k = 0; k < kn; ++k) {
+        const float4 p = __ldg(A.pts + list[k * kPtThreads]);
+        const double x = (double)p.x - (double)q.x, y = (double)p.y - (double)q.y,
+                     z = (double)p.z - (double)q.z;
+        m[0] += x;
+        m[1] += y;
+        m[2] += z;
+        a00 += x * x;
+        a01 += x * y;
+        a02 += x * z;
+        a11 += y * y;
+        a12 += y * z;
+        a22 += z * z;
+      }
     }
-    const double inv = 1.0 / (double)kn;
-    const double mx = m[0] * inv, my = m[1] * inv, mz = m[2] * inv;
+    const double mx = m[0] * A.inv_n, my = m[1] * A.inv_n, mz = m[2] * A.inv_n;
     a00 -= m[0] * mx;
     a01 -= m[0] * my;
     a02 -= m[0] * mz;
@@ -340,7 +468,8 @@ __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
     a12 -= m[1] * mz;
     a22 -= m[2] * mz;
     double v[3];
-    smallest_axis(a00, a01, a02, a11, a12, a22, v);
+    if (!smallest_axis_newton(a00, a01, a02, a11, a12, a22, v))
+      smallest_axis(a00, a01, a02, a11, a12, a22, v);
     double w[3];
     if (A.ref) {
       for (int k = 0; k < 3; ++k) w[k] = (double)A.ref[3 * (int64_t)i + k];
@@ -497,6 +626,8 @@ extern "C" pe_status pe_point_attributes(const float *pos, int64_t n_points, int
   A.K = K;
   A.k_r = k_r;
   A.k_n = k_n;
+  A.inv_r = 1.0 / (double)(k_r > 0 ? k_r : 1);
+  A.inv_n = 1.0 / (double)(k_n > 0 ? k_n : 1);
   A.ref = ref_nrm;
   A.rad = radius;
   A.nrm = normal;

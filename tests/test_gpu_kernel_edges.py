@@ -327,3 +327,34 @@ def test_narrow_fp32_output(M, N, K):
     api.stream_check()
     ref = a.double() @ w.double().T + b.double()
     assert float((y[:M].double() - ref).abs().max()) < 2e-5 * K ** 0.5 and bool((y[M] == 7.0).all())
+
+
+# ---- surfel attributes ----------------------------------------------------------------
+
+# clouds inside and outside the range of the pair arithmetic, and shapes whose two
+# smallest axes are close (the full solution) or not.  The normal is rounded to
+# FP32, an angle of at most 1e-7 from the axis, and its own error adds less than as
+# much again, so n'An exceeds the smallest eigenvalue by at most (2e-7)^2 of the
+# largest; the radius is one rounding away, 2^-24.
+@pytest.mark.parametrize("scale", [1e-12, 1e-7, 1.0, 1e9, 1e16])
+@pytest.mark.parametrize("shape", [(1.0, 0.7, 0.05), (1.0, 0.02, 0.01), (1.0, 0.9, 0.8)])
+def test_point_attributes_scales(scale, shape):
+    import numpy as np
+    from paper_2408_15583_gb300 import api
+    rng, n, k_r, k_n = np.random.default_rng(7), 600, 8, 16
+    pos = (rng.standard_normal((n, 3)) * np.array(shape) * scale + 3.0 * scale).astype(np.float32)
+    rad, nrm = api.point_attributes(torch.tensor(pos, device=DEV), k_r, k_n, None, radius=True,
+                                    normal=True)
+    api.stream_check()
+    rad, nrm = rad.double().cpu().numpy(), nrm.double().cpu().numpy()
+    d = pos[:, None] - pos[None]
+    d2 = (d[..., 0] * d[..., 0] + d[..., 1] * d[..., 1]) + d[..., 2] * d[..., 2]
+    order = np.argsort(d2, axis=1, kind="stable")
+    for i in range(n):
+        r = np.sqrt(d2[i, order[i, 1:k_r + 1]].astype(np.float64)).mean()
+        x = pos[order[i, :k_n]].astype(np.float64) - pos[i].astype(np.float64)
+        x = (x - x.mean(0)) / scale
+        A = x.T @ x
+        lam = np.linalg.eigvalsh(A)
+        assert abs(rad[i] - r) <= 1.01 * 2.0 ** -24 * r
+        assert nrm[i] @ A @ nrm[i] / (nrm[i] @ nrm[i]) - lam[0] < 4.1e-14 * lam[2]
