@@ -203,63 +203,66 @@ __device__ uint32_t view_mask(const pe_geom_layout &L, pe_f3 o, pe_f3 d, float t
       tdel[k] = INFINITY;
     }
   }
-  int x0 = ix[0], x1 = ix[1], x2 = ix[2];
+  // the cell (x0, x1, x2) as x0 << 16 | x1 << 8 | x2: a step off the grid sets
+  // the guard bits 5 to 7 of its field (PE_VGRID = 32), by carry or borrow
+  static_assert(PE_VGRID == 32, "five bits per axis of the packed cell");
+  int P = ix[0] << 16 | ix[1] << 8 | ix[2];
   float m0 = tmax[0], m1 = tmax[1], m2 = tmax[2];
   const float d0 = tdel[0], d1 = tdel[1], d2 = tdel[2];
-  const int s0 = st[0], s1 = st[1], s2 = st[2];
+  const int e0 = st[0] * 65536, e1 = st[1] * 256, e2 = st[2];
+  auto cell_of = [](int p) { return (p >> 6 & 0x7c00) | (p >> 3 & 0x3e0) | (p & 0x1f); };
+  int cid = cell_of(P);
+  uint32_t b = __ldg(L.vmask + cid);
   float t_in = t0;
   bool ended = false;
-  for (int it = 0; it < 3 * n + 3; ++it) {
+  for (int it = 0; it < 3 * PE_VGRID + 3; ++it) {
     // the axis whose boundary comes first (ties as x < y < z order of the
     // comparisons: k = m0 < m1 ? (m0 < m2 ? 0 : 2) : (m1 < m2 ? 1 : 2))
-    const bool k0 = m0 < m1 && m0 < m2;
-    const bool k1 = !(m0 < m1) && m1 < m2;
-    const float t_out = k0 ? m0 : (k1 ? m1 : m2);
-    const int64_t cid = ((int64_t)x0 * n + x1) * n + x2;
-    uint32_t b = __ldg(L.vmask + cid) & ~outside;
-    float s_in = t_in, s_out = t_out;
+    const bool c01 = m0 < m1, k0 = c01 && m0 < m2, k1 = !c01 && m1 < m2;
+    const float t_out = fminf(fminf(m0, m1), m2);
+    // the next cell's bits are fetched before this cell's are looked at
+    const int Pn = P + (k0 ? e0 : (k1 ? e1 : e2));
+    const bool out = t_out > t1 || (Pn & 0xe0e0e0) != 0;
+    const int cn = cell_of(Pn);
+    uint32_t bn = 0;
+    if (!out) bn = __ldg(L.vmask + cn);
+    b &= ~outside;
     if (b) {
       // the cell's slab: the ray's stretch through the cell that lies inside
       // it, [s_in, s_out] (|hs + t hd| <= 1 in the slab's scaled heights);
       // a stretch outside the slab meets none of the cell's disks, so the
       // cell adds no view
+      float s_in = t_in, s_out = t_out;
       const float4 cs = __ldg(L.cslab + cid);
-      const float qx = fmaf(-((float)x0 + 0.5f), cell, oo[0]);
-      const float qy = fmaf(-((float)x1 + 0.5f), cell, oo[1]);
-      const float qz = fmaf(-((float)x2 + 0.5f), cell, oo[2]);
+      const float qx = fmaf(-((float)(P >> 16) + 0.5f), cell, oo[0]);
+      const float qy = fmaf(-((float)(P >> 8 & 0x1f) + 0.5f), cell, oo[1]);
+      const float qz = fmaf(-((float)(P & 0x1f) + 0.5f), cell, oo[2]);
       const float hs = fmaf(cs.x, qx, fmaf(cs.y, qy, fmaf(cs.z, qz, -cs.w)));
       const float hd = fmaf(cs.x, dd[0], fmaf(cs.y, dd[1], cs.z * dd[2]));
       const float r = __fdividef(1.0f, slab_dir(hd));
       const float ta = (-1.0f - hs) * r, tb = (1.0f - hs) * r;
       s_in = fmaxf(s_in, fminf(ta, tb));
       s_out = fminf(s_out, fmaxf(ta, tb));
-      if (!(s_in <= s_out)) b = 0u;
+      if (s_in <= s_out) {
+        for (uint32_t r = b; r; r &= r - 1) {
+          const int v = __ffs(r) - 1;
+          float2 &T = tv[v * stride];
+          if (!((m >> v) & 1u)) T.x = s_in;
+          T.y = s_out;
+        }
+        m |= b;
+      }
     }
-    for (uint32_t r = b; r; r &= r - 1) {
-      const int v = __ffs(r) - 1;
-      float2 &T = tv[v * stride];
-      if (!((m >> v) & 1u)) T.x = s_in;
-      T.y = s_out;
-    }
-    m |= b;
-    if (t_out > t1) {
+    if (out) {
       ended = true;
       break;
     }
-    if (k0) {
-      x0 += s0;
-      m0 = m0 + d0;
-    } else if (k1) {
-      x1 += s1;
-      m1 = m1 + d1;
-    } else {
-      x2 += s2;
-      m2 = m2 + d2;
-    }
-    if ((unsigned)x0 >= (unsigned)n || (unsigned)x1 >= (unsigned)n || (unsigned)x2 >= (unsigned)n) {
-      ended = true;
-      break;
-    }
+    if (k0) m0 += d0;
+    else if (k1) m1 += d1;
+    else m2 += d2;
+    P = Pn;
+    cid = cn;
+    b = bn;
     t_in = t_out;
   }
   if (!ended)  // cannot happen for a line through an n^3 grid; stay conservative
