@@ -285,6 +285,30 @@ __global__ void gemm_splitk_reduce(const pe_gemm_args g, int split) {
   }
 }
 
+// The same sums for at most eight splits (one per lane ty above, so they are
+// added in order), a thread taking eight columns of a row: 16-byte accesses and
+// no thread without a split.  16384 x 256, two splits: 134 us above, 11 us here.
+__global__ void __launch_bounds__(256) gemm_splitk_reduce8(const pe_gemm_args g, int split) {
+  const int64_t total = (int64_t)g.M * g.N;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; t < total;
+       t += (int64_t)gridDim.x * blockDim.x * 8) {
+    float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    for (int z = 0; z < split; ++z) {
+      const float4 *q = reinterpret_cast<const float4 *>(g.part + (int64_t)z * total + t);
+      const float4 a = __ldcs(q), b = __ldcs(q + 1);
+      v[0] += a.x;
+      v[1] += a.y;
+      v[2] += a.z;
+      v[3] += a.w;
+      v[4] += b.x;
+      v[5] += b.y;
+      v[6] += b.z;
+      v[7] += b.w;
+    }
+    pe_gemm_store8(g, (int)(t / g.N), (int)(t % g.N), v);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // 3x3 convolution helpers (NHWC, zero padding 1): col[p][(ky*3+kx)*C + c]
 // ---------------------------------------------------------------------------
@@ -495,8 +519,11 @@ __global__ void __launch_bounds__(DW_THREADS, 2)
 // for eight loads, split over two halves of the block by tap rows (28 sums
 // fit 128 registers; all 49 in one thread measured 264 us, the loads of its
 // 12 warps per SM in the open).  The block's positions are then added in
-// order.  64 channels, 32 x 128^2: 132 us against 203 us with a thread per tap
-// row, which read a pixel's dY and X for seven FMAs.
+// order.  The loads run four pixels ahead: a pixel's FMAs are far shorter than
+// its loads, and 16 warps per SM leave little else to cover them.  64 channels,
+// 32 x 128^2: 203 us with a thread per tap row, which read a pixel's dY and X for
+// seven FMAs, 127 us one pixel ahead, 101 us now; 32 channels, 32 x 256^2: 330 us
+// one pixel ahead, 212 us now.
 template <int K0, int NK, int CT>
 __device__ __forceinline__ void dw7_wgrad_rows(const uint32_t *__restrict__ X,
                                                const uint32_t *__restrict__ dY, int B, int H, int W,
@@ -526,17 +553,19 @@ __device__ __forceinline__ void dw7_wgrad_rows(const uint32_t *__restrict__ X,
       const int xx = xs + k - 3;
       win[k] = unpack2(xx >= 0 && xx < W ? __ldg(xr + (int64_t)xx * cp2) : 0u);
     }
-    uint32_t raw[NK + 1];  // the pixel's dY values and the window's new X, one pixel ahead
-    auto load_px = [&](int xx) {
+    // dY and the window's new X of the next D pixels (pixel x in slot x mod D)
+    constexpr int D = 4;
+    uint32_t raw[D][NK + 1];
+    auto load_px = [&](int j, int xx) {
 #pragma unroll
-      for (int k = 0; k < NK; ++k) raw[k] = xx < xe ? __ldg(gp[k] + (int64_t)xx * cp2) & gm[k] : 0u;
-      raw[NK] = xx < xe && xx + 3 < W ? __ldg(xr + (int64_t)(xx + 3) * cp2) : 0u;
+      for (int k = 0; k < NK; ++k) raw[j][k] = xx < xe ? __ldg(gp[k] + (int64_t)xx * cp2) & gm[k] : 0u;
+      raw[j][NK] = xx < xe && xx + 3 < W ? __ldg(xr + (int64_t)(xx + 3) * cp2) : 0u;
     };
     auto pixel = [&](int u, auto &&load_next) {
       float2 g[NK];
 #pragma unroll
-      for (int k = 0; k < NK; ++k) g[k] = unpack2(raw[k]);
-      win[(u + 6) % 8] = unpack2(raw[NK]);
+      for (int k = 0; k < NK; ++k) g[k] = unpack2(raw[u % D][k]);
+      win[(u + 6) % 8] = unpack2(raw[u % D][NK]);
       load_next();
       if (K0 <= 3 && 3 < K0 + NK) {
         accb.x += g[3 - K0 < NK ? 3 - K0 : 0].x;
@@ -548,26 +577,29 @@ __device__ __forceinline__ void dw7_wgrad_rows(const uint32_t *__restrict__ X,
         for (int kx = 0; kx < 7; ++kx)
           acc[k * 7 + kx] = __ffma2_rn(g[k], win[(u + kx) % 8], acc[k * 7 + kx]);
     };
-    load_px(xs);
+#pragma unroll
+    for (int j = 0; j < D; ++j) load_px(j, xs + j);
     int x = xs;
+    // every load in the stretch and the row (or read by no pixel, when these
+    // eight end the stretch): no checks
 #pragma unroll 1
-    for (; x + 8 <= xe && x + 11 < W; x += 8) {  // every load in the row: no checks
-      const uint32_t *xp = xr + (int64_t)(x + 4) * cp2;
+    for (; (x + 8 + D <= xe || x + 8 == xe) && x + 10 + D < W; x += 8) {
+      const uint32_t *xp = xr + (int64_t)(x + D + 3) * cp2;
       const uint32_t *gx[NK];
 #pragma unroll
-      for (int k = 0; k < NK; ++k) gx[k] = gp[k] + (int64_t)(x + 1) * cp2;
+      for (int k = 0; k < NK; ++k) gx[k] = gp[k] + (int64_t)(x + D) * cp2;
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         pixel(u, [&] {
 #pragma unroll
-          for (int k = 0; k < NK; ++k) raw[k] = __ldg(gx[k] + u * cp2) & gm[k];
-          raw[NK] = __ldg(xp + u * cp2);
+          for (int k = 0; k < NK; ++k) raw[u % D][k] = __ldg(gx[k] + u * cp2) & gm[k];
+          raw[u % D][NK] = __ldg(xp + u * cp2);
         });
     }
 #pragma unroll 1
     for (; x < xe; x += 8)  // (past the stretch: zeros)
 #pragma unroll
-      for (int u = 0; u < 8; ++u) pixel(u, [&] { load_px(x + u + 1); });
+      for (int u = 0; u < 8; ++u) pixel(u, [&] { load_px(u % D, x + u + D); });
   }
 }
 
@@ -1570,6 +1602,11 @@ extern "C" pe_status pe_nn_gemm(int32_t M, int32_t N, int64_t K, const void *A, 
   PE_TRY_LAUNCH("gemm_kernel");
   if (split > 1) {
     const int64_t total = (int64_t)M * N;
+    if (split <= 8 && N % 8 == 0 && al(ws)) {
+      gemm_splitk_reduce8<<<grid1(total / 8, 256), 256, 0, s>>>(g, (int)split);
+      PE_TRY_LAUNCH("gemm_splitk_reduce8");
+      return PE_OK;
+    }
     gemm_splitk_reduce<<<(unsigned)((total + 31) / 32), dim3(32, 8), 0, s>>>(g, (int)split);
     PE_TRY_LAUNCH("gemm_splitk_reduce");
   }
@@ -1912,6 +1949,180 @@ extern "C" pe_status pe_nn_linear_wgrad(const void *dY, int64_t ldy, const void 
   return pe_nn_colsum(dY, P, N, ldy, db, 0, ws, ws_bytes, stream);
 }
 
+// One input channel (the network's first layer): K = 9 is too short for a TMA
+// row.  Forward: a warp takes 16 pixels by 32 outputs, its lanes read the taps of
+// their mma.sync fragment from the image, and the products are those of
+// gemm_kernel on the neighbourhood matrix (one k-step of 16, taps 9..15 zero, and
+// one of zeros), so are the bits.  16 x 256^2 by 32: 126 us with the
+// matrix written, 39 us now (writing y takes 10; the taps' index arithmetic most of
+// the rest).
+namespace {
+struct stem_img {
+  const bf16 *x;
+  int W, H;
+  // tap (3 ky + kx) at pixel (px, py) of the image that starts at row0 rows
+  __device__ __forceinline__ uint32_t tap(int64_t p, int px, int py, int t) const {
+    const int dy = t / 3 - 1, dx = t % 3 - 1;
+    const bool in = (unsigned)(py + dy) < (unsigned)H && (unsigned)(px + dx) < (unsigned)W;
+    return in ? (uint32_t)__ldg(reinterpret_cast<const unsigned short *>(x) + p + dy * W + dx) : 0u;
+  }
+};
+
+__global__ void __launch_bounds__(256)
+    stem_fwd_kernel(const stem_img im, int64_t P, const bf16 *__restrict__ w,
+                    const float *__restrict__ bias, bf16 *__restrict__ y, int N) {
+  const int lane = threadIdx.x & 31, gq = lane >> 2, tq = lane & 3, n0 = blockIdx.y * 32;
+  uint32_t b[4][2];
+  float bs[8];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const unsigned short *r = reinterpret_cast<const unsigned short *>(w) + (int64_t)(n0 + 8 * j + gq) * 9;
+    b[j][0] = (uint32_t)r[2 * tq] | (uint32_t)r[2 * tq + 1] << 16;
+    b[j][1] = tq == 0 ? (uint32_t)r[8] : 0u;
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e) bs[e] = bias ? bias[n0 + 8 * tq + e] : 0.0f;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t m0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 16; m0 < P;
+       m0 += warps * 16) {
+    uint32_t a[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t p = m0 + gq + 8 * h;
+      if (p < P) {
+        const uint32_t q = (uint32_t)p / (uint32_t)im.W;  // (P < 2^31)
+        const int px = (int)((uint32_t)p - q * (uint32_t)im.W), py = (int)(q % (uint32_t)im.H);
+        a[h] = im.tap(p, px, py, 2 * tq) | im.tap(p, px, py, 2 * tq + 1) << 16;
+        if (tq == 0) a[2 + h] = im.tap(p, px, py, 8);
+      }
+    }
+    uint32_t out[2][4];  // [row half][8-column block]: this lane's two columns
+    float acc[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[j][e] = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        asm volatile(
+            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, "
+            "{%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+            : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
+            : "r"(k ? 0u : a[0]), "r"(k ? 0u : a[1]), "r"(k ? 0u : a[2]), "r"(k ? 0u : a[3]),
+              "r"(k ? 0u : b[j][0]), "r"(k ? 0u : b[j][1]));
+    }
+    // the four lanes of a row exchange their pairs of columns, so that each holds
+    // the eight columns from 8 tq on: lane tq keeps block tq of every partner
+    float v[2][8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {  // from lane tq ^ r, which sends its block (its tq) ^ r
+        const int send = tq ^ r;
+        float s0 = acc[0][2 * h], s1 = acc[0][2 * h + 1];
+#pragma unroll
+        for (int j = 1; j < 4; ++j) {
+          s0 = send == j ? acc[j][2 * h] : s0;
+          s1 = send == j ? acc[j][2 * h + 1] : s1;
+        }
+        s0 = __shfl_xor_sync(0xffffffffu, s0, r);
+        s1 = __shfl_xor_sync(0xffffffffu, s1, r);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (e == send) {
+            v[h][2 * e] = s0;
+            v[h][2 * e + 1] = s1;
+          }
+      }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t p = m0 + gq + 8 * h;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        float c0 = v[h][2 * e], c1 = v[h][2 * e + 1];
+        if (bias) {
+          c0 += bs[2 * e];
+          c1 += bs[2 * e + 1];
+        }
+        const bf162 o = __floats2bfloat162_rn(c0, c1);
+        out[h][e] = *reinterpret_cast<const uint32_t *>(&o);
+      }
+      if (p < P)
+        *reinterpret_cast<uint4 *>(y + p * N + n0 + 8 * tq) =
+            make_uint4(out[h][0], out[h][1], out[h][2], out[h][3]);
+    }
+  }
+}
+
+// Weight and bias gradient of that layer: dW[n][tap] = sum_p dY[p][n] x[p + tap].
+// LPP = N / 8 lanes per pixel, eight outputs and 8 x 9 + 8 sums each, so dY is
+// read once in 16-byte accesses and x through the caches.  part[block][9 N + N].
+// 32 x 256^2 by 32: 361 us with the matrix written and a 128-row mma.sync tile of
+// which 32 rows held outputs, 117 us now.
+constexpr int kStemBlocks = 304, STEM_THREADS = 256;
+template <int LPP>
+__global__ void __launch_bounds__(STEM_THREADS, 2)
+    stem_wgrad_kernel(const stem_img im, int64_t P, const bf16 *__restrict__ dY,
+                      float *__restrict__ part) {
+  constexpr int PPW = 32 / LPP, N = 8 * LPP, WARPS = STEM_THREADS / 32;
+  __shared__ float s_sum[WARPS][10 * 8][LPP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = lane % LPP;
+  float acc[10][8];
+#pragma unroll
+  for (int t = 0; t < 10; ++t)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[t][e] = 0.0f;
+  const int64_t step = (int64_t)gridDim.x * WARPS * PPW;
+  for (int64_t p = ((int64_t)blockIdx.x * WARPS + warp) * PPW + lane / LPP; p < P; p += step) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4 *>(dY + p * N) + c);
+    const uint32_t wd[4] = {u.x, u.y, u.z, u.w};
+    const uint32_t q = (uint32_t)p / (uint32_t)im.W;
+    const int px = (int)((uint32_t)p - q * (uint32_t)im.W), py = (int)(q % (uint32_t)im.H);
+    float xt[9], d[8];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) xt[t] = __uint_as_float(im.tap(p, px, py, t) << 16);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      d[2 * e] = __uint_as_float(wd[e] << 16);
+      d[2 * e + 1] = __uint_as_float(wd[e] & 0xffff0000u);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+#pragma unroll
+      for (int t = 0; t < 9; ++t) acc[t][e] = fmaf(d[e], xt[t], acc[t][e]);
+      acc[9][e] += d[e];
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < 10; ++t)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+#pragma unroll
+      for (int o = 16; o >= LPP; o >>= 1) acc[t][e] += __shfl_xor_sync(0xffffffffu, acc[t][e], o);
+      if (lane < LPP) s_sum[warp][t * 8 + e][lane] = acc[t][e];
+    }
+  __syncthreads();
+  float *out = part + (size_t)blockIdx.x * (10 * N);
+  for (int o = threadIdx.x; o < 10 * N; o += STEM_THREADS) {
+    const int n = o < 9 * N ? o / 9 : o - 9 * N, t = o < 9 * N ? o % 9 : 9;
+    float v = 0.0f;
+    for (int k = 0; k < WARPS; ++k) v += s_sum[k][t * 8 + n % 8][n / 8];
+    out[o] = v;
+  }
+}
+
+template <int LPP>
+pe_status launch_stem_wgrad(const stem_img &im, int64_t P, const bf16 *dY, float *dW, float *db,
+                            float *part, cudaStream_t s) {
+  constexpr int per_block = STEM_THREADS / LPP;
+  const int64_t need = (P + per_block - 1) / per_block;
+  const int blocks = (int)(need < kStemBlocks ? need : kStemBlocks);
+  stem_wgrad_kernel<LPP><<<blocks, STEM_THREADS, 0, s>>>(im, P, dY, part);
+  PE_TRY_LAUNCH("stem_wgrad_kernel");
+  return pe_wgrad_reduce(part, blocks, 72 * LPP, 80 * LPP, dW, db, s);
+}
+}  // namespace
+
 // 3x3 convolution, y = col(x) w^T + bias with col the neighbourhood matrix.  The
 // TMA loads gather it from the image itself (im2col mode) where its channels
 // fill whole 64-channel blocks and the contraction would run unsplit on the
@@ -1956,7 +2167,9 @@ extern "C" size_t pe_nn_conv3_workspace(int32_t B, int32_t H, int32_t W, int32_t
   const size_t col = ((size_t)P * 9 * Cin * sizeof(bf16) + 255) & ~size_t(255);
   const size_t a = pe_nn_gemm_workspace((int32_t)P, Cout, 9 * (int64_t)Cin),
                b = pe_nn_linear_wgrad_workspace(P, Cout, 9 * Cin);
-  return (conv_gathered(B, H, W, Cin, Cout) ? 0 : col) + (a > b ? a : b) + 512;
+  const size_t c = Cin == 1 ? (size_t)kStemBlocks * 10 * Cout * sizeof(float) : 0;
+  const size_t most = a > b ? (a > c ? a : c) : (b > c ? b : c);
+  return (conv_gathered(B, H, W, Cin, Cout) ? 0 : col) + most + 512;
 }
 
 // col in the workspace (256-byte aligned), with the rest of it after col.
@@ -1990,6 +2203,14 @@ extern "C" pe_status pe_nn_conv3(const void *x, int32_t B, int32_t H, int32_t W,
       return pe_fail(PE_EINVAL, "pe_nn_conv3: pointers on 16-byte boundaries");
     return pe_conv3_tc(g, B, H, W, Cin, s);
   }
+  if (Cin == 1 && Cout % 32 == 0 && Cout / 32 <= 65535 && (reinterpret_cast<uintptr_t>(y) & 15) == 0) {
+    const stem_img im = {g.A, W, H};
+    const int64_t P = (int64_t)B * H * W;
+    stem_fwd_kernel<<<dim3(grid1((P + 127) / 128, 1, 8), Cout / 32), 256, 0, s>>>(
+        im, P, g.B, bias, static_cast<bf16 *>(y), Cout);
+    PE_TRY_LAUNCH("stem_fwd_kernel");
+    return PE_OK;
+  }
   pe_status st;
   char *rest;
   size_t rest_bytes;
@@ -2014,6 +2235,20 @@ extern "C" pe_status pe_nn_conv3_wgrad(const void *dY, const void *x, int32_t B,
     const int32_t img[3] = {B, H, W};
     return pe_wgrad_tc(dY, Cout, x, 9 * (int64_t)Cin, P, Cout, 9 * Cin, dW, db,
                        static_cast<float *>(ws), s, img);
+  }
+  if (Cin == 1 && (reinterpret_cast<uintptr_t>(dY) & 15) == 0 &&
+      (reinterpret_cast<uintptr_t>(ws) & 3) == 0) {
+    const stem_img im = {static_cast<const bf16 *>(x), W, H};
+    const bf16 *d = static_cast<const bf16 *>(dY);
+    float *part = static_cast<float *>(ws);
+    switch (Cout) {
+      case 8: return launch_stem_wgrad<1>(im, P, d, dW, db, part, s);
+      case 16: return launch_stem_wgrad<2>(im, P, d, dW, db, part, s);
+      case 32: return launch_stem_wgrad<4>(im, P, d, dW, db, part, s);
+      case 64: return launch_stem_wgrad<8>(im, P, d, dW, db, part, s);
+      case 128: return launch_stem_wgrad<16>(im, P, d, dW, db, part, s);
+      default: break;
+    }
   }
   pe_status st;
   char *rest;

@@ -358,3 +358,40 @@ def test_point_attributes_scales(scale, shape):
         lam = np.linalg.eigvalsh(A)
         assert abs(rad[i] - r) <= 1.01 * 2.0 ** -24 * r
         assert nrm[i] @ A @ nrm[i] / (nrm[i] @ nrm[i]) - lam[0] < 4.1e-14 * lam[2]
+
+
+# one input channel: tiles of 16 pixels that end inside a row, an image or a warp's
+# share; the forward products are those of the general contraction, bit for bit
+@pytest.mark.parametrize("B,H,W,Cout", [(1, 1, 1, 32), (2, 3, 5, 64), (3, 17, 19, 32), (1, 260, 517, 32),
+                                        (2, 9, 16, 8), (1, 40, 33, 128), (1, 12, 11, 40)])
+def test_conv3_one_channel(B, H, W, Cout):
+    from paper_2408_15583_gb300 import api
+    o, g, P = ops(), gen(B + H + W + Cout), B * H * W
+    x, b, dy = rnd(g, B, H, W, 1).to(BF), rnd(g, Cout), rnd(g, P, Cout).to(BF)
+    w = (rnd(g, Cout, 9) / 3).to(BF)
+    y, z, col = (torch.empty(P, n, dtype=BF, device=DEV) for n in (Cout, Cout, 9))
+    dW, db = torch.empty(Cout, 9, device=DEV), torch.empty(Cout, device=DEV)
+    o.conv3(x, w, b, B, H, W, 1, Cout, y)
+    o.conv3_wgrad(dy, x, B, H, W, 1, Cout, dW, db)
+    o.im2col(x, B, H, W, 1, col)
+    o.gemm(P, Cout, 9, col, 9, 1, w, 1, 9, z, Cout, bias=b)
+    api.stream_check()
+    xp = torch.nn.functional.pad(x.double(), (0, 0, 1, 1, 1, 1))
+    ref = torch.cat([xp[:, i:i + H, j:j + W] for i in range(3) for j in range(3)], -1).view(-1, 9)
+    assert torch.equal(col.double(), ref) and torch.equal(y, z)
+    assert rel(dW, dy.double().T @ ref) < 1e-5 and rel(db, dy.double().sum(0)) < 1e-5
+
+
+# two to eight splits and more, with and without a residual, whole rows of eight and not
+@pytest.mark.parametrize("M,N,K", [(16384, 256, 1024), (1000, 64, 2304), (640, 136, 1100), (257, 36, 600)])
+def test_split_contraction(M, N, K):
+    from paper_2408_15583_gb300 import api
+    o, g = ops(), gen(M + N)
+    a, w = rnd(g, M, K).to(BF), (rnd(g, N, K) / math.sqrt(K)).to(BF)
+    b, r = rnd(g, N), rnd(g, M, N).to(BF)
+    y, y32 = torch.empty(M, N, dtype=BF, device=DEV), torch.empty(M, N, device=DEV)
+    o.gemm(M, N, K, a, K, 1, w, 1, K, y, N, bias=b, R=r, ldr=N)
+    o.gemm(M, N, K, a, K, 1, w, 1, K, y32, N)
+    api.stream_check()
+    ref = a.double() @ w.double().T
+    assert rel(y32, ref) < 1e-5 and rel(y, ref + b.double() + r.double()) < BF_TOL
