@@ -240,6 +240,16 @@ __device__ __forceinline__ void add_term(float kf, float khi, float klo, float a
   }
 }
 
+// Chunk of the i-th block of a group: the middle ones first, the rims last.
+// The target lies in the middle of its screen, so the rim's chunks hold few
+// rays or none, and the blocks that finish a launch are short ones (in slot
+// order the last group's middle chunks ran on a part of the SMs: 4 x 509^2 rays,
+// 33 uneven frequencies 166 -> 153 us; the sphere's sweep 20.42 -> 19.93 ms).
+__device__ __forceinline__ int middle_out(int i, int n) {
+  const int mid = (n - 1) / 2;
+  return i & 1 ? mid + (i + 1) / 2 : mid - i / 2;
+}
+
 __global__ void __launch_bounds__(kPoThreads, 4)
     po_kernel(const pe_hits h, const __grid_constant__ po_consts C, double *__restrict__ part) {
   // per staged ray: {au, av, dh, dl}, {Va.e1, Va.e2, Vc.e1, Vc.e2}: two
@@ -248,8 +258,8 @@ __global__ void __launch_bounds__(kPoThreads, 4)
   __shared__ int s_warp[kPoThreads / 32];
   __shared__ double s_red[kPoThreads][kAcc];
 
-  const int g = blockIdx.y;  // group within this launch
-  const int chunk = blockIdx.x;
+  const int g = blockIdx.x;  // group within this launch
+  const int chunk = middle_out(blockIdx.y, C.n_chunks);
   const int tid = threadIdx.x;
   const int FL = C.fl, RL = kPoThreads / FL;
   const int lane_f = tid % FL, lane_r = tid / FL;
@@ -498,8 +508,8 @@ __global__ void __launch_bounds__(kPoThreads, PE_PO_MINB)
   static_assert(sizeof(double) * kAcc <= 6 * sizeof(float4), "the sums fit the rays' memory");
   __shared__ int s_warp[2 * (kPoThreads / 32)];
 
-  const int g = blockIdx.y;
-  const int chunk = blockIdx.x;
+  const int g = blockIdx.x;
+  const int chunk = middle_out(blockIdx.y, C.n_chunks);
   const int tid = threadIdx.x;
   const int FL = C.fl, RL = kPoThreads / FL;  // frequency-chunk lanes, ray lanes
   const int lane_f = tid % FL, lane_r = tid / FL;
@@ -894,7 +904,7 @@ pe_status pe_launch_po(const pe_hits &h, int32_t n_groups, int64_t rpg, const fl
       const double df = nf > 1 ? (freqs[fb + nf - 1] - freqs[fb]) / (double)(nf - 1) : 0.0;
       for (int f = 0; uniform && f < nf; ++f)
         uniform = fabs(freqs[fb + f] - (freqs[fb] + f * df)) <= 1e-9 * fabs(freqs[fb + f]);
-      dim3 grid(C.n_chunks, ng);
+      dim3 grid(ng, C.n_chunks);
       if (uniform) {
         const double dkr = df / c0;
         C.dkhi = (float)dkr;
