@@ -17,6 +17,7 @@ from __future__ import annotations
 
 import ctypes as C
 from dataclasses import dataclass
+from functools import cached_property
 from typing import Dict, List
 
 import numpy as np
@@ -32,7 +33,7 @@ LN_EPS = 1e-6
 
 
 def _p(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 class Ops:
@@ -45,8 +46,13 @@ class Ops:
         self._ws = torch.empty(0, dtype=torch.uint8, device=self.dev)
 
     def s(self):
-        st = self.stream if self.stream is not None else torch.cuda.current_stream(self.dev)
-        return C.c_void_p(st.cuda_stream)
+        if self.stream is not None:
+            return self.stream.cuda_stream
+        if self.dev.type != "cuda":
+            return torch.cuda.current_stream(self.dev).cuda_stream      # (raises)
+        # the handle alone: a Stream object takes ten times as long to make
+        i = self.dev.index
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
 
     def ws(self, nbytes):
         if self._ws.numel() < nbytes:
@@ -158,7 +164,7 @@ class Slot:
     off: int
     shape: tuple
 
-    @property
+    @cached_property
     def n(self):
         return int(np.prod(self.shape))
 
@@ -187,6 +193,7 @@ class UNet:
         self.grad = torch.zeros(off, dtype=F32, device=self.dev)
         self.m = torch.zeros(off, dtype=F32, device=self.dev)
         self.v = torch.zeros(off, dtype=F32, device=self.dev)
+        self._views = {}
         self.ops.to_bf16(self.master, self.mirror)
         self.t = 0
 
@@ -203,6 +210,28 @@ class UNet:
         s = self.slots[name]
         return self.grad[s.off:s.off + s.n].view(s.shape)
 
+    # The same views for the layer calls, made once per buffer: slicing and
+    # shaping one takes about 8 us, and a pass asks for 186 (forward) or 280
+    # (backward) of them, more than the GPU needs for the layers of a small
+    # batch.  A buffer that was replaced gets new ones (the views keep theirs
+    # alive, so an equal address is the same memory).
+    def _views_of(self, which, make):
+        flat = getattr(self, which)
+        at, views = self._views.get(which, (None, None))
+        if at != flat.data_ptr():
+            views = {k: make(k) for k in self.slots}
+            self._views[which] = (flat.data_ptr(), views)
+        return views
+
+    def _pf(self, name):
+        return self._views_of("master", self.pf)[name]
+
+    def _pb(self, name):
+        return self._views_of("mirror", self.pb)[name]
+
+    def _g(self, name):
+        return self._views_of("grad", self.g)[name]
+
     def params_numpy(self):
         host = self.master.cpu().numpy()
         return {k: host[s.off:s.off + s.n].reshape(s.shape).copy() for k, s in self.slots.items()}
@@ -215,16 +244,16 @@ class UNet:
         o = self.ops
         P = B * H * W
         a = self._empty(P, Cc)
-        o.dw(x, self.pf(p + ".dw.w"), self.pf(p + ".dw.b"), B, H, W, Cc, a)
+        o.dw(x, self._pf(p + ".dw.w"), self._pf(p + ".dw.b"), B, H, W, Cc, a)
         bn = self._empty(P, Cc)
         mean = self._empty(P, dtype=F32)
         rstd = self._empty(P, dtype=F32)
-        o.ln(a, self.pf(p + ".ln.g"), self.pf(p + ".ln.b"), P, Cc, bn, mean, rstd)
+        o.ln(a, self._pf(p + ".ln.g"), self._pf(p + ".ln.b"), P, Cc, bn, mean, rstd)
         z1 = self._empty(P, 4 * Cc)
         h = self._empty(P, 4 * Cc)
-        o.linear(bn, Cc, self.pb(p + ".pw1.w"), self.pf(p + ".pw1.b"), h, 4 * Cc, Z=z1, gelu=True)
+        o.linear(bn, Cc, self._pb(p + ".pw1.w"), self._pf(p + ".pw1.b"), h, 4 * Cc, Z=z1, gelu=True)
         y = self._empty(P, Cc)
-        o.linear(h, 4 * Cc, self.pb(p + ".pw2.w"), self.pf(p + ".pw2.b"), y, Cc, R=x, ldr=Cc)
+        o.linear(h, 4 * Cc, self._pb(p + ".pw2.w"), self._pf(p + ".pw2.b"), y, Cc, R=x, ldr=Cc)
         tape.append(("block", p, (x, a, bn, mean, rstd, z1, h, B, H, W, Cc)))
         return y
 
@@ -233,34 +262,34 @@ class UNet:
         p, (x, a, bn, mean, rstd, z1, h, B, H, W, Cc) = rec
         P = B * H * W
         dz1 = self._empty(P, 4 * Cc)          # dL/dz1 = (dy . W2) * GELU'(z1), one GEMM
-        o.linear_bwd(dy, h, 4 * Cc, self.pb(p + ".pw2.w"), dz1, 4 * Cc, self.g(p + ".pw2.w"),
-                     self.g(p + ".pw2.b"), gelu_z=z1)
+        o.linear_bwd(dy, h, 4 * Cc, self._pb(p + ".pw2.w"), dz1, 4 * Cc, self._g(p + ".pw2.w"),
+                     self._g(p + ".pw2.b"), gelu_z=z1)
         dbn = self._empty(P, Cc)
-        o.linear_bwd(dz1, bn, Cc, self.pb(p + ".pw1.w"), dbn, Cc, self.g(p + ".pw1.w"),
-                     self.g(p + ".pw1.b"))
+        o.linear_bwd(dz1, bn, Cc, self._pb(p + ".pw1.w"), dbn, Cc, self._g(p + ".pw1.w"),
+                     self._g(p + ".pw1.b"))
         da = self._empty(P, Cc)
-        o.ln_bwd(dbn, a, self.pf(p + ".ln.g"), mean, rstd, P, Cc, da, self.g(p + ".ln.g"),
-                 self.g(p + ".ln.b"))
+        o.ln_bwd(dbn, a, self._pf(p + ".ln.g"), mean, rstd, P, Cc, da, self._g(p + ".ln.g"),
+                 self._g(p + ".ln.b"))
         dx = self._empty(P, Cc)
-        o.dw_bwd(x, da, self.pf(p + ".dw.w"), B, H, W, Cc, dx, self.g(p + ".dw.w"),
-                 self.g(p + ".dw.b"))
+        o.dw_bwd(x, da, self._pf(p + ".dw.w"), B, H, W, Cc, dx, self._g(p + ".dw.w"),
+                 self._g(p + ".dw.b"))
         o.copy(dy, Cc, 0, dx, Cc, 0, P, Cc, accumulate=True)      # residual
         return dx
 
     def _conv3_fwd(self, x, name, B, H, W, Cin, Cout, tape):
         y = self._empty(B * H * W, Cout)
-        self.ops.conv3(x, self.pb(name + ".w"), self.pf(name + ".b"), B, H, W, Cin, Cout, y)
+        self.ops.conv3(x, self._pb(name + ".w"), self._pf(name + ".b"), B, H, W, Cin, Cout, y)
         tape.append(("conv3", name, (x, B, H, W, Cin, Cout)))
         return y
 
     def _conv3_bwd(self, dy, rec, need_dx=True):
         o = self.ops
         name, (x, B, H, W, Cin, Cout) = rec
-        o.conv3_wgrad(dy, x, B, H, W, Cin, Cout, self.g(name + ".w"), self.g(name + ".b"))
+        o.conv3_wgrad(dy, x, B, H, W, Cin, Cout, self._g(name + ".w"), self._g(name + ".b"))
         if not need_dx:
             return None
         dcol = self._empty(B * H * W, 9 * Cin)
-        o.linear_dgrad(dy, self.pb(name + ".w"), dcol, 9 * Cin)
+        o.linear_dgrad(dy, self._pb(name + ".w"), dcol, 9 * Cin)
         dx = self._empty(B * H * W, Cin)
         o.im2col(dcol, B, H, W, Cin, dx, backward=True)
         return dx
@@ -284,7 +313,7 @@ class UNet:
                 o.maxpool(y, B, h, w, c[lvl - 1], pooled, arg)
                 h, w = h // 2, w // 2
                 y2 = self._empty(B * h * w, c[lvl])
-                o.linear(pooled, c[lvl - 1], self.pb(f"down{lvl}.w"), self.pf(f"down{lvl}.b"), y2,
+                o.linear(pooled, c[lvl - 1], self._pb(f"down{lvl}.w"), self._pf(f"down{lvl}.b"), y2,
                          c[lvl])
                 tape.append(("down", lvl, (pooled, arg, B, h, w)))
                 y = y2
@@ -304,13 +333,13 @@ class UNet:
                 o.shuffle(up, B, hh, ww, c[lvl], cat, 2 * c[lvl], 0)
                 o.copy(skips[lvl], c[lvl], 0, cat, 2 * c[lvl], c[lvl], cat.shape[0], c[lvl])
                 fu = self._empty(cat.shape[0], c[lvl])
-                o.linear(cat, 2 * c[lvl], self.pb(f"{head}.fuse{lvl}.w"),
-                         self.pf(f"{head}.fuse{lvl}.b"), fu, c[lvl])
+                o.linear(cat, 2 * c[lvl], self._pb(f"{head}.fuse{lvl}.w"),
+                         self._pf(f"{head}.fuse{lvl}.b"), fu, c[lvl])
                 dt.append(("fuse", lvl, (cat, B, dims[lvl][0], dims[lvl][1], hh, ww)))
                 u = self._block_fwd(fu, f"{head}.blk{lvl}", B, dims[lvl][0], dims[lvl][1], c[lvl], dt)
             out = self._empty(B * H * W, nout, dtype=F32)
             # the depth head refines the coarse input: correction + input
-            o.linear(u, c[0], self.pb(f"{head}.head.w"), self.pf(f"{head}.head.b"), out, nout,
+            o.linear(u, c[0], self._pb(f"{head}.head.w"), self._pf(f"{head}.head.b"), out, nout,
                      R=x if head == "depth" else None, ldr=1)
             dt.append(("head", head, (u,)))
             outs[head] = out if nout > 1 else out.view(-1)
@@ -332,8 +361,8 @@ class UNet:
             o.to_bf16(g32.contiguous(), gb)
             (_, _, (u,)) = dt[-1]
             du = self._empty(u.shape[0], c[0])
-            o.linear_bwd(gb, u, c[0], self.pb(f"{head}.head.w"), du, c[0],
-                         self.g(f"{head}.head.w"), self.g(f"{head}.head.b"))
+            o.linear_bwd(gb, u, c[0], self._pb(f"{head}.head.w"), du, c[0],
+                         self._g(f"{head}.head.w"), self._g(f"{head}.head.b"))
             i = len(dt) - 2
             for lvl in range(0, self.L - 1):
                 # records in reverse: block, fuse, conv3 (up)
@@ -344,8 +373,8 @@ class UNet:
                 assert kind == "fuse"
                 P2 = cat.shape[0]
                 dcat = self._empty(P2, 2 * c[lvl])
-                o.linear_bwd(dfu, cat, 2 * c[lvl], self.pb(f"{head}.fuse{lvl}.w"), dcat, 2 * c[lvl],
-                             self.g(f"{head}.fuse{lvl}.w"), self.g(f"{head}.fuse{lvl}.b"))
+                o.linear_bwd(dfu, cat, 2 * c[lvl], self._pb(f"{head}.fuse{lvl}.w"), dcat, 2 * c[lvl],
+                             self._g(f"{head}.fuse{lvl}.w"), self._g(f"{head}.fuse{lvl}.b"))
                 o.copy(dcat, 2 * c[lvl], c[lvl], dskip[lvl], c[lvl], 0, P2, c[lvl], accumulate=True)
                 dup = self._empty(B * hh * ww, 4 * c[lvl])
                 o.shuffle(dcat, B, hh, ww, c[lvl], dup, 2 * c[lvl], 0, backward=True)
@@ -368,8 +397,8 @@ class UNet:
                 kind, _, (pooled, arg, _, h, w) = enc[i]
                 assert kind == "down"
                 dpool = self._empty(pooled.shape[0], c[lvl - 1])
-                o.linear_bwd(dy, pooled, c[lvl - 1], self.pb(f"down{lvl}.w"), dpool, c[lvl - 1],
-                             self.g(f"down{lvl}.w"), self.g(f"down{lvl}.b"))
+                o.linear_bwd(dy, pooled, c[lvl - 1], self._pb(f"down{lvl}.w"), dpool, c[lvl - 1],
+                             self._g(f"down{lvl}.w"), self._g(f"down{lvl}.b"))
                 dfull = self._empty(B * 2 * h * 2 * w, c[lvl - 1])
                 o.maxpool(dpool, B, 2 * h, 2 * w, c[lvl - 1], dfull, arg, backward=True)
                 o.copy(dfull, c[lvl - 1], 0, dskip[lvl - 1], c[lvl - 1], 0, dfull.shape[0],

@@ -395,3 +395,34 @@ def test_split_contraction(M, N, K):
     api.stream_check()
     ref = a.double() @ w.double().T
     assert rel(y32, ref) < 1e-5 and rel(y, ref + b.double() + r.double()) < BF_TOL
+
+
+# ---- the network's parameter views ---------------------------------------------
+
+# the layer calls' views belong to the buffers: a network whose buffers were
+# replaced computes with the new ones, and so does one updated in place
+@pytest.mark.parametrize("how", ["replaced", "in place"])
+def test_parameter_views_follow_their_buffers(how):
+    import scenes
+    from paper_2408_15583_gb300.learned import UNet
+    widths, blocks, H = (8, 8), (1, 1), 16
+    a, b = (UNet(scenes.unet_init(seed, widths, blocks), widths, blocks, DEV) for seed in (1, 2))
+    x = rnd(gen(3), H * H).to(BF)
+
+    def step(net):
+        outs, tape = net.forward(x, 1, H, H)
+        net.backward(tape, {k: torch.ones_like(v) for k, v in outs.items()})
+        return outs, net.grad.clone()
+
+    before, _ = step(a)
+    want, want_grad = step(b)
+    for name in ("master", "mirror", "grad"):
+        if how == "replaced":
+            setattr(a, name, getattr(b, name).clone())
+        else:
+            getattr(a, name).copy_(getattr(b, name))
+    got, got_grad = step(a)
+    assert not torch.equal(before["depth"], want["depth"])
+    for k in want:
+        assert torch.equal(got[k], want[k])
+    assert torch.equal(got_grad, want_grad)
