@@ -215,22 +215,25 @@ class UNet:
     # (backward) of them, more than the GPU needs for the layers of a small
     # batch.  A buffer that was replaced gets new ones (the views keep theirs
     # alive, so an equal address is the same memory).
-    def _views_of(self, which, make):
+    def _view_of(self, which, make, name):
         flat = getattr(self, which)
         at, views = self._views.get(which, (None, None))
         if at != flat.data_ptr():
-            views = {k: make(k) for k in self.slots}
+            views = {}
             self._views[which] = (flat.data_ptr(), views)
-        return views
+        t = views.get(name)
+        if t is None:
+            t = views[name] = make(name)
+        return t
 
     def _pf(self, name):
-        return self._views_of("master", self.pf)[name]
+        return self._view_of("master", self.pf, name)
 
     def _pb(self, name):
-        return self._views_of("mirror", self.pb)[name]
+        return self._view_of("mirror", self.pb, name)
 
     def _g(self, name):
-        return self._views_of("grad", self.g)[name]
+        return self._view_of("grad", self.g, name)
 
     def params_numpy(self):
         host = self.master.cpu().numpy()
