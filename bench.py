@@ -358,24 +358,24 @@ MARCH_BYTES_PER_HIT = 76
 # DRAM bytes (read + write) per bounce query of march_kernel from one ncu
 # capture of the sweep's march on a smaller case (one 8-angle batch of the
 # sphere workload through pe_rcs_sweep; profiles/march_kernel_sphere_batch.md:
-# 91.1 MB over 6,332,964 queries), valid only for the sources it was taken on
+# 90.3 MB over 6,332,964 queries), valid only for the sources it was taken on
 # (their SHA-256 prefixes); scaled to a full launch by the number of queries.
-_SWEEP_SOURCES = {"include/pointemray.h": "867cc444e32855cc",
+_SWEEP_SOURCES = {"include/pointemray.h": "394d762d844f8b7d",
                   "paper_2408_15583_gb300/csrc/pe_internal.cuh": "2dc3ec4e588ae1ce",
                   "paper_2408_15583_gb300/csrc/sweep.cu": "9f2bcf7b228eaa30"}
-MARCH_NCU_TRAFFIC = {"bytes_per_query": 14.39,
+MARCH_NCU_TRAFFIC = {"bytes_per_query": 14.26,
                      "sources": dict(_SWEEP_SOURCES, **{
-                         "paper_2408_15583_gb300/csrc/trace.cu": "04fbdf628ec696d9",
-                         "paper_2408_15583_gb300/csrc/aggregate.cu": "a2f21815ee049028"})}
+                         "paper_2408_15583_gb300/csrc/trace.cu": "68196cfec0db80a6",
+                         "paper_2408_15583_gb300/csrc/aggregate.cu": "5329920b92b9c858"})}
 
 # DRAM bytes (read + write) per ray slot of po_rot_kernel from one ncu capture
 # of the sweep's field sum on one 8-angle sphere batch
-# (profiles/po_kernel_sphere_batch.md: 115.9 MB over 8 x 1024^2 slots), valid
+# (profiles/po_kernel_sphere_batch.md: 115.3 MB over 8 x 1024^2 slots), valid
 # for the sources it was taken on; scaled to a full launch by its slots
 # (angles x W x H).
-PO_NCU_TRAFFIC = {"bytes_per_slot": 13.81,
+PO_NCU_TRAFFIC = {"bytes_per_slot": 13.74,
                   "sources": dict(_SWEEP_SOURCES, **{
-                      "paper_2408_15583_gb300/csrc/po.cu": "4eb889207db41b89"})}
+                      "paper_2408_15583_gb300/csrc/po.cu": "1d87c1fb0c3a98f5"})}
 
 
 def _traffic_valid(rec):

@@ -483,13 +483,13 @@ __device__ __forceinline__ float rev_phase(float khi, float klo, float dhi, floa
 }
 
 // Two frequencies share every packed FP32 instruction (FFMA2 and FMUL2, the
-// same roundings as one at a time: the sums keep their bits).  That halves
-// the instructions of the larger part of a term; the price is that what a ray brings to both frequencies
-// lies twice in shared memory, two and a half more 16-byte broadcast loads per
-// ray and thread against 16 FMAs saved.  518M -> 428M warp instructions for 8
-// angles of 1024^2 rays at 64 frequencies, but the FMA pipe's
-// work stays: 6 x 500^2 rays at 33
-// frequencies 142 -> 137 us, the sphere's sweep 20.55 -> 20.42 ms.
+// same roundings as one at a time: the sums keep their bits).  That halves the
+// instructions of the larger part of a term; the price is that what a ray
+// brings to both frequencies lies twice in shared memory, two and a half more
+// 16-byte broadcast loads per ray and thread against 16 FMAs saved.  518M ->
+// 428M warp instructions for 8 angles of 1024^2 rays at 64 frequencies, but
+// the FMA pipe's work stays: 6 x 500^2 rays at 33 frequencies 142 -> 137 us,
+// the sphere's sweep 20.55 -> 20.42 ms.
 template <int FT, bool SMC>
 __global__ void __launch_bounds__(kPoThreads, PE_PO_MINB)
     po_rot_kernel(const pe_hits h, const __grid_constant__ po_consts C, double *__restrict__ part) {

@@ -451,7 +451,7 @@ class GraphedUNet:
     forward pass alone.  Each call copies its inputs into the captured
     buffers and replays: the same kernels in the same order as the eager
     calls, so the results are the same bit for bit, without the host's
-    per-layer launch work (about 1,260 launches per training step) between
+    per-layer launch work (about 500 launches per training step) between
     the kernels.  Captured once per shape, at the first call (after one eager
     warm-up pass that sizes the workspaces)."""
 
