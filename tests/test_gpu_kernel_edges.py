@@ -426,3 +426,48 @@ def test_parameter_views_follow_their_buffers(how):
     for k in want:
         assert torch.equal(got[k], want[k])
     assert torch.equal(got_grad, want_grad)
+
+
+# ---- Canny hysteresis over its tiles --------------------------------------------
+
+# a weak depth step along a serpentine corridor, strong at its start only, on
+# screens around the 64-pixel tiles: the edge follows the corridor through several
+# tiles and passes, and the splats equal the oracle's bit for bit
+@pytest.mark.parametrize("n", [8, 63, 64, 65, 129, 200])
+def test_canny_edge_followed_over_tiles(n):
+    import numpy as np
+    import oracle
+    from paper_2408_15583_gb300 import api
+    from paper_2408_15583_gb300._lib import PeParams
+    frame = ([0.0, 0.0, 5.0], [1.0, 0.0, 0.0], [0.0, 1.0, 0.0], [0.0, 0.0, -1.0])
+    view = oracle.View(*(np.array(a) for a in frame), pitch=0.125, W=n, H=n)
+    lane = np.zeros((n, n), bool)
+    for k, r in enumerate(range(3, n - 6, 14)):
+        lane[r:r + 6, 4:n - 4] = True
+        lane[r:r + 20, (n - 10 if k % 2 == 0 else 4):][:, :6] = True
+    lane[n - 3:] = False
+    start = lane & (np.arange(n)[:, None] < 9) & (np.arange(n)[None] < 12)
+    nrm = np.tile([0.0, 0.0, 1.0], (n * n, 1))
+
+    def splats(depth):
+        g = oracle.Gfb(depth=depth.ravel(), idx=np.zeros(n * n, np.int64), nrm=nrm, view=view, pix=None)
+        fp = oracle.FuseParams(tau=3.0, bmin=np.array([-16.0, -16.0, -16.0]), inv_vox=8.0, G=256,
+                               edge_mode=1)
+        want = oracle.aggregate([g], fp, "fp32")
+        nd = torch.from_numpy(np.concatenate([nrm, depth.reshape(-1, 1)], 1).astype(np.float32)).to(DEV)
+        prm = PeParams(eps=0.125, overlap_r=0.125, edge_tau=3.0, fuse_grid=256,
+                       bbox_min=(-16.0, -16.0, -16.0), inv_voxel=8.0, edge_mode=1)
+        geom = api.aggregate_views([api.view_from_struct(*frame, 0.125, n, n)], nd,
+                                   torch.ones(n * n, dtype=torch.uint8, device=DEV), prm)
+        cr, _ = geom.planes()
+        cr = cr.cpu().numpy()
+        ids = np.flatnonzero(cr[:, 3] > 0)
+        assert np.array_equal(ids, want.id)
+        assert np.array_equal(cr[ids, :3].astype(np.float64), want.c)
+        return ids
+
+    weak = 5.0 + 0.875 * lane
+    alone = splats(weak)
+    followed = splats(np.where(start, 7.0, weak))
+    if n >= 63:     # far more pixels become edges than the strong start's own rim
+        assert len(alone) - len(followed) > 4 * n
