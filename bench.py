@@ -366,7 +366,7 @@ _SWEEP_SOURCES = {"include/pointemray.h": "394d762d844f8b7d",
 MARCH_NCU_TRAFFIC = {"bytes_per_query": 14.26,
                      "sources": dict(_SWEEP_SOURCES, **{
                          "paper_2408_15583_gb300/csrc/trace.cu": "68196cfec0db80a6",
-                         "paper_2408_15583_gb300/csrc/aggregate.cu": "b8c25fb1c6a781b5"})}
+                         "paper_2408_15583_gb300/csrc/aggregate.cu": "fdf6326359cdb8e2"})}
 
 # DRAM bytes (read + write) per ray slot of po_rot_kernel from one ncu capture
 # of the sweep's field sum on one 8-angle sphere batch

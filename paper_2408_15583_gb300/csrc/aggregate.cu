@@ -126,8 +126,8 @@ __global__ void canny_nms_kernel(const __grid_constant__ pe_geom_layout L,
 // updates (pixels only rise).  A launch is bound by its latency, and an edge
 // advances a tile per pass where it advanced a pixel: 8 views of 384^2 of the
 // noisy composite took 96 passes, 661 us, and 12 synchronisations; their geometry
-// now takes 832 us where it took 1526.  Tiles of 64^2 hold whole edges of most screens and still give every SM
-// a block at 8 views of 384^2; a tile without a weak pixel ends after its loads.
+// now takes 832 us where it took 1526.  Tiles of 64^2 still give every SM a block
+// at 8 views of 384^2; a tile without a weak pixel ends after its loads.
 constexpr int kHystTile = 64, kHystThreads = 256;
 
 __global__ void __launch_bounds__(kHystThreads)
