@@ -324,6 +324,14 @@ __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
   const int c[3] = {cell_1d(g, q.x, 0), cell_1d(g, q.y, 1), cell_1d(g, q.z, 2)};
   const float qq[3] = {q.x, q.y, q.z};
   const int K = A.K;
+  // A NaN coordinate makes NaN of every distance it enters, and a NaN enters no
+  // list: such a point has no neighbours and is nobody's.
+  if (q.x != q.x || q.y != q.y || q.z != q.z) {
+    if (A.rad) A.rad[i] = NAN;
+    if (A.nrm)
+      for (int k = 0; k < 3; ++k) A.nrm[3 * (int64_t)i + k] = NAN;
+    return;
+  }
   float bd[KT];
 #pragma unroll
   for (int k = 0; k < KT; ++k) bd[k] = INFINITY;
@@ -364,7 +372,19 @@ __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
     pe_raise(A.err, PE_ERR_OVERFLOW);
     return;
   }
-  if (A.rad) {
+  // (an entry that no distance took is infinite, like a distance that overflows)
+  bool full = true;
+  if (A.rad && !(at(A.k_r) < INFINITY)) {
+    uint32_t found = 0;
+    for_runs(A.offs, G, c, 0, s, [&](uint32_t b, uint32_t e) {
+      for (uint32_t m = b; m < e; ++m) found += d2_pts(q, __ldg(A.pts + m)) >= 0.0f;
+    });
+    // (an infinite coordinate is at a NaN distance from itself)
+    full = found >= (uint32_t)A.k_r + (d2_pts(q, q) == 0.0f);
+  }
+  if (!full) {
+    A.rad[i] = NAN;
+  } else if (A.rad) {
     // the first entry is the point's own zero; were it pushed out by more than
     // K coincident points, every entry would be zero
     // (a root of d: its float r and the rest d - r^2, exact in one FMA, over 2 r)
@@ -414,6 +434,10 @@ __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
         }
       }
     });
+    if (n_lt != below || n_eq != kn) {  // fewer than k_n distances in the whole cloud
+      for (int k = 0; k < 3; ++k) A.nrm[3 * (int64_t)i + k] = NAN;
+      return;
+    }
     // moments about the query point, of exact differences
     double m[3] = {0.0, 0.0, 0.0};
     double a00 = 0, a01 = 0, a02 = 0, a11 = 0, a12 = 0, a22 = 0;

@@ -112,3 +112,44 @@ def test_argument_errors():
         api.point_attributes(p, 8, 16)            # fewer points than neighbours
     with pytest.raises(RuntimeError):
         api.point_attributes(torch.zeros(100, 3, device=DEV), 8, 40)   # k_n > 32
+
+
+@pytest.mark.parametrize("k_r,k_n", [(8, 16), (31, 32), (4, 3)])
+def test_nan_points_have_no_neighbours(k_r, k_n):
+    """A point with a NaN coordinate gets NaN and is nobody's neighbour: the other
+    points' radii are those of the cloud without it, their normals too (one FP32
+    rounding of a unit vector's component, 2^-24, and as much for the order of
+    the sums).  3000 and 3005 points take the same grid."""
+    rng = np.random.default_rng(k_r + k_n)
+    clean = rng.random((3000, 3)).astype(np.float32)
+    bad = np.sort(rng.choice(3005, 5, replace=False))
+    pos = np.zeros((3005, 3), np.float32)
+    good = np.setdiff1d(np.arange(3005), bad)
+    pos[good] = clean
+    pos[bad] = rng.random((5, 3)).astype(np.float32)
+    for row, axes in zip(bad, ([0], [1], [2], [0, 1], [0, 1, 2])):
+        pos[row, axes] = np.nan
+    r, n = _gpu(pos, k_r, k_n)
+    rc, nc = _gpu(clean, k_r, k_n)
+    assert np.isnan(r[bad]).all() and np.isnan(n[bad]).all()
+    assert np.array_equal(r[good], rc)
+    assert np.abs(n[good] - nc).max() <= 2.0 ** -23
+
+
+# 40 points of which all but `finite` are NaN: a point's normal needs k_n = 16
+# points, its radius k_r = 8 others
+@pytest.mark.parametrize("finite", [1, 8, 9, 15, 16])
+def test_too_few_points_besides_nan(finite):
+    rng = np.random.default_rng(finite)
+    pos = np.full((40, 3), np.nan, np.float32)
+    keep = np.sort(rng.choice(40, finite, replace=False))
+    pos[keep] = rng.random((finite, 3)).astype(np.float32)
+    r, n = _gpu(pos, 8, 16)
+    rest = np.setdiff1d(np.arange(40), keep)
+    assert np.isnan(r[rest]).all() and np.isnan(n[rest]).all()
+    if finite >= 9:
+        idx, d2 = oracle.knn(pos[keep], 9)
+        assert np.array_equal(r[keep], oracle.knn_radius(idx, d2, np.arange(finite), 8))
+    else:
+        assert np.isnan(r[keep]).all()
+    assert np.isnan(n).all() if finite < 16 else np.isfinite(n[keep]).all()
