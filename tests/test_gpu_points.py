@@ -153,3 +153,24 @@ def test_too_few_points_besides_nan(finite):
     else:
         assert np.isnan(r[keep]).all()
     assert np.isnan(n).all() if finite < 16 else np.isfinite(n[keep]).all()
+
+
+# neighbourhoods whose two smallest axes coincide (collinear, lattice, coincident
+# points), where the last bit of a sum picks the axis, and ordinary ones; many
+# points to a cell
+@pytest.mark.parametrize("name", ["line", "lattice", "coincident", "cube", "octar"])
+def test_the_same_call_gives_the_same_bits(name):
+    rng = np.random.default_rng(5)
+    pos = {
+        "line": lambda: np.outer(rng.random(20000), [0.3, 0.5, 0.8]),
+        "lattice": lambda: np.stack(np.meshgrid(*[np.arange(27) * 0.1] * 3), -1).reshape(-1, 3),
+        "coincident": lambda: np.repeat(rng.random((400, 3)), 40, axis=0),
+        "cube": lambda: rng.random((20000, 3)),
+        "octar": lambda: scenes.octar(20000, 2.0, seed=3).pos,
+    }[name]().astype(np.float32)
+    pos = rng.permutation(pos)
+    first = _gpu(pos, 8, 16)
+    for _ in range(6):
+        again = _gpu(pos, 8, 16)
+        for a, b in zip(first, again):
+            assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
