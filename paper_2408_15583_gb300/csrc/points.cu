@@ -127,7 +127,7 @@ __global__ void scatter_points(const float *__restrict__ pos, int64_t n,
 // The records with the points of a cell by index, so that what is added up in
 // this order (the moments of a normal) is the same on every run: a thread per
 // point counts the smaller indices of its cell.  A million points, about 36 to a
-// cell: 16 us of the 836 for radii and normals.
+// cell: 16 us of the 860 for radii and normals.
 __global__ void sort_cells(const float *__restrict__ pos, int64_t n,
                            const uint32_t *__restrict__ cell_of, const uint32_t *__restrict__ offs,
                            const uint32_t *__restrict__ idx, float4 *__restrict__ pts) {
@@ -285,6 +285,7 @@ struct knn_args {
   const uint32_t *offs;
   int K, k_r, k_n;
   double inv_r, inv_n;  // 1 / k_r, 1 / k_n
+  uint32_t err_r;       // bound of the error of k_r roots added in pairs, in 2^-53 of the sum
   const float *ref;
   float *rad, *nrm;
   unsigned int *err;
@@ -332,7 +333,8 @@ __device__ __forceinline__ void for_runs(const uint32_t *__restrict__ offs, int 
 // one by one (13.6 of 32 lanes active); 1.28 ms with both scans as above and
 // moments, roots and eigenvectors in FP64, at a 64th of the FP32 rate; 0.68 ms now.
 template <int KT>
-__global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
+__global__ void __launch_bounds__(kPtThreads, KT <= 16 ? 8 : (KT <= 24 ? 7 : 6))
+    knn_kernel(const knn_args A) {
   extern __shared__ uint32_t s_list[];  // [k_n][kPtThreads]: positions in pts
   const grid_info g = *A.gi;
   const int G = g.G;
@@ -408,18 +410,32 @@ __global__ void __launch_bounds__(kPtThreads) knn_kernel(const knn_args A) {
     // K coincident points, every entry would be zero
     // (a root of d: its float r and the rest d - r^2, exact in one FMA, over 2 r)
     pair_sum sum;
-    double tiny = 0.0;
+    bool in_range = true;
 #pragma unroll
     for (int e = 1; e < KT; ++e)
       if (e <= A.k_r) {
         if (bd[e] > kPairMin && bd[e] < kPairMax) {
           const float r = __fsqrt_rn(bd[e]);
           sum.add(r, __fdividef(fmaf(-r, r, bd[e]), 2.0f * r));
-        } else {
-          tiny += sqrt((double)bd[e]);
+        } else if (bd[e] != 0.0f) {
+          in_range = false;
         }
       }
-    A.rad[i] = (float)((sum.value() + tiny) * A.inv_r);
+    // Unless a boundary between two floats lies within the pair's error of the
+    // mean, the FP64 mean rounds to the same float; else (for one point in 40000
+    // at k_r = 8) FP64 decides.  A float takes 24 of the mean's 53 bits: a
+    // boundary is where the other 29 are one half.
+    const double mean = sum.value() * A.inv_r;
+    float rad = (float)mean;
+    const uint32_t rest = (uint32_t)__double2loint(mean) & 0x1fffffffu;
+    if (!in_range || rest - 0x10000000u + A.err_r <= 2u * A.err_r) {
+      double total = 0.0;
+#pragma unroll
+      for (int e = 1; e < KT; ++e)
+        if (e <= A.k_r) total += sqrt((double)bd[e]);
+      rad = (float)(total / (double)A.k_r);
+    }
+    A.rad[i] = rad;
   }
   if (A.nrm) {
     const int kn = A.k_n;
@@ -680,6 +696,9 @@ extern "C" pe_status pe_point_attributes(const float *pos, int64_t n_points, int
   A.k_n = k_n;
   A.inv_r = 1.0 / (double)(k_r > 0 ? k_r : 1);
   A.inv_n = 1.0 / (double)(k_n > 0 ? k_n : 1);
+  // k_r corrections, each summed with roundings of at most 3 k_r 2^-48 of the sum;
+  // a root's own correction errs by at most 2^-46 of it; 2^-48 = 2^5 2^-53
+  A.err_r = (uint32_t)((3 * k_r * k_r + 8) << 5);
   A.ref = ref_nrm;
   A.rad = radius;
   A.nrm = normal;

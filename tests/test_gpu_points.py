@@ -174,3 +174,39 @@ def test_the_same_call_gives_the_same_bits(name):
         again = _gpu(pos, 8, 16)
         for a, b in zip(first, again):
             assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
+
+
+# little-endian floats: neighbours' distances from the origin along an axis, found
+# by search, whose mean lies within 2^-44 of a boundary between two floats
+_NEAR_A_ROUNDING_BOUNDARY = [
+    "4519983e0f4da63e700af53e87132e3fe268843fc5278c3fd87b9f3f1f9db93f",
+    "ea1f083f38ec113fd3f61e3fd6542a3f6ca43a3f41d9603f3d7c913f65d4d43f",
+    "bc86b53ee0e3b63e6a60e73ec6f9643f20086e3fc6b38c3fa635913f25caa53f",
+    "003f8b3eb073a83e2a50d53e56fb003fb3ac1e3f12514f3faaae8f3fec7ed13f",
+    "c410933eb69b0d3f7d15123f4d5b1c3f38dc2c3f32ff353fb49a6a3f7a1eae3f",
+    "ffea8c3e72ca323ff3746f3f62f8863f287c933ff00d983f5a729a3f1cfebc3f",
+    "79abbe3ed647103f42b1393fd9ad533f2a787c3fb6bd913f5325943f9148b83f",
+    "052dd33eb2d1223f6e2f353fa096553fd695743f9d95813fce17923fff9dd73f",
+    "ec58883ec0888e3e260aa83ea33fbe3eec7cce3e0d8edd3e95e8e93e974cfd3e392cff3efe64013f"
+    "7e26093f24992a3f7d1b333fdd53363f9b2d433ff4f7433f557e4e3fb1d94e3fe07a513fd3c2623f"
+    "8b88723f1471753fc900773f269d843f56668c3fee708e3f2aa98e3fa118953f1e16993fbd039d3f"
+    "3f81a13f",
+    "4847863e14d48d3e82d2a73ec312bb3e8977c53e4cafd23e5e36053f45481b3fd2d8213f3815243f"
+    "28b0263f65262f3f09f03a3fc6b63c3fb173493f2f715d3f49d8633f9cba643f3fd5683f16f9683f"
+    "1b606b3f490a783f8684783fba98843f74cb873fbbc88d3f7ce78e3f442a903f4f6f923f60319b3f"
+    "6062d43f",
+]
+
+
+@pytest.mark.parametrize("case", range(len(_NEAR_A_ROUNDING_BOUNDARY)))
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_radius_is_the_rounded_fp64_mean(case, axis):
+    x = np.frombuffer(bytes.fromhex(_NEAR_A_ROUNDING_BOUNDARY[case]), "<f4")
+    k = len(x)
+    pos = np.zeros((k + 1, 3), np.float32)
+    pos[1:, axis] = x
+    idx, d2 = oracle.knn(pos, k + 1)
+    from paper_2408_15583_gb300 import api
+    r, _ = api.point_attributes(torch.from_numpy(pos).to(DEV), k, 3, normal=False)
+    api.stream_check()
+    assert np.array_equal(r.cpu().numpy(), oracle.knn_radius(idx, d2, np.arange(k + 1), k))
