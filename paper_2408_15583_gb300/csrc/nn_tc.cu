@@ -517,10 +517,10 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
+  uint32_t c = 0;  // k-blocks whose loads the producer issued
   if (warp == 0) {
     if (lane == 0) {
       // ---- producer ------------------------------------------------------
-      uint32_t c = 0;  // k-blocks issued
       bool ok = true;
       for (int it = blockIdx.x; ok && it < g.items; it += gridDim.x) {
         const int m0 = (it / g.tiles_n) * TC_BM, n0 = (it % g.tiles_n) * BN;
@@ -538,14 +538,11 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
           tma_load_2d(sa + cfg::A_BYTES, &tmB, kb * TC_BK, n0, full + s);
         }
       }
-      if (!ok)  // copies in flight land before the shared memory is released
-        for (uint32_t k = c > (uint32_t)S ? c - S : 0; k < c; ++k)
-          mbar_wait(full + k % S, (k / S) & 1u);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       // ---- product issuer ------------------------------------------------
-      uint32_t c = 0, i = 0;
+      uint32_t i = 0;
       bool ok = true;
       for (int it = blockIdx.x; ok && it < g.items; it += gridDim.x, ++i) {
         const uint32_t st = i & 1u;
@@ -572,10 +569,6 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
           tc_commit(empty + s);
         }
         if (ok) tc_commit(tfull + st);
-      }
-      if (!ok) {  // products in flight complete before the tensor memory is freed
-        tc_commit(drain);
-        mbar_wait(drain, 0u);
       }
     }
   } else {
@@ -776,9 +769,23 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
     }
     if (lane == 0) bulk_wait_all();
   }
+  __syncthreads();
+  if (*s_fail) {
+    // whichever role gave up: the copies in flight land before the shared memory
+    // is released (each block's full barrier completes when its bytes arrived),
+    // the products in flight complete before the tensor memory is freed
+    if (warp == 0 && lane == 0) {
+      atomicOr(g.err, PE_ERR_TIMEOUT);
+      for (uint32_t k = c > (uint32_t)S ? c - S : 0; k < c; ++k)
+        mbar_wait(full + k % S, (k / S) & 1u);
+    }
+    if (warp == 1 && lane == 0) {
+      tc_commit(drain);
+      mbar_wait(drain, 0u);
+    }
+  }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && *s_fail) atomicOr(g.err, PE_ERR_TIMEOUT);
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
@@ -882,15 +889,13 @@ __global__ void __launch_bounds__(WG_THREADS)
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
 
+  int issued = 0;  // pixel blocks whose loads the producer issued
   if (warp == 0) {
     if (lane == 0) {
-      bool ok = true;
-      int kb = 0;
-      for (; kb < nk; ++kb) {
+      for (int kb = 0; kb < nk; ++kb) {
         const int s = kb % g.stages;
         if (!st_wait(empty + s, ((uint32_t)(kb / g.stages) & 1u) ^ 1u, g.wait_limit, &s_fail)) {
           s_fail = 1;
-          ok = false;
           break;
         }
         uint8_t *sa = base + (size_t)s * stage_bytes;
@@ -906,10 +911,8 @@ __global__ void __launch_bounds__(WG_THREADS)
           if (cb) load_conv_box(d, &tmB, g.img, n0 + 64 * b, px, full + s);
           else tma_load_2d(d, &tmB, n0 + 64 * b, px, full + s);
         }
+        issued = kb + 1;
       }
-      if (!ok)
-        for (int k = kb > g.stages ? kb - g.stages : 0; k < kb; ++k)
-          mbar_wait(full + k % g.stages, (uint32_t)(k / g.stages) & 1u);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -937,12 +940,7 @@ __global__ void __launch_bounds__(WG_THREADS)
         }
         tc_commit(empty + s);
       }
-      if (ok) {
-        tc_commit(&accum);
-      } else {
-        tc_commit(&drain);
-        mbar_wait(&drain, 0u);
-      }
+      if (ok) tc_commit(&accum);
     }
   } else {
     const int t = threadIdx.x - 64, j = t & 7, r0 = t >> 3;
@@ -1038,9 +1036,20 @@ __global__ void __launch_bounds__(WG_THREADS)
       }
     }
   }
+  __syncthreads();
+  if (s_fail) {  // as in gemm_stream_kernel: nothing is left in flight
+    if (warp == 0 && lane == 0) {
+      atomicOr(g.err, PE_ERR_TIMEOUT);
+      for (int k = issued > g.stages ? issued - g.stages : 0; k < issued; ++k)
+        mbar_wait(full + k % g.stages, (uint32_t)(k / g.stages) & 1u);
+    }
+    if (warp == 1 && lane == 0) {
+      tc_commit(&drain);
+      mbar_wait(&drain, 0u);
+    }
+  }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && s_fail) atomicOr(g.err, PE_ERR_TIMEOUT);
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(g.cols)

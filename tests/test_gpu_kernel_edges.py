@@ -117,6 +117,46 @@ def test_streaming_contraction_gives_up_and_recovers(mode):
     assert rel(out, torch.nn.functional.gelu(pre) if mode == "gelu" else pre) < BF_TOL
 
 
+# with few polls a wait deep in the loop may fail, in any role, while others have
+# copies or products in flight: the call says so or is whole, and the next computes
+@pytest.mark.parametrize("polls", [1, 2, 5])
+@pytest.mark.parametrize("mode", ["plain", "residual", "gelu", "wgrad"])
+def test_contraction_recovers_whichever_wait_gives_up(mode, polls):
+    from paper_2408_15583_gb300 import _lib
+    lib = _lib.load()
+    o, g = ops(), gen(polls)
+    M, N, K = 90_000, 128, 320
+    A, B = rnd(g, M, K).to(BF), rnd(g, N, K).to(BF)
+    R, Z = rnd(g, M, N).to(BF), torch.empty(M, N, dtype=BF, device=DEV)
+    kw = dict(residual=dict(R=R, ldr=N), gelu=dict(Z=Z, ldz=N, gelu=True)).get(mode, {})
+    stream = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    out = torch.empty(M, N, dtype=BF, device=DEV)
+    dW, db = torch.empty(N, K, device=DEV), torch.empty(N, device=DEV)
+    ws = torch.empty(lib.pe_nn_linear_wgrad_workspace(M, N, K), dtype=torch.uint8, device=DEV)
+    ptr = lambda t: C.c_void_p(t.data_ptr())
+
+    def call():
+        if mode == "wgrad":
+            assert lib.pe_nn_linear_wgrad(ptr(R), N, ptr(A), K, M, N, K, ptr(dW), ptr(db), ptr(ws),
+                                          ws.numel(), stream) == 0
+        else:
+            o.gemm(M, N, K, A, K, 1, B, 1, K, out, N, **kw)
+        return lib.pe_stream_check(stream), (dW if mode == "wgrad" else out).clone()
+
+    status, want = call()
+    assert status == 0
+    for _ in range(3):
+        try:
+            assert lib.pe_nn_set_wait_limit(polls) == 0
+            status, got = call()
+        finally:
+            lib.pe_nn_set_wait_limit(-1)
+        assert status in (0, 4)                       # PE_OK or PE_ETIMEOUT
+        assert status == 4 or torch.equal(got, want)
+        status, got = call()
+        assert status == 0 and torch.equal(got, want)
+
+
 # ---- depthwise 7x7 --------------------------------------------------------------
 
 # images smaller than the stencil, ragged rows and columns, odd pair counts and
