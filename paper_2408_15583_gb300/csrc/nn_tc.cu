@@ -349,8 +349,11 @@ struct st_cfg {
   static_assert((STAGES * STAGE) % 1024 == 0 && STAGING % 1024 == 0 && (BARS * 8) % 16 == 0,
                 "alignment of the slabs, the barriers and the bias");
   static constexpr uint32_t IDESC = tc_cfg<BN>::IDESC;
-  static int smem(int bias_floats) {
-    return 1024 + STAGES * STAGE + STAGING + BARS * 8 + 16 + bias_floats * 4 +
+  // the bias of N columns takes whole slabs: the epilogue reads a slab's width of
+  // it also where the columns end inside the slab
+  static __host__ __device__ constexpr int bias_floats(int n) { return (n + COLS - 1) / COLS * COLS; }
+  static int smem(int n_bias) {
+    return 1024 + STAGES * STAGE + STAGING + BARS * 8 + 16 + bias_floats(n_bias) * 4 +
            (MODE == 3 ? DG_FLOATS * 4 : 0);
   }
 };
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__(ST_THREADS, 2)
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  const int n_pad = g.bias ? (g.N + 31) & ~31 : 0;
+  const int n_pad = g.bias ? cfg::bias_floats(g.N) : 0;
   if (g.bias)
     for (int i = threadIdx.x; i < n_pad; i += ST_THREADS) s_bias[i] = i < g.N ? g.bias[i] : 0.0f;
   float *s_dg = s_bias + n_pad;  // [DG_N], 1 for z > 0; from DG_NEG on for z < 0
@@ -1252,7 +1255,7 @@ pe_status launch_stream(const pe_gemm_args &g, cudaStream_t s, const conv_img *c
   a.err = pe_err_word();
   const int most = 2 * tc_sms();  // two CTAs per SM
   gemm_stream_kernel<BN, MODE, WIDE><<<a.items < most ? a.items : most, ST_THREADS,
-                                 cfg::smem(g.bias ? (g.N + 31) / 32 * 32 : 0), s>>>(ma, mb, mc, mx,
+                                 cfg::smem(g.bias ? g.N : 0), s>>>(ma, mb, mc, mx,
                                                                                     a);
   PE_TRY_LAUNCH("gemm_stream_kernel");
   return PE_OK;
