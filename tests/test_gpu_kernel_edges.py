@@ -190,6 +190,30 @@ def test_depthwise(B, H, W, C):
     assert rel(db, dy.double().sum((0, 1, 2))) < 1e-5
 
 
+# an infinity or NaN of X reaches exactly the taps that read it: one per channel
+# pair, near each side of images whose rows are and are not whole groups of eight
+@pytest.mark.parametrize("H,W", [(9, 17), (4, 5), (7, 64), (40, 130), (2, 16)])
+@pytest.mark.parametrize("value", [math.inf, math.nan])
+def test_depthwise_weight_gradient_of_infinities(H, W, value):
+    o, g, B, C = ops(), gen(H + W), 2, 64
+    x, dy = rnd(g, B, H, W, C).to(BF), rnd(g, B, H, W, C).to(BF)
+    spots = [(y, x_) for y in (0, 1, 2, H - 1, H - 2, H // 2) for x_ in (0, 2, W - 1, W - 2, W // 2)
+             if 0 <= y < H and 0 <= x_ < W][:C // 2]
+    for k, (y, x_) in enumerate(spots):
+        x[k % B, y, x_, 2 * k] = value
+    w = rnd(g, 7, 7, C)
+    dx = torch.empty(B * H * W, C, dtype=BF, device=DEV)
+    dw, db = torch.empty(7, 7, C, device=DEV), torch.empty(C, device=DEV)
+    o.dw_bwd(x, dy, w, B, H, W, C, dx, dw, db)
+    xp = torch.nn.functional.pad(x.double(), (0, 0, 3, 3, 3, 3))
+    want = torch.stack([(xp[:, i:i + H, j:j + W] * dy.double()).sum((0, 1, 2))
+                        for i in range(7) for j in range(7)]).view(7, 7, C)
+    assert torch.equal(dw.isfinite(), want.isfinite())
+    ok = want.isfinite()
+    assert bool((~ok).any()) and rel(dw[ok], want[ok]) < 1e-5
+    assert rel(db, dy.double().sum((0, 1, 2))) < 1e-5
+
+
 # ---- LayerNorm ------------------------------------------------------------------
 
 # one pixel, a block's 64 and its neighbours, more pixels than resident blocks;
