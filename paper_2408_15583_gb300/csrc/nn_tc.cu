@@ -1303,7 +1303,7 @@ pe_status launch_stream_shape(int mode, const pe_gemm_args &g, cudaStream_t s) {
 // 128-row accumulators share a tile as far as tensor memory (512 columns) and
 // shared memory allow.  About 304 CTAs (two per SM where their tensor memory
 // fits; a constant, so that sums do not depend on the device), at least 512
-// pixels each.
+// pixels each unless the mma.sync kernel makes more sums.
 struct wg_plan {
   int a_is_dy, mt, nt, nbx, sets, tiles_m, tiles_n, stages, smem;
   int64_t px, splits;
@@ -1331,12 +1331,14 @@ wg_plan plan_wgrad(int64_t P, int N, int K) {
   w.smem = w.stages * stage + 1024;
   const int64_t tiles = (int64_t)w.tiles_m * w.tiles_n;
   int64_t splits = ((w.cols <= 256 ? 304 : 152) + tiles - 1) / tiles;
-  const int64_t sums = pe_gemm_split(N, K, P);  // of the mma.sync kernel
-  if (splits * w.sets < sums) splits = (sums + w.sets - 1) / w.sets;
   const int64_t most_splits = (P + 511) / 512;
   if (splits > most_splits) splits = most_splits;
+  // at least the sums of the mma.sync kernel (one per 256 pixels at most)
+  const int64_t least = (pe_gemm_split(N, K, P) + w.sets - 1) / w.sets;
+  if (splits < least) splits = least;
   w.px = (P + splits - 1) / splits;
   w.px = (w.px + WG_PX - 1) / WG_PX * WG_PX;
+  if (w.px > WG_PX && (P + w.px - 1) / w.px < least) w.px -= WG_PX;
   w.splits = (P + w.px - 1) / w.px;
   return w;
 }

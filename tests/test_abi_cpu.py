@@ -231,3 +231,17 @@ def test_parameters_equal_the_oracles(lib, G, tau):
                 assert f32(prm.bbox_min[k]) == f32(fp.bmin[k])
             assert f32(prm.eps) == f32(eps) and f32(prm.overlap_r) == f32(eps)
             assert prm.edge_mode == fp.edge_mode == 0
+
+
+# A weight gradient makes at least as many sums over the pixels as the split
+# mma.sync contraction (each drifts with the products added into it).  In these
+# shapes a tile has one set of accumulators, so every sum is a partial dW and db
+# in the workspace: sums x (N K + N) floats.
+@pytest.mark.parametrize("N,K", [(512, 128), (128, 512), (256, 128), (128, 256), (1024, 256),
+                                 (256, 576), (512, 512)])
+@pytest.mark.parametrize("P", [16, 255, 8192, 16384, 26000, 32768, 33000, 65536, 131072, 500001,
+                               2 ** 21])
+def test_weight_gradient_sums_no_longer_than_the_split_contraction(lib, N, K, P):
+    gemm = lib.pe_nn_gemm_workspace(N, K, P)          # 256 bytes, and splits x N K floats
+    splits = max(1, (gemm - 256) // (4 * N * K))
+    assert lib.pe_nn_linear_wgrad_workspace(P, N, K) >= 4 * splits * (N * K + N)
