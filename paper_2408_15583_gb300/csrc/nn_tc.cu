@@ -951,13 +951,16 @@ __global__ void __launch_bounds__(WG_THREADS)
     float *out = g.part + (int64_t)blockIdx.x * ((int64_t)g.N * g.K + g.N);
     if (sums) {
       // dY's columns: thread t adds chunk j (eight channels) of every box at
-      // pixels r0, r0 + 16, ...
+      // pixels r0, r0 + 16, ...: a block's four values, then the blocks' sums
+      // with the error of each addition kept (Knuth's two-sum), so that a long
+      // stretch costs no precision: plain chains over up to thousands of pixels
+      // were less exact than the column sums of 256 pixels that they replace.
       const int nd = g.a_is_dy ? a_boxes : g.nbx, d0 = g.a_is_dy ? 0 : a_boxes;
-      float sum[8][8];
+      float sum[8][8], lost[8][8];
 #pragma unroll
       for (int b = 0; b < 8; ++b)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) sum[b][e] = 0.0f;
+        for (int e = 0; e < 8; ++e) sum[b][e] = lost[b][e] = 0.0f;
       for (int kb = 0; kb < nk; ++kb) {
         const int s = kb % g.stages;
         ok = __all_sync(0xffffffffu,
@@ -968,15 +971,23 @@ __global__ void __launch_bounds__(WG_THREADS)
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
           if (b < nd) {
+            float v[8];
 #pragma unroll
             for (int r = 0; r < WG_PX / 16; ++r) {
               const uint4 u = *reinterpret_cast<const uint4 *>(sd + b * WG_BOX + r * 16 * 128);
               const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                sum[b][2 * e] += __uint_as_float(w[e] << 16);
-                sum[b][2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
+                const float v0 = __uint_as_float(w[e] << 16), v1 = __uint_as_float(w[e] & 0xffff0000u);
+                v[2 * e] = r ? v[2 * e] + v0 : v0;
+                v[2 * e + 1] = r ? v[2 * e + 1] + v1 : v1;
               }
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const float a = sum[b][e], t = __fadd_rn(a, v[e]), z = __fsub_rn(t, a);
+              lost[b][e] += __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(v[e], z));
+              sum[b][e] = t;
             }
           }
         }
@@ -987,7 +998,8 @@ __global__ void __launch_bounds__(WG_THREADS)
       for (int b = 0; b < 8; ++b)
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          float v = sum[b][e];
+          // (the error of an infinite sum is NaN)
+          float v = fabsf(lost[b][e]) < INFINITY ? sum[b][e] + lost[b][e] : sum[b][e];
           v += __shfl_xor_sync(0xffffffffu, v, 8);
           v += __shfl_xor_sync(0xffffffffu, v, 16);
           if (lane < 8) s_db[warp - 2][64 * b + 8 * j + e] = v;

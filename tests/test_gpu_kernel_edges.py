@@ -270,6 +270,23 @@ def test_linear_weight_gradient(P, N, K):
     assert rel(db, dy.double().sum(0)) < 1e-5
 
 
+# the bias gradient of long stretches: dY = 1 at 64 pixels of every 4096, else 2^-22,
+# half an ulp of what a plain chain of sums then holds (it drops nearly all of
+# them: 78 to 144 ulps).  With the errors kept, what is left to round: each
+# thread's sum, two shuffles, three warps, the splits by eights and their eight sums
+@pytest.mark.parametrize("N,K", [(1024, 256), (512, 576), (128, 1152)])
+def test_bias_gradient_of_long_stretches(N, K):
+    o, g, P = ops(), gen(N), 131072
+    dy = torch.full((P, N), 2.0 ** -22, dtype=BF, device=DEV)
+    dy.view(P // 4096, 4096, N)[:, :64] = 1.0
+    x, W = rnd(g, P, K).to(BF), rnd(g, N, K).to(BF)
+    dW, db = torch.empty(N, K, device=DEV), torch.empty(N, device=DEV)
+    o.linear_bwd(dy, x, K, W, None, 0, dW, db, need_dx=False)
+    want = float(dy[:, 0].double().sum())
+    splits = o.lib.pe_nn_linear_wgrad_workspace(P, N, K) // (4 * (N * K + N))   # at most
+    steps = 1 + 2 + 3 + -(-splits // 8) + 8
+    assert float((db.double() - want).abs().max()) <= steps * 2.0 ** -24 * want
+
 # ---- surfel attributes --------------------------------------------------------------
 
 # a lattice, where many neighbours tie at the k_n-th distance (the smaller index is
