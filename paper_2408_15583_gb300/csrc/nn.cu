@@ -618,7 +618,7 @@ __device__ __forceinline__ void dw7_wgrad_rows(const uint32_t *__restrict__ X,
 template <int CT>
 __global__ void __launch_bounds__(DWG_THREADS, 2)
     dw7_wgrad_kernel(const uint32_t *__restrict__ X, const uint32_t *__restrict__ dY, int B, int H,
-                     int W, int C_, int cpb_, int seg, float *__restrict__ part) {
+                     int W, int C_, int cpb_, int seg, int reps, float *__restrict__ part) {
   const int C = CT ? CT : C_;
   const int cpb = CT ? (CT / 2 < 32 ? CT / 2 : 32) : cpb_;
   const int cp2 = C >> 1;
@@ -637,27 +637,39 @@ __global__ void __launch_bounds__(DWG_THREADS, 2)
     else
       dw7_wgrad_rows<4, 3, CT>(X, dY, B, H, W, cp2, cp, seg, first, stride, acc, accb);
   }
-  // positions of the block, added in order into shared memory
-  extern __shared__ float2 s_w[];  // [50][cpb]
-  for (int i = threadIdx.x; i < 50 * cpb; i += DWG_THREADS) s_w[i] = make_float2(0.f, 0.f);
-  for (int k = 0; k < slots; ++k) {
+  // positions of the block, added in a fixed order in shared memory: `reps` of
+  // them side by side, then by halves (one after the other, the 32 positions of 8
+  // channels and the 128 of two were most of a small image's time and of its
+  // rounding)
+  extern __shared__ float2 s_w[];  // [reps][50][cpb]
+  const int n_w = 50 * cpb;
+  for (int i = threadIdx.x; i < reps * n_w; i += DWG_THREADS) s_w[i] = make_float2(0.f, 0.f);
+  for (int k = 0; k < slots; k += reps) {
     __syncthreads();
-    if (on && slot == k) {
+    if (on && slot >= k && slot < k + reps) {
       const int t0 = half * 28, n = half ? 21 : 28;
+      float2 *w = s_w + (slot - k) * n_w + lc;
 #pragma unroll
       for (int j = 0; j < 28; ++j) {
         if (j >= n) break;
-        float2 v = s_w[(t0 + j) * cpb + lc];
+        float2 v = w[(t0 + j) * cpb];
         v.x += acc[j].x;
         v.y += acc[j].y;
-        s_w[(t0 + j) * cpb + lc] = v;
+        w[(t0 + j) * cpb] = v;
       }
       if (!half) {
-        float2 v = s_w[49 * cpb + lc];
+        float2 v = w[49 * cpb];
         v.x += accb.x;
         v.y += accb.y;
-        s_w[49 * cpb + lc] = v;
+        w[49 * cpb] = v;
       }
+    }
+  }
+  for (int o = reps / 2; o > 0; o /= 2) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < o * n_w; i += DWG_THREADS) {
+      s_w[i].x += s_w[i + o * n_w].x;
+      s_w[i].y += s_w[i + o * n_w].y;
     }
   }
   __syncthreads();
@@ -1696,20 +1708,37 @@ extern "C" pe_status pe_nn_dwconv7(const void *X, const float *w, const float *b
   return launch_dw7<false>(X, w, bias, B, H, W, C, Y, s);
 }
 
-// Stretch of a row a weight-gradient thread walks at a time, and the partials
-// per channel chunk: about 304 blocks over the chunks (two per SM; a constant,
-// so that the order of the sums does not depend on the device).
-static int dw_seg(int32_t W) { return W >= 128 ? 64 : (W >= 64 ? 32 : 16); }
-static int dw_chunks(int32_t B, int32_t H, int32_t W, int32_t C) {
+// The weight gradient's split (by constants and sizes only, so that the order of
+// the sums does not depend on the device): the stretch of a row a thread walks
+// at a time, shorter where the image has too few of them for the threads; the
+// partials per channel chunk, about 304 blocks over the chunks (two per SM), or
+// a multiple of that where a thread's chain of additions would be longer than that
+// of one thread for every 1024th row (128 and 256 channels; FP32's rounding grows
+// with the chain: error against 64 bits, 32 x 32^2 by 256, 8.5e-8 -> 8.0e-8, the
+// whole backward 79 -> 94 us; 32 x 64^2 by 128 120 -> 131 us); and the positions
+// added side by side, two turns within 26 KB.
+struct dw_plan {
+  int seg, chunks, reps;
+};
+static dw_plan plan_dw(int32_t B, int32_t H, int32_t W, int32_t C) {
+  dw_plan w;
   const int cpb = dw_cpb(C), slots = DWG_THREADS / 2 / cpb, gy = (C / 2 + cpb - 1) / cpb;
-  const int64_t items = (int64_t)B * H * ((W + dw_seg(W) - 1) / dw_seg(W));
-  const int64_t need = (items + slots - 1) / slots, most = (304 + gy - 1) / gy;
-  return (int)(need < most ? need : most);
+  const int64_t rows = (int64_t)B * H, most = (304 + gy - 1) / gy;
+  w.seg = W >= 128 ? 64 : (W >= 64 ? 32 : 16);
+  while (w.seg > 8 && rows * ((W + w.seg - 1) / w.seg) < most * slots) w.seg /= 2;
+  const int64_t items = rows * ((W + w.seg - 1) / w.seg), need = (items + slots - 1) / slots;
+  const int64_t per = (rows + 1023) / 1024 * W / (W < w.seg ? W : w.seg);  // (at least one)
+  const int64_t least = ((items + per - 1) / per + slots - 1) / slots;
+  const int64_t chunks = (least + most - 1) / most * most;
+  w.chunks = (int)(need < chunks ? need : chunks);
+  w.reps = 1;
+  while (2 * w.reps <= slots && 2 * w.reps * 50 * cpb * (int)sizeof(float2) <= 26 * 1024) w.reps *= 2;
+  return w;
 }
 
 extern "C" size_t pe_nn_dwconv7_bwd_workspace(int32_t B, int32_t H, int32_t W, int32_t C) {
   if (B <= 0 || H <= 0 || W <= 0 || C < 2) return 0;
-  return (size_t)dw_chunks(B, H, W, C) * 50 * C * sizeof(float) + 256;
+  return (size_t)plan_dw(B, H, W, C).chunks * 50 * C * sizeof(float) + 256;
 }
 
 // dX (nullable), dw [7][7][C] and db [C] (FP32, overwritten).
@@ -1725,21 +1754,21 @@ extern "C" pe_status pe_nn_dwconv7_bwd(const void *X, const void *dY, const floa
     if (st != PE_OK) return st;
   }
   if (dw || db) {
-    const int chunks = dw_chunks(B, H, W, C);
+    const dw_plan p = plan_dw(B, H, W, C);
+    const int chunks = p.chunks;
     size_t need = (size_t)chunks * 50 * C * sizeof(float);
     if (!ws || ws_bytes < need) return pe_fail(PE_ENOMEM, "pe_nn_dwconv7_bwd: workspace");
     float *part = static_cast<float *>(ws);
     const int cpb = dw_cpb(C);
     const dim3 grid((unsigned)chunks, (unsigned)((C / 2 + cpb - 1) / cpb));
-    const size_t smem = sizeof(float2) * 50 * cpb;
+    const size_t smem = sizeof(float2) * 50 * cpb * p.reps;
     const uint32_t *x = static_cast<const uint32_t *>(X), *g = static_cast<const uint32_t *>(dY);
-    const int seg = dw_seg(W);
     switch (C) {
-      case 32: dw7_wgrad_kernel<32><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part); break;
-      case 64: dw7_wgrad_kernel<64><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part); break;
-      case 128: dw7_wgrad_kernel<128><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part); break;
-      case 256: dw7_wgrad_kernel<256><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part); break;
-      default: dw7_wgrad_kernel<0><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, seg, part);
+      case 32: dw7_wgrad_kernel<32><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, p.seg, p.reps, part); break;
+      case 64: dw7_wgrad_kernel<64><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, p.seg, p.reps, part); break;
+      case 128: dw7_wgrad_kernel<128><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, p.seg, p.reps, part); break;
+      case 256: dw7_wgrad_kernel<256><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, p.seg, p.reps, part); break;
+      default: dw7_wgrad_kernel<0><<<grid, DWG_THREADS, smem, s>>>(x, g, B, H, W, C, cpb, p.seg, p.reps, part);
     }
     PE_TRY_LAUNCH("dw7_wgrad_kernel");
     // part[chunk][50][C]: taps 0..48 -> dw, 49 -> db; sum the chunks in

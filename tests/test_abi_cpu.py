@@ -245,3 +245,15 @@ def test_weight_gradient_sums_no_longer_than_the_split_contraction(lib, N, K, P)
     gemm = lib.pe_nn_gemm_workspace(N, K, P)          # 256 bytes, and splits x N K floats
     splits = max(1, (gemm - 256) // (4 * N * K))
     assert lib.pe_nn_linear_wgrad_workspace(P, N, K) >= 4 * splits * (N * K + N)
+
+
+# A depthwise weight gradient's additions in FP32: no longer chains than one for
+# every 1024th row of the images makes.  The workspace holds blocks x 50 C floats
+# (and 256 bytes), a block 128 / (channel pairs, at most 32) chains.
+@pytest.mark.parametrize("C", [8, 32, 64, 96, 128, 192, 256, 512])
+@pytest.mark.parametrize("B,H,W", [(32, 256, 256), (32, 128, 128), (32, 64, 64), (32, 32, 32), (1, 64, 64),
+                                   (8, 128, 128), (3, 1000, 64), (64, 512, 128)])
+def test_depthwise_weight_gradient_chains(lib, B, H, W, C):
+    blocks = (lib.pe_nn_dwconv7_bwd_workspace(B, H, W, C) - 256) // (50 * C * 4)
+    chains = blocks * (128 // min(C // 2, 32))
+    assert chains * -(-B * H // 1024) >= B * H

@@ -214,6 +214,24 @@ def test_depthwise_weight_gradient_of_infinities(H, W, value):
     assert rel(db, dy.double().sum((0, 1, 2))) < 1e-5
 
 
+# the split of the weight gradient: positions added side by side (64 for two channels
+# to two for 64 and more), stretches of 8 to 64 pixels, more blocks for 128 channels and up
+@pytest.mark.parametrize("B,H,W,C", [(1, 64, 64, 8), (1, 3, 200, 2), (2, 33, 9, 6), (3, 40, 130, 12),
+                                     (4, 64, 64, 32), (40, 32, 32, 128), (34, 32, 17, 256)])
+def test_depthwise_weight_gradient_split(B, H, W, C):
+    o, g = ops(), gen(B + H + W + C)
+    x, dy = rnd(g, B, H, W, C).to(BF), rnd(g, B, H, W, C).to(BF)
+    w = rnd(g, 7, 7, C)
+    dx = torch.empty(B * H * W, C, dtype=BF, device=DEV)
+    dw, db = torch.empty(7, 7, C, device=DEV), torch.empty(C, device=DEV)
+    o.dw_bwd(x, dy, w, B, H, W, C, dx, dw, db)
+    xp = torch.nn.functional.pad(x.double(), (0, 0, 3, 3, 3, 3))
+    want = torch.stack([(xp[:, i:i + H, j:j + W] * dy.double()).sum((0, 1, 2))
+                        for i in range(7) for j in range(7)]).view(7, 7, C)
+    assert rel(dw, want) < 1e-5
+    assert rel(db, dy.double().sum((0, 1, 2))) < 1e-5
+
+
 # ---- LayerNorm ------------------------------------------------------------------
 
 # one pixel, a block's 64 and its neighbours, more pixels than resident blocks;
