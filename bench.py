@@ -360,7 +360,7 @@ MARCH_BYTES_PER_HIT = 76
 # sphere workload through pe_rcs_sweep; profiles/march_kernel_sphere_batch.md:
 # 90.3 MB over 6,332,964 queries), valid only for the sources it was taken on
 # (their SHA-256 prefixes); scaled to a full launch by the number of queries.
-_SWEEP_SOURCES = {"include/pointemray.h": "394d762d844f8b7d",
+_SWEEP_SOURCES = {"include/pointemray.h": "3634f8ae32c9a0ff",
                   "paper_2408_15583_gb300/csrc/pe_internal.cuh": "2dc3ec4e588ae1ce",
                   "paper_2408_15583_gb300/csrc/sweep.cu": "9f2bcf7b228eaa30"}
 MARCH_NCU_TRAFFIC = {"bytes_per_query": 14.26,

@@ -192,9 +192,12 @@ pe_status pe_build_gfb_topk(const pe_view *views, int32_t n_views, const float *
  *               from the bounding-box centre.
  * pos_dev: FP32 [n][3]; radius_dev [n], normal_dev [n][3] (FP32, either may
  * be null).  Neighbours are exact: ordered by the FP32 squared distance
- * (dx*dx + dy*dy) + dz*dz, ties by index; distances summed in FP64 in that
- * order; mean and covariance in FP64.  Requires 1 <= k_r <= 31, 3 <= k_n <=
- * 32, n >= max(k_r + 1, k_n), n < 2^32; ws of
+ * (dx*dx + dy*dy) + dz*dz, ties by index.  The radius is the mean of the FP64
+ * sum in that order, rounded; mean and covariance are summed in pairs of FP32
+ * (about 46 bits), in FP64 where two eigenvalues are close.  Two calls give the
+ * same bits.  A point with a NaN coordinate gets NaN and is nobody's neighbour;
+ * so does one with fewer than k_r others, or k_n points, left.  Requires 1 <= k_r
+ * <= 31, 3 <= k_n <= 32, n >= max(k_r + 1, k_n), n < 2^32; ws of
  * pe_point_attributes_workspace(n) bytes (256-byte aligned). */
 size_t pe_point_attributes_workspace(int64_t n_points);
 

@@ -223,9 +223,11 @@ __device__ void smallest_axis(double a00, double a01, double a02, double a11, do
 // result's precision rests on (about 100 operations; the square roots, divisions,
 // arc cosine and cosine of the full solution take several times as many).  False
 // (and no result) where the two smallest eigenvalues are close, since Newton's
-// steps need the cubic's slope, and for matrices out of the floats' range.
+// steps need the cubic's slope, for matrices out of the floats' range, and where
+// the squared deviation p^2 from a multiple of the identity, q^2 times the
+// identity's, is not above iso q^2.
 __device__ bool smallest_axis_newton(double a00, double a01, double a02, double a11, double a12,
-                                     double a22, double out[3]) {
+                                     double a22, float iso, double out[3]) {
   const double q = (a00 + a11 + a22) * (1.0 / 3.0);
   const double b00 = a00 - q, b11 = a11 - q, b22 = a22 - q;
   float p2;
@@ -234,7 +236,7 @@ __device__ bool smallest_axis_newton(double a00, double a01, double a02, double 
                 w = (float)a12;
     p2 = x * x + y * y + z * z + 2.0f * (u * u + v * v + w * w);
   }
-  if (!(p2 > 1e-30f && p2 < 1e30f)) return false;
+  if (!(p2 > 1e-30f && p2 < 1e30f && p2 > iso * ((float)q * (float)q))) return false;
   const double ip = (double)rsqrtf(p2 * (1.0f / 6.0f));
   const double c00 = b00 * ip, c11 = b11 * ip, c22 = b22 * ip, c01 = a01 * ip, c02 = a02 * ip,
                c12 = a12 * ip;
@@ -325,7 +327,10 @@ __device__ __forceinline__ void for_runs(const uint32_t *__restrict__ offs, int 
 // The second scan, for the normal, collects the points nearer than the k_n-th
 // distance and, of those at it, the smallest indices, into shared memory; their
 // moments about the query point are then summed by all lanes together, in pairs
-// of floats, and the axis found with as little FP64 as its precision needs.
+// of floats (within 2^-38 of the sum of the products' sizes, 2^-46 as a rule), and
+// the axis found with as little FP64 as its precision needs.  Where the axis is
+// badly conditioned (two near eigenvalues, or three), the moments are summed again
+// in FP64; elsewhere 2^-46 of them moves the axis by less than 2^-32.
 // The points are read as 16-byte records in cell order, a run per (x, y) column
 // of cells, and queries follow the same order, so a warp mostly reads the same
 // records.  A million points, k_r = 8, k_n = 16: 2.35 ms with lists of (distance,
@@ -473,9 +478,9 @@ __global__ void __launch_bounds__(kPtThreads, KT <= 16 ? 8 : (KT <= 24 ? 7 : 6))
       for (int k = 0; k < 3; ++k) A.nrm[3 * (int64_t)i + k] = NAN;
       return;
     }
-    // moments about the query point, of exact differences
-    double m[3] = {0.0, 0.0, 0.0};
-    double a00 = 0, a01 = 0, a02 = 0, a11 = 0, a12 = 0, a22 = 0;
+    // moments about the query point, of exact differences; then about the mean
+    double v[3];
+    bool have = false;
     if (tau > kPairMin && tau < kPairMax) {
       pair_sum mx, my, mz, xx, xy, xz, yy, yz, zz;
       for (int k = 0; k < kn; ++k) {
@@ -494,23 +499,22 @@ __global__ void __launch_bounds__(kPtThreads, KT <= 16 ? 8 : (KT <= 24 ? 7 : 6))
         yz.add_product(y, dy, z, dz);
         zz.add_product(z, dz, z, dz);
       }
-      m[0] = mx.value();
-      m[1] = my.value();
-      m[2] = mz.value();
-      a00 = xx.value();
-      a01 = xy.value();
-      a02 = xz.value();
-      a11 = yy.value();
-      a12 = yz.value();
-      a22 = zz.value();
-    } else {
+      const double m0 = mx.value(), m1 = my.value(), m2 = mz.value();
+      const double c0 = m0 * A.inv_n, c1 = m1 * A.inv_n, c2 = m2 * A.inv_n;
+      have = smallest_axis_newton(xx.value() - m0 * c0, xy.value() - m0 * c1, xz.value() - m0 * c2,
+                                  yy.value() - m1 * c1, yz.value() - m1 * c2, zz.value() - m2 * c2,
+                                  1e-4f, v);
+    }
+    if (!have) {
+      double m0 = 0, m1 = 0, m2 = 0, a00 = 0, a01 = 0, a02 = 0, a11 = 0, a12 = 0, a22 = 0;
+#pragma unroll 1
       for (int k = 0; k < kn; ++k) {
         const float4 p = __ldg(A.pts + list[k * kPtThreads]);
         const double x = (double)p.x - (double)q.x, y = (double)p.y - (double)q.y,
                      z = (double)p.z - (double)q.z;
-        m[0] += x;
-        m[1] += y;
-        m[2] += z;
+        m0 += x;
+        m1 += y;
+        m2 += z;
         a00 += x * x;
         a01 += x * y;
         a02 += x * z;
@@ -518,17 +522,16 @@ __global__ void __launch_bounds__(kPtThreads, KT <= 16 ? 8 : (KT <= 24 ? 7 : 6))
         a12 += y * z;
         a22 += z * z;
       }
+      const double c0 = m0 * A.inv_n, c1 = m1 * A.inv_n, c2 = m2 * A.inv_n;
+      a00 -= m0 * c0;
+      a01 -= m0 * c1;
+      a02 -= m0 * c2;
+      a11 -= m1 * c1;
+      a12 -= m1 * c2;
+      a22 -= m2 * c2;
+      if (!smallest_axis_newton(a00, a01, a02, a11, a12, a22, 0.0f, v))
+        smallest_axis(a00, a01, a02, a11, a12, a22, v);
     }
-    const double mx = m[0] * A.inv_n, my = m[1] * A.inv_n, mz = m[2] * A.inv_n;
-    a00 -= m[0] * mx;
-    a01 -= m[0] * my;
-    a02 -= m[0] * mz;
-    a11 -= m[1] * my;
-    a12 -= m[1] * mz;
-    a22 -= m[2] * mz;
-    double v[3];
-    if (!smallest_axis_newton(a00, a01, a02, a11, a12, a22, v))
-      smallest_axis(a00, a01, a02, a11, a12, a22, v);
     double w[3];
     if (A.ref) {
       for (int k = 0; k < 3; ++k) w[k] = (double)A.ref[3 * (int64_t)i + k];

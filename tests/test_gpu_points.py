@@ -210,3 +210,23 @@ def test_radius_is_the_rounded_fp64_mean(case, axis):
     r, _ = api.point_attributes(torch.from_numpy(pos).to(DEV), k, 3, normal=False)
     api.stream_check()
     assert np.array_equal(r.cpu().numpy(), oracle.knn_radius(idx, d2, np.arange(k + 1), k))
+
+
+@pytest.mark.parametrize("shells", [2, 4, 5])
+def test_normals_of_nearly_isotropic_neighbourhoods(shells):
+    """Six points per shell on the axes at a, b, c, neighbouring floats: the axis is
+    z, with eigenvalues 1e-7 apart.  FP64 sums leave some 1e-16 of the moments, so
+    1e-9 of the axis; 32 roundings of 2^-53 would leave 2e-8 at the very most of a
+    component whose cross moments are all of one sign (they are not), so 2^-27."""
+    rng = np.random.default_rng(shells)
+    worst = 0.0
+    for _ in range(20):
+        a = (0.5 + rng.random(shells)).astype(np.float32)
+        b = np.nextafter(a, np.float32(0))
+        c = np.nextafter(b, np.float32(0))
+        z = np.zeros_like(a)
+        pos = np.concatenate([np.stack(r, 1) for s in (np.float32(1), np.float32(-1))
+                              for r in ((s * a, z, z), (z, s * b, z), (z, z, s * c))])
+        _, n = _gpu(pos, 1, 6 * shells)
+        worst = max(worst, float(np.abs(n[:, :2]).max()))
+    assert worst < 2.0 ** -27
