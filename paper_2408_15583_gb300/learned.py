@@ -48,11 +48,13 @@ class Ops:
     def s(self):
         if self.stream is not None:
             return self.stream.cuda_stream
-        if self.dev.type != "cuda":
-            return torch.cuda.current_stream(self.dev).cuda_stream      # (raises)
-        # the handle alone: a Stream object takes ten times as long to make
+        # the handle alone, where this torch gives it (the name is not public): a
+        # Stream object takes ten times as long to make
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None or self.dev.type != "cuda":          # (no CUDA device: raises)
+            return torch.cuda.current_stream(self.dev).cuda_stream
         i = self.dev.index
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
+        return raw(torch.cuda.current_device() if i is None else i)
 
     def ws(self, nbytes):
         if self._ws.numel() < nbytes:

@@ -257,3 +257,16 @@ def test_depthwise_weight_gradient_chains(lib, B, H, W, C):
     blocks = (lib.pe_nn_dwconv7_bwd_workspace(B, H, W, C) - 256) // (50 * C * 4)
     chains = blocks * (128 // min(C // 2, 32))
     assert chains * -(-B * H // 1024) >= B * H
+
+
+def test_stream_handle_without_torchs_raw_getter(monkeypatch):
+    # the layer calls take the current stream's handle from the public Stream where
+    # torch has no _cuda_getCurrentRawStream
+    import torch
+    from paper_2408_15583_gb300.learned import Ops
+    o = object.__new__(Ops)
+    o.dev, o.stream = torch.device("cuda:0"), None
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream",
+                        lambda dev: type("S", (), {"cuda_stream": 77 + dev.index}))
+    assert o.s() == 77
