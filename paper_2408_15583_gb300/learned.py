@@ -307,7 +307,13 @@ class UNet:
         o = self.ops
         tape: List = []
         c = self.widths
-        y = self._conv3_fwd(x.view(-1, 1), "stem", B, H, W, 1, c[0], tape)
+        # the tape holds a copy of x: the stem's gradient is that of this pass, also
+        # when the caller has changed x since
+        P = B * H * W
+        xs = self._empty(P, 1)
+        k = 8 if P % 8 == 0 else 1
+        o.copy(x.view(-1, 1), k, 0, xs, k, 0, P // k, k)
+        y = self._conv3_fwd(xs, "stem", B, H, W, 1, c[0], tape)
         skips = []
         dims = []
         h, w = H, W

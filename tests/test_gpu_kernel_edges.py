@@ -527,6 +527,27 @@ def test_parameter_views_follow_their_buffers(how):
     assert torch.equal(got_grad, want_grad)
 
 
+# the gradients are those of the forward pass, whatever the caller did to its input
+# in between
+@pytest.mark.parametrize("widths,H", [((32, 64), 16), ((8,), 5)])
+def test_gradients_after_the_input_was_overwritten(widths, H):
+    import scenes
+    from paper_2408_15583_gb300.learned import UNet
+    blocks = (1,) * len(widths)
+    net = UNet(scenes.unet_init(4, widths, blocks), widths, blocks, DEV)
+    x = rnd(gen(5), H * H).to(BF)
+
+    def step(overwrite):
+        mine = x.clone()
+        outs, tape = net.forward(mine, 1, H, H)
+        if overwrite:
+            mine.fill_(3.0)
+        net.backward(tape, {k: torch.ones_like(v) for k, v in outs.items()})
+        return net.grad.clone()
+
+    assert torch.equal(step(False), step(True))
+
+
 # ---- Canny hysteresis over its tiles --------------------------------------------
 
 # a weak depth step along a serpentine corridor, strong at its start only, on
