@@ -490,7 +490,9 @@ class GraphedUNet:
         g = torch.cuda.CUDAGraph()
         with torch.cuda.graph(g):
             out = fn()
-        return g, out
+        # the replays write the workspace of this moment: kept with the graph, since
+        # a later call that needs more replaces it
+        return g, out, self.net.ops.ws(0)
 
     def train_step(self, x, d_gt, n_gt, m_gt, lr):
         """One training step (the graph, then AdamW); returns the loss vector."""
@@ -502,7 +504,7 @@ class GraphedUNet:
             # the warm-up inside the capture runs forward and backward once;
             # its gradients are overwritten by the replay below
             self._train = self._capture(self._fwd_bwd)
-        g, loss = self._train
+        g, loss, _ = self._train
         g.replay()
         self.net.adamw(lr)
         return loss
@@ -514,7 +516,7 @@ class GraphedUNet:
         if self._infer is None:
             self._infer = self._capture(
                 lambda: self.net.forward(self.x, self.B, self.H, self.W)[0])
-        g, outs = self._infer
+        g, outs, _ = self._infer
         g.replay()
         return outs
 

@@ -548,6 +548,29 @@ def test_gradients_after_the_input_was_overwritten(widths, H):
     assert torch.equal(step(False), step(True))
 
 
+# a captured pass goes on writing the workspace it was captured with: a larger eager
+# pass, which takes a larger one, leaves that memory to the graph
+def test_captured_pass_keeps_its_workspace():
+    import gc
+    import scenes
+    from paper_2408_15583_gb300.learned import GraphedUNet, UNet
+    widths, blocks, H = (8, 16), (1, 1), 32
+    net = UNet(scenes.unet_init(6, widths, blocks), widths, blocks, DEV)
+    g = gen(7)
+    x, big = rnd(g, H * H).to(BF), rnd(g, 16 * H * H).to(BF)
+    graphed = GraphedUNet(net, 1, H, H)
+    want = {k: v.clone() for k, v in graphed.forward(x).items()}
+    at, size = net.ops._ws.data_ptr(), net.ops._ws.numel()
+    net.forward(big, 16, H, H)
+    assert net.ops._ws.data_ptr() != at
+    gc.collect()
+    others = [torch.full((size,), 7, dtype=torch.uint8, device=DEV) for _ in range(8)]
+    got = graphed.forward(x)
+    assert all(torch.equal(got[k], want[k]) for k in want)
+    assert all(bool((t == 7).all()) for t in others)
+    assert all(t.data_ptr() >= at + size or t.data_ptr() + size <= at for t in others)
+
+
 # ---- Canny hysteresis over its tiles --------------------------------------------
 
 # a weak depth step along a serpentine corridor, strong at its start only, on
