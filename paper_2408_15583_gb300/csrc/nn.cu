@@ -2013,6 +2013,7 @@ __global__ void __launch_bounds__(256)
     stem_fwd_kernel(const stem_img im, int64_t P, const bf16 *__restrict__ w,
                     const float *__restrict__ bias, bf16 *__restrict__ y, int N) {
   const int lane = threadIdx.x & 31, gq = lane >> 2, tq = lane & 3, n0 = blockIdx.y * 32;
+  const bool vec = (reinterpret_cast<uintptr_t>(y) & 15) == 0;
   uint32_t b[4][2];
   float bs[8];
 #pragma unroll
@@ -2088,9 +2089,14 @@ __global__ void __launch_bounds__(256)
         const bf162 o = __floats2bfloat162_rn(c0, c1);
         out[h][e] = *reinterpret_cast<const uint32_t *>(&o);
       }
-      if (p < P)
-        *reinterpret_cast<uint4 *>(y + p * N + n0 + 8 * tq) =
-            make_uint4(out[h][0], out[h][1], out[h][2], out[h][3]);
+      bf16 *dst = y + p * N + n0 + 8 * tq;
+      if (p < P && vec) {
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(out[h][0], out[h][1], out[h][2], out[h][3]);
+      } else if (p < P) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          reinterpret_cast<unsigned short *>(dst)[e] = (unsigned short)(out[h][e / 2] >> (16 * (e & 1)));
+      }
     }
   }
 }
@@ -2100,8 +2106,9 @@ __global__ void __launch_bounds__(256)
 // read once in 16-byte accesses and x through the caches.  part[block][9 N + N].
 // 32 x 256^2 by 32: 361 us with the matrix written and a 128-row mma.sync tile of
 // which 32 rows held outputs, 117 us now.
+// VEC: rows of dY on 16-byte boundaries.
 constexpr int kStemBlocks = 304, STEM_THREADS = 256;
-template <int LPP>
+template <int LPP, bool VEC>
 __global__ void __launch_bounds__(STEM_THREADS, 2)
     stem_wgrad_kernel(const stem_img im, int64_t P, const bf16 *__restrict__ dY,
                       float *__restrict__ part) {
@@ -2115,8 +2122,18 @@ __global__ void __launch_bounds__(STEM_THREADS, 2)
     for (int e = 0; e < 8; ++e) acc[t][e] = 0.0f;
   const int64_t step = (int64_t)gridDim.x * WARPS * PPW;
   for (int64_t p = ((int64_t)blockIdx.x * WARPS + warp) * PPW + lane / LPP; p < P; p += step) {
-    const uint4 u = __ldg(reinterpret_cast<const uint4 *>(dY + p * N) + c);
-    const uint32_t wd[4] = {u.x, u.y, u.z, u.w};
+    uint32_t wd[4];
+    if (VEC) {
+      const uint4 u = __ldg(reinterpret_cast<const uint4 *>(dY + p * N) + c);
+      wd[0] = u.x;
+      wd[1] = u.y;
+      wd[2] = u.z;
+      wd[3] = u.w;
+    } else {
+      const unsigned short *r = reinterpret_cast<const unsigned short *>(dY + p * N) + 8 * c;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) wd[e] = (uint32_t)__ldg(r + 2 * e) | (uint32_t)__ldg(r + 2 * e + 1) << 16;
+    }
     const uint32_t q = (uint32_t)p / (uint32_t)im.W;
     const int px = (int)((uint32_t)p - q * (uint32_t)im.W), py = (int)(q % (uint32_t)im.H);
     float xt[9], d[8];
@@ -2158,7 +2175,10 @@ pe_status launch_stem_wgrad(const stem_img &im, int64_t P, const bf16 *dY, float
   constexpr int per_block = STEM_THREADS / LPP;
   const int64_t need = (P + per_block - 1) / per_block;
   const int blocks = (int)(need < kStemBlocks ? need : kStemBlocks);
-  stem_wgrad_kernel<LPP><<<blocks, STEM_THREADS, 0, s>>>(im, P, dY, part);
+  if ((reinterpret_cast<uintptr_t>(dY) & 15) == 0)
+    stem_wgrad_kernel<LPP, true><<<blocks, STEM_THREADS, 0, s>>>(im, P, dY, part);
+  else
+    stem_wgrad_kernel<LPP, false><<<blocks, STEM_THREADS, 0, s>>>(im, P, dY, part);
   PE_TRY_LAUNCH("stem_wgrad_kernel");
   return pe_wgrad_reduce(part, blocks, 72 * LPP, 80 * LPP, dW, db, s);
 }
@@ -2202,6 +2222,14 @@ static bool conv_gathered(int32_t B, int32_t H, int32_t W, int32_t Cin, int32_t 
          pe_conv3_tc_sizes(B, H, W, Cin, Cout);
 }
 
+// Whether the one-channel kernels above take a layer's forward pass, its gradient.
+static bool stem_fwd_sizes(int32_t Cin, int32_t Cout) {
+  return Cin == 1 && Cout % 32 == 0 && Cout / 32 <= 65535;
+}
+static bool stem_wgrad_sizes(int32_t Cin, int32_t Cout) {
+  return Cin == 1 && (Cout == 8 || Cout == 16 || Cout == 32 || Cout == 64 || Cout == 128);
+}
+
 extern "C" size_t pe_nn_conv3_workspace(int32_t B, int32_t H, int32_t W, int32_t Cin, int32_t Cout) {
   if (!conv_sizes(B, H, W, Cin, Cout)) return 0;
   const int64_t P = (int64_t)B * H * W;
@@ -2209,6 +2237,7 @@ extern "C" size_t pe_nn_conv3_workspace(int32_t B, int32_t H, int32_t W, int32_t
   const size_t a = pe_nn_gemm_workspace((int32_t)P, Cout, 9 * (int64_t)Cin),
                b = pe_nn_linear_wgrad_workspace(P, Cout, 9 * Cin);
   const size_t c = Cin == 1 ? (size_t)kStemBlocks * 10 * Cout * sizeof(float) : 0;
+  if (stem_fwd_sizes(Cin, Cout) && stem_wgrad_sizes(Cin, Cout)) return c + 512;  // neither writes col
   const size_t most = a > b ? (a > c ? a : c) : (b > c ? b : c);
   return (conv_gathered(B, H, W, Cin, Cout) ? 0 : col) + most + 512;
 }
@@ -2244,7 +2273,7 @@ extern "C" pe_status pe_nn_conv3(const void *x, int32_t B, int32_t H, int32_t W,
       return pe_fail(PE_EINVAL, "pe_nn_conv3: pointers on 16-byte boundaries");
     return pe_conv3_tc(g, B, H, W, Cin, s);
   }
-  if (Cin == 1 && Cout % 32 == 0 && Cout / 32 <= 65535 && (reinterpret_cast<uintptr_t>(y) & 15) == 0) {
+  if (stem_fwd_sizes(Cin, Cout)) {
     const stem_img im = {g.A, W, H};
     const int64_t P = (int64_t)B * H * W;
     stem_fwd_kernel<<<dim3(grid1((P + 127) / 128, 1, 8), Cout / 32), 256, 0, s>>>(
@@ -2277,18 +2306,16 @@ extern "C" pe_status pe_nn_conv3_wgrad(const void *dY, const void *x, int32_t B,
     return pe_wgrad_tc(dY, Cout, x, 9 * (int64_t)Cin, P, Cout, 9 * Cin, dW, db,
                        static_cast<float *>(ws), s, img);
   }
-  if (Cin == 1 && (reinterpret_cast<uintptr_t>(dY) & 15) == 0 &&
-      (reinterpret_cast<uintptr_t>(ws) & 3) == 0) {
+  if (stem_wgrad_sizes(Cin, Cout)) {
     const stem_img im = {static_cast<const bf16 *>(x), W, H};
     const bf16 *d = static_cast<const bf16 *>(dY);
-    float *part = static_cast<float *>(ws);
+    float *part = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
     switch (Cout) {
       case 8: return launch_stem_wgrad<1>(im, P, d, dW, db, part, s);
       case 16: return launch_stem_wgrad<2>(im, P, d, dW, db, part, s);
       case 32: return launch_stem_wgrad<4>(im, P, d, dW, db, part, s);
       case 64: return launch_stem_wgrad<8>(im, P, d, dW, db, part, s);
-      case 128: return launch_stem_wgrad<16>(im, P, d, dW, db, part, s);
-      default: break;
+      default: return launch_stem_wgrad<16>(im, P, d, dW, db, part, s);
     }
   }
   pe_status st;

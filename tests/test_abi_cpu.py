@@ -270,3 +270,12 @@ def test_stream_handle_without_torchs_raw_getter(monkeypatch):
     monkeypatch.setattr(torch.cuda, "current_stream",
                         lambda dev: type("S", (), {"cuda_stream": 77 + dev.index}))
     assert o.s() == 77
+
+
+@pytest.mark.parametrize("Cout", [32, 64, 128])
+def test_one_channel_convolution_workspace(lib, Cout):
+    # neither pass of a one-channel convolution writes the neighbourhood matrix (18
+    # bytes per pixel) there; elsewhere the workspace holds it
+    sums = 304 * 10 * Cout * 4
+    assert lib.pe_nn_conv3_workspace(32, 256, 256, 1, Cout) <= sums + 1024
+    assert lib.pe_nn_conv3_workspace(32, 256, 256, 1, 40) >= 18 * 32 * 256 * 256

@@ -481,6 +481,32 @@ def test_conv3_one_channel(B, H, W, Cout):
     assert rel(dW, dy.double().T @ ref) < 1e-5 and rel(db, dy.double().sum(0)) < 1e-5
 
 
+# rows off 16-byte boundaries: the same bits
+@pytest.mark.parametrize("Cout", [8, 32, 64, 128, 40])
+def test_conv3_one_channel_unaligned(Cout):
+    from paper_2408_15583_gb300 import api
+    o, g, (B, H, W) = ops(), gen(Cout), (2, 21, 19)
+    P = B * H * W
+    x, b, dy = rnd(g, P).to(BF), rnd(g, Cout), rnd(g, P, Cout).to(BF)
+    w = (rnd(g, Cout, 9) / 3).to(BF)
+
+    def off(t):
+        return torch.empty(t.numel() + 1, dtype=t.dtype, device=DEV)[1:].view(t.shape).copy_(t)
+
+    res = []
+    for f in (lambda t: t, off):
+        y = f(torch.full((P, Cout), 7.0, dtype=BF, device=DEV))
+        dW, db = torch.empty(Cout, 9, device=DEV), torch.empty(Cout, device=DEV)
+        o.conv3(f(x), f(w), b, B, H, W, 1, Cout, y)
+        o.conv3_wgrad(f(dy), f(x), B, H, W, 1, Cout, dW, db)
+        api.stream_check()
+        res.append((y, dW, db))
+    assert torch.equal(res[0][0], res[1][0])
+    assert rel(res[1][1], res[0][1]) < 1e-5 and rel(res[1][2], res[0][2]) < 1e-5
+    if Cout != 40:
+        assert torch.equal(res[0][1], res[1][1]) and torch.equal(res[0][2], res[1][2])
+
+
 # two to eight splits and more, with and without a residual, whole rows of eight and not
 @pytest.mark.parametrize("M,N,K", [(16384, 256, 1024), (1000, 64, 2304), (640, 136, 1100), (257, 36, 600)])
 def test_split_contraction(M, N, K):
