@@ -1796,6 +1796,9 @@ extern "C" pe_status pe_nn_layernorm(const void *X, const float *gamma, const fl
         static_cast<const bf16 *>(X), gamma, beta, P, eps, static_cast<bf16 *>(Y), mean, rstd);
     PE_TRY_LAUNCH("ln_fwd_narrow_kernel");
   } else if (al16 && (C == 64 || C == 128 || C == 256)) {
+    // (the widths of the network's levels; the kernel takes any multiple of 32, an
+    // instance each, and the other widths have a warp per pixel and 2-byte loads,
+    // which took four times as long at 64 channels)
     const bf16 *x = static_cast<const bf16 *>(X);
     bf16 *y = static_cast<bf16 *>(Y);
     const int blocks = grid1(P, LN_THREADS / 4, 8);
@@ -1838,7 +1841,7 @@ extern "C" pe_status pe_nn_layernorm_bwd(const void *dY, const void *X, const fl
   float *part = static_cast<float *>(ws);
   auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   if (al16(X) && al16(dY) && al16(dX) && (C == 32 || C == 64 || C == 128)) {
-    // (256 channels would hold 256 values and sums per thread)
+    // (as forward, but 256 channels would hold 256 values and sums per thread)
     const bf16 *x = static_cast<const bf16 *>(X), *dy = static_cast<const bf16 *>(dY);
     bf16 *dx = static_cast<bf16 *>(dX);
     const int nb = ln_bwd_blocks(P);

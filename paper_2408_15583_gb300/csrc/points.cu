@@ -11,8 +11,8 @@
 // growing Chebyshev radius until its k-th distance is below the distance to
 // every unsearched cell.  Neighbours are ordered by (FP32 squared distance,
 // index), with the squared distance evaluated in one fixed order, so the
-// neighbour sets -- and the radii, summed in FP64 from the nearest on -- equal a
-// brute-force search bit for bit.
+// neighbour sets -- and the radii, which round as FP64 sums from the nearest on
+// do -- equal a brute-force search bit for bit.
 #include <cstring>
 
 #include "pe_internal.cuh"
@@ -127,7 +127,7 @@ __global__ void scatter_points(const float *__restrict__ pos, int64_t n,
 // The records with the points of a cell by index, so that what is added up in
 // this order (the moments of a normal) is the same on every run: a thread per
 // point counts the smaller indices of its cell.  A million points, about 36 to a
-// cell: 16 us of the 860 for radii and normals.
+// cell: 18 us of the 850 for radii and normals.
 __global__ void sort_cells(const float *__restrict__ pos, int64_t n,
                            const uint32_t *__restrict__ cell_of, const uint32_t *__restrict__ offs,
                            const uint32_t *__restrict__ idx, float4 *__restrict__ pts) {
@@ -336,7 +336,8 @@ __device__ __forceinline__ void for_runs(const uint32_t *__restrict__ offs, int 
 // records.  A million points, k_r = 8, k_n = 16: 2.35 ms with lists of (distance,
 // index) in local memory, insertion by a data-dependent loop and 27 cells visited
 // one by one (13.6 of 32 lanes active); 1.28 ms with both scans as above and
-// moments, roots and eigenvectors in FP64, at a 64th of the FP32 rate; 0.68 ms now.
+// moments, roots and eigenvectors in FP64, at a 64th of the FP32 rate; 0.70 ms now
+// (0.02 of it for radii that round as FP64 does and for points that are NaN).
 template <int KT>
 __global__ void __launch_bounds__(kPtThreads, KT <= 16 ? 8 : (KT <= 24 ? 7 : 6))
     knn_kernel(const knn_args A) {
