@@ -305,6 +305,23 @@ def test_bias_gradient_of_long_stretches(N, K):
     steps = 1 + 2 + 3 + -(-splits // 8) + 8
     assert float((db.double() - want).abs().max()) <= steps * 2.0 ** -24 * want
 
+# an infinite or NaN dY reaches its own bias and weights alone, as infinity or NaN
+@pytest.mark.parametrize("N,K", [(256, 64), (64, 256)])
+def test_bias_gradient_of_infinities(N, K):
+    o, g, P = ops(), gen(N), 5000
+    dy, x = rnd(g, P, N).to(BF), (rnd(g, P, K).abs() + 0.5).to(BF)
+    dy[5, 3], dy[4000, 9], dy[70, 17] = math.inf, -math.inf, math.nan
+    dy[100, 33], dy[101, 33] = math.inf, -math.inf
+    W = rnd(g, N, K).to(BF)
+    dW, db = torch.empty(N, K, device=DEV), torch.empty(N, device=DEV)
+    o.linear_bwd(dy, x, K, W, None, 0, dW, db, need_dx=False)
+    want = dy.double().sum(0)
+    ok = want.isfinite()
+    assert torch.equal(db.isfinite(), ok) and rel(db[ok], want[ok]) < 1e-5
+    assert torch.equal(db[~ok].nan_to_num(7.0), want[~ok].float().nan_to_num(7.0))
+    assert torch.equal(dW.isfinite().all(1), ok) and torch.equal(dW.isfinite().any(1), ok)
+
+
 # ---- surfel attributes --------------------------------------------------------------
 
 # a lattice, where many neighbours tie at the k_n-th distance (the smaller index is
